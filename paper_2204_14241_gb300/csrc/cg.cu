@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "team.h"
 
 namespace hmc {
 
@@ -285,6 +286,12 @@ __global__ void k_phi_to32(const double* __restrict__ a, float* __restrict__ b, 
     if (i < n) b[i] = (float)a[i];
 }
 
+int launch_phi_to32(hmc_ctx* ctx, const double* a, float* b, int64_t n) {
+    k_phi_to32<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(a, b, n);
+    HMC_LAUNCH(ctx, "k_phi_to32");
+    return HMC_OK;
+}
+
 // ---- host driver ---------------------------------------------------------------------------
 // FP64 true residual r = b - A x for the start from a guess and the reliable updates, as two
 // passes through ctx->d_z64: t_ = D^dagger x, then r = b - D t_ with the complex64 copy and the
@@ -320,8 +327,8 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
     if constexpr (kMixed) {
         xv = ctx->d_x32; rv = ctx->d_r32; pv = ctx->d_p32; pw = ctx->d_p32b; qv = ctx->d_q32;
         zv = precond ? ctx->d_z32 : ctx->d_r32;
-        k_phi_to32<<<(unsigned)((3 * lat.V + 255) / 256), 256, 0, sm>>>(phi64, ctx->d_phi32, 3 * lat.V);
-        HMC_LAUNCH(ctx, "k_phi_to32");
+        const int rc32 = launch_phi_to32(ctx, phi64, ctx->d_phi32, 3 * lat.V);
+        if (rc32) return rc32;
         phiR = ctx->d_phi32;
         HMC_CUDA(ctx, cudaMemsetAsync(ctx->d_x32, 0, nrhs * n * sizeof(float2), sm));
     } else {
@@ -564,6 +571,9 @@ int cg_run(hmc_ctx* ctx, int chain, const double* phi, const double2* b, double2
            double tol, int maxit, int precond, hmc_cg_stats* st, bool use_x0, bool* y_ready) {
     const Lat& lat = ctx->chains[chain].lat;
     if (y_ready) *y_ready = false;
+    bool done = false;
+    const int rc = team_solve(ctx, lat, phi, b, x, nrhs, tol, maxit, precond, st, use_x0, y_ready, &done);
+    if (done || rc) return rc;
     if (ctx->p.solver_mode == HMC_SOLVER_MIXED)
         return run<float>(ctx, lat, phi, b, x, nrhs, tol, maxit, precond, st, use_x0, y_ready);
     return run<double>(ctx, lat, phi, b, x, nrhs, tol, maxit, precond, st, use_x0, y_ready);

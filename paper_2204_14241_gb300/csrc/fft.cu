@@ -345,7 +345,7 @@ static int add_plan(hmc_ctx* ctx, int n) {
     return HMC_OK;
 }
 
-static PcTables* get_pc(hmc_ctx* ctx, int L, int Nt) {
+PcTables* get_pc(hmc_ctx* ctx, int L, int Nt) {
     for (auto& t : ctx->pcs)
         if (t.L == L && t.Nt == Nt) return &t;
     return nullptr;

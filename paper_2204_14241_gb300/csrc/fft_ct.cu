@@ -12,6 +12,7 @@
 //   kTau:   the preconditioner's tau pass (twist, forward FFT, P-hat, inverse FFT, twist).
 #include <cmath>
 
+#include "dft.cuh"
 #include "internal.h"
 #include "fft_ct.h"
 
@@ -46,151 +47,6 @@ constexpr RadixList radices(int N) {
 }
 
 constexpr int kThreads = 256;
-
-// Twiddles known at compile time: cos and sin of 2 pi m / R from their Taylor series on
-// [-pi/2, pi/2] (20 terms; the series' own truncation error there is below 1e-20).
-constexpr double kPi = 3.14159265358979323846264338327950288;
-__host__ __device__ constexpr double ct_sin_series(double x) {
-    double t = x, s = x;
-    for (int n = 1; n < 20; ++n) { t *= -x * x / ((2.0 * n) * (2.0 * n + 1.0)); s += t; }
-    return s;
-}
-__host__ __device__ constexpr double ct_cos_series(double x) {
-    double t = 1.0, s = 1.0;
-    for (int n = 1; n < 20; ++n) { t *= -x * x / ((2.0 * n - 1.0) * (2.0 * n)); s += t; }
-    return s;
-}
-__host__ __device__ constexpr double ct_cos2pi(int m, int R) {
-    m %= R;
-    if (m < 0) m += R;
-    double x = 2.0 * kPi * m / R;
-    if (x > kPi) x -= 2.0 * kPi;
-    if (x > kPi / 2) return -ct_cos_series(kPi - x);
-    if (x < -kPi / 2) return -ct_cos_series(-kPi - x);
-    return ct_cos_series(x);
-}
-__host__ __device__ constexpr double ct_sin2pi(int m, int R) {
-    m %= R;
-    if (m < 0) m += R;
-    double x = 2.0 * kPi * m / R;
-    if (x > kPi) x -= 2.0 * kPi;
-    if (x > kPi / 2) return ct_sin_series(kPi - x);
-    if (x < -kPi / 2) return ct_sin_series(-kPi - x);
-    return ct_sin_series(x);
-}
-template <int R> struct TwR { float c[R], s[R]; };   // cos, sin of 2 pi m / R
-template <int R> __host__ __device__ constexpr TwR<R> make_tw() {
-    TwR<R> t{};
-    for (int m = 0; m < R; ++m) { t.c[m] = (float)ct_cos2pi(m, R); t.s[m] = (float)ct_sin2pi(m, R); }
-    return t;
-}
-
-__device__ __forceinline__ float2 cmulf(float2 a, float c, float s) {   // a * (c + i s)
-    return make_float2(a.x * c - a.y * s, a.x * s + a.y * c);
-}
-
-// Prime-size DFTs on registers: v[p] <- sum_q v[q] w^{pq}, w = e^{DIR 2 pi i / R}.
-template <int R, int DIR>
-__device__ __forceinline__ void bfly_prime(float2* v) {
-    if constexpr (R == 2) {
-        const float2 a = v[0], b = v[1];
-        v[0] = make_float2(a.x + b.x, a.y + b.y);
-        v[1] = make_float2(a.x - b.x, a.y - b.y);
-    } else if constexpr (R == 4) {
-        const float2 a = v[0], b = v[1], c = v[2], d = v[3];
-        const float2 s0 = make_float2(a.x + c.x, a.y + c.y), s1 = make_float2(a.x - c.x, a.y - c.y);
-        const float2 s2 = make_float2(b.x + d.x, b.y + d.y), s3 = make_float2(b.x - d.x, b.y - d.y);
-        const float2 s3r = make_float2(-DIR * s3.y, DIR * s3.x);   // s3 * (DIR i)
-        v[0] = make_float2(s0.x + s2.x, s0.y + s2.y);
-        v[2] = make_float2(s0.x - s2.x, s0.y - s2.y);
-        v[1] = make_float2(s1.x + s3r.x, s1.y + s3r.y);
-        v[3] = make_float2(s1.x - s3r.x, s1.y - s3r.y);
-    } else if constexpr (R == 3) {
-        // X1,2 = v0 - (v1 + v2)/2 +- DIR i (sqrt3/2)(v1 - v2)
-        constexpr float h = (float)ct_sin2pi(1, 3);
-        const float2 t1 = make_float2(v[1].x + v[2].x, v[1].y + v[2].y);
-        const float2 d = make_float2(DIR * h * (v[1].x - v[2].x), DIR * h * (v[1].y - v[2].y));
-        const float2 m = make_float2(v[0].x - 0.5f * t1.x, v[0].y - 0.5f * t1.y);
-        v[0] = make_float2(v[0].x + t1.x, v[0].y + t1.y);
-        v[1] = make_float2(m.x - d.y, m.y + d.x);
-        v[2] = make_float2(m.x + d.y, m.y - d.x);
-    } else if constexpr (R == 5) {
-        // pairs (1, 4) and (2, 3): X_{1,4} = m1 +- i n1, X_{2,3} = m2 +- i n2
-        constexpr float c1 = (float)ct_cos2pi(1, 5), c2 = (float)ct_cos2pi(2, 5);
-        constexpr float s1 = (float)ct_sin2pi(1, 5), s2 = (float)ct_sin2pi(2, 5);
-        const float2 a1 = make_float2(v[1].x + v[4].x, v[1].y + v[4].y);
-        const float2 a2 = make_float2(v[2].x + v[3].x, v[2].y + v[3].y);
-        const float2 b1 = make_float2(v[1].x - v[4].x, v[1].y - v[4].y);
-        const float2 b2 = make_float2(v[2].x - v[3].x, v[2].y - v[3].y);
-        const float2 m1 = make_float2(v[0].x + c1 * a1.x + c2 * a2.x, v[0].y + c1 * a1.y + c2 * a2.y);
-        const float2 m2 = make_float2(v[0].x + c2 * a1.x + c1 * a2.x, v[0].y + c2 * a1.y + c1 * a2.y);
-        const float2 n1 = make_float2(DIR * (s1 * b1.x + s2 * b2.x), DIR * (s1 * b1.y + s2 * b2.y));
-        const float2 n2 = make_float2(DIR * (s2 * b1.x - s1 * b2.x), DIR * (s2 * b1.y - s1 * b2.y));
-        v[0] = make_float2(v[0].x + a1.x + a2.x, v[0].y + a1.y + a2.y);
-        v[1] = make_float2(m1.x - n1.y, m1.y + n1.x);
-        v[4] = make_float2(m1.x + n1.y, m1.y - n1.x);
-        v[2] = make_float2(m2.x - n2.y, m2.y + n2.x);
-        v[3] = make_float2(m2.x + n2.y, m2.y - n2.x);
-    } else {
-        constexpr TwR<R> T = make_tw<R>();
-        float2 out[R];
-#pragma unroll
-        for (int p = 0; p < R; ++p) {
-            float2 acc = v[0];
-#pragma unroll
-            for (int q = 1; q < R; ++q) {
-                const float2 t = cmulf(v[q], T.c[(p * q) % R], DIR * T.s[(p * q) % R]);
-                acc.x += t.x;
-                acc.y += t.y;
-            }
-            out[p] = acc;
-        }
-#pragma unroll
-        for (int p = 0; p < R; ++p) v[p] = out[p];
-    }
-}
-
-// R = R1 * R2 point DFT on registers by one Cooley-Tukey split: with n = n1 + R1 n2 and
-// k = k2 + R2 k1, X[k] = sum_n1 w_R1^{n1 k1} w_R^{n1 k2} sum_n2 v[n] w_R2^{n2 k2}.
-template <int R1, int R2, int DIR>
-__device__ __forceinline__ void bfly_split(float2* v) {
-    constexpr int R = R1 * R2;
-    constexpr TwR<R> T = make_tw<R>();
-    float2 u[R];
-#pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1) {
-        float2 w[R2];
-#pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) w[n2] = v[n1 + R1 * n2];
-        bfly_prime<R2, DIR>(w);
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2)
-            u[n1 * R2 + k2] = (n1 * k2 == 0) ? w[k2] : cmulf(w[k2], T.c[(n1 * k2) % R], DIR * T.s[(n1 * k2) % R]);
-    }
-#pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) {
-        float2 z[R1];
-#pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) z[n1] = u[n1 * R2 + k2];
-        bfly_prime<R1, DIR>(z);
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) v[k2 + R2 * k1] = z[k1];
-    }
-}
-
-template <int R, int DIR>
-__device__ __forceinline__ void bfly(float2* v) {
-    if constexpr (R == 2 || R == 3 || R == 4 || R == 5) bfly_prime<R, DIR>(v);
-    else if constexpr (R == 6) bfly_split<2, 3, DIR>(v);
-    else if constexpr (R == 8) bfly_split<2, 4, DIR>(v);
-    else if constexpr (R == 9) bfly_split<3, 3, DIR>(v);
-    else if constexpr (R == 10) bfly_split<2, 5, DIR>(v);
-    else if constexpr (R == 12) bfly_split<4, 3, DIR>(v);
-    else if constexpr (R == 15) bfly_split<3, 5, DIR>(v);
-    else if constexpr (R == 16) bfly_split<4, 4, DIR>(v);
-    else if constexpr (R == 20) bfly_split<4, 5, DIR>(v);
-    else static_assert(R == 2, "unsupported radix");
-}
 
 template <int N, int NL, int R, int Ns, int DIR>
 __device__ __forceinline__ void stage_ct(const float2* src, float2* dst, const float2* __restrict__ tw) {

@@ -217,7 +217,7 @@ static void free_all(hmc_ctx* ctx) {
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     ctx->cap_stream = nullptr;
     batch_free(ctx);
-    void* bs[] = {ctx->batch_phi32, ctx->d_energy, ctx->batch.bar, ctx->batch.iters, ctx->batch.ch};
+    void* bs[] = {ctx->batch_phi32, ctx->d_energy, ctx->batch.ch};
     for (void* b : bs)
         if (b) cudaFree(b);
     for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
@@ -328,7 +328,6 @@ int hmc_init(const hmc_params* p, int n_chains, const hmc_chain* chains, void* c
         (rc = dalloc(ctx, &ctx->d_pi, nbw)) || (rc = dalloc(ctx, &ctx->d_F, nbw)) || (rc = dalloc(ctx, &ctx->d_vel, nbw)) ||
         (batch && ((rc = dalloc(ctx, &ctx->batch_phi32, 3 * ctx->vtot)) ||
                    (rc = dalloc(ctx, &ctx->d_energy, 9 * (int64_t)n_chains)) ||
-                   (rc = dalloc(ctx, &ctx->batch.bar, 2)) || (rc = dalloc(ctx, &ctx->batch.iters, 4)) ||
                    (rc = dalloc(ctx, &ctx->batch.ch, n_chains)))) ||
         (rc = dalloc(ctx, &ctx->d_z, nb)) || (rc = dalloc(ctx, &ctx->d_fft, nb)) ||
         (rc = dalloc(ctx, &ctx->d_part, ctx->part_cap)) || (rc = dalloc(ctx, &ctx->d_red, 64)) ||
@@ -945,7 +944,7 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
         rc = leapfrog();
     }
     // statistics of every solve, read once
-    std::vector<int> its((size_t)std::max(nsol, 1) * nc, 0), nru(std::max(nsol, 1), 0);
+    std::vector<int> its((size_t)std::max(nsol, 1) * nc, 0), nru((size_t)std::max(nsol, 1) * nc, 0);
     std::vector<double> wres((size_t)std::max(nsol, 1) * nc, 0.0);
     std::vector<int> tot_it(nc, 0);
     std::vector<double> worst(nc, 0.0);
@@ -957,7 +956,7 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
                 hmc_traj_stats& ts = ctx->tstats[c];
                 ts.iterations[j] = its[(size_t)j * nc + c];
                 ts.true_resid[j] = wres[(size_t)j * nc + c];
-                ts.reliable_updates += nru[j];
+                ts.reliable_updates += nru[(size_t)j * nc + c];
                 tot_it[c] += its[(size_t)j * nc + c];
                 worst[c] = std::max(worst[c], wres[(size_t)j * nc + c]);
             }

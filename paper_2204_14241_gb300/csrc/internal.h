@@ -52,30 +52,47 @@ struct ChainDesc {
     double r;
 };
 
-// Chain table of the batched solve (batch.cu): geometry, item offset of the chain's K
-// right-hand sides in the concatenated vectors, and its fields.
+// n / d for 0 <= n < 2^31 as umulhi(n, m) >> s (team.cu)
+struct FastDiv {
+    unsigned m, s;
+};
+
+// Geometry and fields of a chain in the team solver (team.cu): item offset of the chain's K right-hand
+// sides in the concatenated vectors.
 struct BChainDev {
     int L, Nt, LL;
-    float invL, invLL;
+    FastDiv dL, dLL;
     int64_t V;
     int64_t off;
     const double* phi64;
     const float* phi32;
 };
 
+// Statistics of one (chain, right-hand side) pair after a solve.
+struct TeamStat {
+    double r2true, b2;
+    int iters, n_ru;
+    int flags;   // 1: not converged, 2: non-finite
+    int pad;
+};
+
+struct TeamCap {   // resident blocks of one team kernel
+    int id;
+    size_t smem;
+    int blocks;
+};
+
 // Device state of the batched solve, built on first use for a right-hand-side count.
 struct BatchWork {
-    int K = 0, ntiles = 0, grid = 0;
-    int kcap = 0, ntiles_cap = 0;   // capacities allocated at hmc_init (nrhs_max right-hand sides)
-    void* tiles = nullptr;      // tile table
-    int* pair_t0 = nullptr;     // first tile of each (chain, RHS) pair
-    void* sc = nullptr;         // per-pair solver scalars
-    double* part = nullptr;     // per-tile partial sums
-    unsigned* bar = nullptr;    // grid barrier words
-    int* iters = nullptr;       // [0] iterations of the slowest pair, [1] reliable updates, [2] active pairs
+    int K = 0, grid = 0;
+    int kcap = 0, cap = 0;      // right-hand sides and resident blocks allocated for at hmc_init
+    void* pairs = nullptr;      // TeamPair table, each team's pairs together
+    int2* blk = nullptr;        // per block: first pair of its team, number of pairs
+    unsigned long long* part = nullptr;   // partial sums
+    unsigned* bar = nullptr;    // an arrival counter per pair
     BChainDev* ch = nullptr;    // chain table (n_chains entries)
-    void* hist = nullptr;       // per-solve statistics of every pair, HMC_MAX_SOLVES solves of a trajectory
-    int* hist_ru = nullptr;     // reliable updates of each solve
+    TeamStat* hist = nullptr;   // per-solve statistics of every pair, HMC_MAX_SOLVES solves of a trajectory
+    int* fail = nullptr;        // failure flags of every solve of the trajectory
     std::vector<BChainDev> hch; // host copy of the chain table of the current trajectory
 };
 
@@ -165,6 +182,7 @@ struct hmc_ctx {
     int* d_flags = nullptr;           // device error word [0]: bit 0 a bounded wait gave up, bit 1 its drain did too
     int* h_flags = nullptr;           // pinned mirror
 
+    std::vector<hmc::TeamCap> team_caps;      // resident blocks of the team kernels
 };
 
 namespace hmc {
@@ -250,6 +268,7 @@ int launch_boson(hmc_ctx* ctx, const Lat& lat, double r, const double* phi, doub
 
 // fft.cu
 FftPlan* get_plan(hmc_ctx* ctx, int n);
+PcTables* get_pc(hmc_ctx* ctx, int L, int Nt);
 int build_plans(hmc_ctx* ctx);
 void free_plans(hmc_ctx* ctx);
 // unitary FFT of complex data viewed as [outer][n][inner] along the middle axis, in place
@@ -292,13 +311,13 @@ unsigned int bounds_take_strip();
 
 // batch.cu: all (chain, RHS) pairs of the context solve A X = b in one persistent launch (mixed
 // precision, no preconditioner). b, x: concatenated [chain][k][V][4] complex128.
-// batch_alloc (hmc_init) allocates the workspace for nrhs_max; batched_begin builds the tile
-// table for K right-hand sides and uploads the chain table (phi pointers) of a trajectory;
+// batch_alloc (hmc_init) allocates the workspace for nrhs_max; batched_begin deals the blocks to the
+// pairs for K right-hand sides and uploads the chain table (phi pointers) of a trajectory;
 // batched_solve enqueues one solve of every pair from b into x (from x when use_x0) and records
 // its statistics in slot `slot` on the device, with no host synchronisation (so it can be
 // captured in a CUDA graph); batched_collect reads the statistics of solves [0, nsolves) back: per
-// solve and chain the iterations of its slowest pair and its worst true relative residual, per
-// solve the reliable updates.
+// solve and chain the iterations of its slowest pair, its worst true relative residual and its reliable
+// updates.
 int batch_alloc(hmc_ctx* ctx);
 int batched_begin(hmc_ctx* ctx, int K, const double* const* phi);
 int batched_solve(hmc_ctx* ctx, int K, const double2* b, double2* x, bool use_x0, double tol, int maxit, int slot);
@@ -311,6 +330,9 @@ int check_device_flags(hmc_ctx* ctx);
 
 // reductions: sum nblk partials for each of k rows into out[k] (device)
 int reduce_rows(hmc_ctx* ctx, const double* part, int k, int nblk, double* out);
+
+// b = (float) a (cg.cu)
+int launch_phi_to32(hmc_ctx* ctx, const double* a, float* b, int64_t n);
 
 // cg.cu; with use_x0 the solve starts from the contents of x instead of zero. y_ready (may be
 // null): set when ctx->d_z64 holds D^dagger x of the returned solution, computed in FP64 by the

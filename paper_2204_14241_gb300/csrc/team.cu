@@ -1,0 +1,1135 @@
+// Whole solves A X = varphi (Eq. linsys) in one launch: CG or preconditioned CG (P of Eq. precon), in
+// complex64 with FP64 reliable updates or in complex128, by teams of blocks.
+//
+// Every (chain, right-hand side) pair is a system of its own, so it gets its own team of T resident
+// blocks with its own barrier, scalars and stopping test; nothing waits for another pair. (With one
+// barrier for all pairs, every pair of a 64-chain batch stood still for each other pair's reliable
+// updates, 225 of them in a solve.) A team is a thread-block cluster where the system is small, else blocks
+// of a cooperative launch.
+//
+// Small lattices are bound by latency, a launch or a barrier after every few microseconds of work: with a
+// launch per step and the host reading flags an iteration took 27 to 60 us (CG, PCG) whatever the size, here
+// 5 to 7 and 14 to 30 up to some 30000 sites. From about 10^5 sites memory bounds complex64 and the FP64 pipe
+// complex128.
+//
+// Work is dealt in items, one band's two spin components of one site (16 bytes in complex64): a block
+// owns a contiguous range of its pair's 2 V items, or, for the preconditioned phases, whole (time
+// slice, band) planes. Phases of one iteration, separated by team barriers:
+//   CG, complex64   p = r + beta p_old formed at each item and its neighbours on the fly, t_ =
+//                   D^dagger p, <p, A p> = ||t_||^2 | q = D t_ (never stored), x, r, ||r||^2
+//   CG, complex128  t_ = D^dagger p | q, x, r | p = r + beta p: the FP64 pipe bounds it, so that p is
+//                   not formed seven times
+//   PCG             t_ = D^dagger p | q, x, r of a plane, then its (x, y) FFT in shared memory | tau
+//                   FFT, P-hat, inverse, <r, z> | inverse (x, y) FFT, p = z + beta p
+// Each block sums its team's partials itself, in the same order, so all blocks hold the same scalars
+// and take the same decisions: no scalar kernel, no flag to read back, no host in the loop.
+// Vectors that other blocks write are read with plain loads: the barrier's acquire drops the SM's L1
+// lines, and within a phase L1 then serves the neighbours (read through L2 instead, 14 site loads per site
+// in the first phase, and with FP64 sums, an iteration of the 64-chain batch took 0.37 ms; now 0.17).
+//
+// A cooperative team's barrier spins on a counter with a time limit; a block that gives up sets the device
+// error word and returns.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "dft.cuh"
+#include "fft_ct.h"
+#include "internal.h"
+#include "team.h"
+
+namespace hmc {
+
+template <typename R> struct It { cplx<R> s[2]; };   // one band of one site: its two spin components
+
+template <typename R> __device__ __forceinline__ It<R> ld_it(const cplx<R>* v, int64_t i) {
+    It<R> o;
+    if constexpr (sizeof(R) == 4) {
+        const float4 a = *reinterpret_cast<const float4*>(v + 2 * i);
+        o.s[0] = make_float2(a.x, a.y);
+        o.s[1] = make_float2(a.z, a.w);
+    } else {
+        o.s[0] = v[2 * i];
+        o.s[1] = v[2 * i + 1];
+    }
+    return o;
+}
+template <typename R> __device__ __forceinline__ void st_it(cplx<R>* v, int64_t i, const It<R>& o) {
+    if constexpr (sizeof(R) == 4) {
+        *reinterpret_cast<float4*>(v + 2 * i) = make_float4(o.s[0].x, o.s[0].y, o.s[1].x, o.s[1].y);
+    } else {
+        v[2 * i] = o.s[0];
+        v[2 * i + 1] = o.s[1];
+    }
+}
+template <typename R> __device__ __forceinline__ It<R> axpy_it(R a, const It<R>& x, const It<R>& y) {
+    It<R> o;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        o.s[s].x = fma(a, x.s[s].x, y.s[s].x);
+        o.s[s].y = fma(a, x.s[s].y, y.s[s].y);
+    }
+    return o;
+}
+
+// v with its sign changed when bit 0 of `neg` is set (integer units: an FP64 multiply costs a slot of
+// the pipe that bounds the FP64 phases)
+__device__ __forceinline__ float flip(float v, int neg) {
+    return __int_as_float(__float_as_int(v) ^ (neg << 31));
+}
+__device__ __forceinline__ double flip(double v, int neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg << 31), __double2loint(v));
+}
+
+__device__ __forceinline__ int fdiv(int n, FastDiv d) { return (int)(__umulhi((unsigned)n, d.m) >> d.s); }
+
+// Item i of D v (DAG = false) or D^dagger v: the stencil of site_op (common.cuh) for one band, the
+// vector read through ld(item).
+template <typename R, bool DAG, typename Ld>
+__device__ __forceinline__ It<R> d_item(const BChainDev& g, const Coef<R>& cf, const R* __restrict__ phi, int i,
+                                        const Ld& ld, It<R>* centre = nullptr) {
+    const int band = i & 1, s = i >> 1;
+    const int t = fdiv(s, g.dLL), rem = s - t * g.LL, y = fdiv(rem, g.dL), x = rem - y * g.L;
+    const int L = g.L, LL = g.LL, hop = 2 * ((int)g.V - LL);
+    const It<R> c = ld(i), w = ld(i ^ 1);
+    const It<R> xm = ld(x ? i - 2 : i + 2 * (L - 1)), xp = ld(x + 1 < L ? i + 2 : i - 2 * (L - 1));
+    const It<R> ym = ld(y ? i - 2 * L : i + 2 * (LL - L)), yp = ld(y + 1 < L ? i + 2 * L : i - 2 * (LL - L));
+    const int edge = DAG ? (t == 0) : (t + 1 == g.Nt);   // the time hop crosses the antiperiodic boundary
+    const It<R> tn = ld(DAG ? (edge ? i + hop : i - 2 * LL) : (edge ? i - hop : i + 2 * LL));
+    const R f = flip(cf.cpl, (x + y) & 1);
+    const R q1 = f * __ldg(phi + s), q2 = f * __ldg(phi + g.V + s), q3 = f * __ldg(phi + 2 * g.V + s);
+    const R d = band ? cf.diag[1] : cf.diag[0], hx = band ? cf.hx[1] : cf.hx[0], hy = band ? cf.hy[1] : cf.hy[0];
+    It<R> o;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        o.s[q].x = fma(d, c.s[q].x, flip(tn.s[q].x, edge));
+        o.s[q].y = fma(d, c.s[q].y, flip(tn.s[q].y, edge));
+        o.s[q].x = fma(hx, xm.s[q].x + xp.s[q].x, o.s[q].x);
+        o.s[q].y = fma(hx, xm.s[q].y + xp.s[q].y, o.s[q].y);
+        o.s[q].x = fma(hy, ym.s[q].x + yp.s[q].x, o.s[q].x);
+        o.s[q].y = fma(hy, ym.s[q].y + yp.s[q].y, o.s[q].y);
+    }
+    const cplx<R> w0 = w.s[0], w1 = w.s[1];
+    o.s[0].x = fma(q3, w0.x, fma(q1, w1.x, fma(q2, w1.y, o.s[0].x)));
+    o.s[0].y = fma(q3, w0.y, fma(q1, w1.y, fma(-q2, w1.x, o.s[0].y)));
+    o.s[1].x = fma(-q3, w1.x, fma(q1, w0.x, fma(-q2, w0.y, o.s[1].x)));
+    o.s[1].y = fma(-q3, w1.y, fma(q1, w0.y, fma(q2, w0.x, o.s[1].y)));
+    if (centre) *centre = c;
+    return o;
+}
+
+// Per-thread sum of squares: FP64, or an FP32 pair with exact products and compensated additions (48
+// bits). Converting every component of an FP32 vector for an FP64 sum takes more of the FP64 pipe's
+// time (two lanes a clock per SM) than the rest of a phase takes.
+template <typename R> struct Sum2;
+template <> struct Sum2<double> {
+    using T = double;
+    double v = 0.0;
+    __device__ __forceinline__ void add(double w, double x) { v = fma(w * x, x, v); }
+    __device__ __forceinline__ void sq(double x) { v = fma(x, x, v); }
+    __device__ __forceinline__ void plus(const Sum2& o) { v += o.v; }
+    __device__ __forceinline__ unsigned long long bits() const { return (unsigned long long)__double_as_longlong(v); }
+    __device__ __forceinline__ void from(unsigned long long b) { v = __longlong_as_double((long long)b); }
+    __device__ __forceinline__ double get() const { return v; }
+};
+template <> struct Sum2<float> {
+    using T = float;
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void term(float p, float e) {   // += p + e
+        const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b))));
+        hi = s;
+    }
+    __device__ __forceinline__ void sq(float x) {
+        const float p = __fmul_rn(x, x);
+        term(p, __fmaf_rn(x, x, -p));
+    }
+    __device__ __forceinline__ void add(float w, float x) {   // w x^2, w x rounded once
+        const float y = __fmul_rn(w, x), p = __fmul_rn(y, x);
+        term(p, __fmaf_rn(y, x, -p));
+    }
+    __device__ __forceinline__ void plus(const Sum2& o) { term(o.hi, o.lo); }
+    __device__ __forceinline__ unsigned long long bits() const {
+        return (unsigned long long)__float_as_uint(hi) << 32 | __float_as_uint(lo);
+    }
+    __device__ __forceinline__ void from(unsigned long long b) {
+        hi = __uint_as_float((unsigned)(b >> 32));
+        lo = __uint_as_float((unsigned)b);
+    }
+    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+};
+template <typename S> __device__ __forceinline__ void warp_plus(S& a, int from_lane_bit) {   // xor tree below the bit
+    for (int o = from_lane_bit; o > 0; o >>= 1) {
+        S b;
+        b.from(__shfl_xor_sync(0xffffffffu, a.bits(), o));
+        a.plus(b);
+    }
+}
+template <typename R> __device__ __forceinline__ void sq_it(Sum2<R>& a, const It<R>& o) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        a.sq(o.s[s].x);
+        a.sq(o.s[s].y);
+    }
+}
+
+// a / b to an ulp or so: two Newton steps on the FP32 quotient (FP64 latency is what a scalar costs here: a
+// full division takes three times as long), or the division where FP32 does not reach
+__device__ __forceinline__ double quot(double a, double b) {
+    const float bf = (float)b, af = (float)a;
+    if (!(fabsf(bf) > 1e-30f && fabsf(bf) < 1e30f && fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return a / b;
+    const double y = (double)(1.0f / bf);
+    double q = a * y;
+    q = fma(fma(-q, b, a), y, q);
+    return fma(fma(-q, b, a), y, q);
+}
+
+struct NoSum {   // a barrier without a sum
+    using T = float;
+    __device__ __forceinline__ void plus(const NoSum&) {}
+    __device__ __forceinline__ unsigned long long bits() const { return 0; }
+    __device__ __forceinline__ void from(unsigned long long) {}
+    __device__ __forceinline__ double get() const { return 0.0; }
+};
+
+// ---- team ------------------------------------------------------------------------------------------
+// Scalars of a solve, in shared memory: written by one thread, so that no other spends the FP64 pipe's
+// time on them (a double division by all 256 threads takes 0.7 us of it).
+template <typename R> struct Ctl {
+    double rr, b2, r2, r2true, r2max;
+    R alpha, beta;
+    int it, n_ru, hold, wait;
+    int active, nonfinite, met, ru, last;
+    int ok;
+};
+
+struct Team {
+    int b0, T, rank;            // first block, blocks, this block's place
+    unsigned* cnt;              // arrivals, never reset within a launch
+    unsigned long long* part;   // [2][gridDim.x] partial sums, by the barrier's parity
+    unsigned long long* cpart;  // [2][16], shared memory: the same for a cluster
+    unsigned epoch;
+    bool never;                 // the next barrier waits for more arrivals than there are blocks (timeout test)
+    bool shared_sm;             // other blocks may be at work on this SM
+    int* flags;
+    long long timeout_ns;
+};
+
+__device__ __forceinline__ long long gtimer() {
+    long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Waits for `want` arrivals (one lane). An acquiring load drops the SM's L1 lines, other blocks' too, so
+// where others share the SM the polls are relaxed with one fence after them (0.3 us more).
+__device__ __forceinline__ bool wait_arrivals(const Team& tm, unsigned want) {
+    long long t0 = 0;
+    for (unsigned n = 1;; ++n) {
+        unsigned v;
+        if (tm.shared_sm) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(tm.cnt) : "memory");
+        else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(tm.cnt) : "memory");
+        if ((int)(v - want) >= 0) break;
+        if ((n & 63) == 0) {
+            const long long now = gtimer();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > tm.timeout_ns) {
+                atomicOr(tm.flags, 1);
+                return false;
+            }
+        }
+    }
+    if (tm.shared_sm) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return true;
+}
+
+// Barrier of the team's blocks with the sum of `acc` over all their threads; writes before it are seen by
+// plain loads after it. All blocks add in the same order; lane 0 then runs fin(sum) for everybody. False
+// (with the error word set) when the wait gives up.
+//  CLU: the team is a thread-block cluster; partials go to every block's shared memory and the hardware
+//       barrier orders them: 0.4 thousand clocks, 1.5 with the data's way through L2.
+//  otherwise: an arrival counter in L2, 2.5 to 3.2 thousand clocks for 16 to 150 blocks, and 0.7 for the
+//       partials. (Blocks that post their partial with the barrier's epoch in one 16-byte word for all the
+//       others to poll save the second read, but took 4.5 to 5.9 from 50 blocks on.)
+template <bool CLU, typename S, typename C, typename Fin>
+__device__ __forceinline__ bool sync_sum(Team& tm, C& ctl, unsigned long long* red, S acc, const Fin& fin) {
+    constexpr bool k64 = sizeof(typename S::T) == 8;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if constexpr (k64) {
+        red[threadIdx.x] = acc.bits();
+    } else {
+        warp_plus(acc, 16);
+        if (lane == 0) red[w] = acc.bits();
+    }
+    __syncthreads();
+    ++tm.epoch;
+    const int par = tm.epoch & 1;
+    if (w == 0) {
+        if constexpr (k64) {
+            // one warp adds the block's values: in the shuffle tree of every warp each addition would take
+            // the SM's FP64 pipe 16 clocks a warp
+            for (int j = 1; j < nw; ++j) {
+                S o;
+                o.from(red[lane + 32 * j]);
+                acc.plus(o);
+            }
+            warp_plus(acc, 16);
+        } else {
+            acc = S();
+            if (lane < nw) acc.from(red[lane]);
+            warp_plus(acc, nw > 8 ? 8 : 4);   // 8 or 16 warps
+        }
+        if constexpr (CLU) {
+            if (lane < tm.T) {
+                const unsigned mine = (unsigned)__cvta_generic_to_shared(tm.cpart + 16 * par + tm.rank);
+                unsigned theirs;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(lane));
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(theirs), "l"(acc.bits()) : "memory");
+            }
+        }
+    }
+    bool ok = true;
+    if constexpr (CLU) {
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (w == 0) {
+            acc = S();
+            if (lane < tm.T) acc.from(tm.cpart[16 * par + lane]);
+            warp_plus(acc, 8);
+        }
+    } else if (w == 0 && (tm.T > 1 || tm.never)) {
+        unsigned long long* row = tm.part + par * gridDim.x + tm.b0;
+        if (lane == 0) {
+            __stcg(row + tm.rank, acc.bits());
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(tm.cnt) : "memory");
+            ok = wait_arrivals(tm, tm.epoch * tm.T + (tm.never ? 1u << 20 : 0u));
+        }
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        __syncwarp();
+        if (!std::is_same<S, NoSum>::value) {
+            acc = S();
+            for (int b = lane; b < tm.T; b += 32) {
+                S o;
+                o.from(__ldcg(row + b));
+                acc.plus(o);
+            }
+            warp_plus(acc, 16);
+        }
+    }
+    if (w == 0 && lane == 0) {
+        ctl.ok = ok ? 1 : 0;
+        if (ok) fin(acc.get());
+    }
+    __syncthreads();
+    tm.never = false;
+    return ctl.ok != 0;
+}
+
+// ---- FFTs of the preconditioned phases ---------------------------------------------------------------
+// All R-point DFTs of one step over lines of single components in shared memory, forward sign. The tile
+// holds planes of `nl` lines, `plane` entries apart; line l of a plane starts at (l & 1) + (l >> 1) * ls, the
+// points of DFT f at f * fs + m * ps; with tw, output m is multiplied by tw[f m]. Inverse steps run the same
+// code on data with re and im exchanged.
+struct Lines {
+    int np, plane, nl;   // planes, entries between them, lines of a plane
+    FastDiv dnl;
+};
+template <int R, typename C>
+__device__ __noinline__ void dft_pass(C* sm, const Lines ln, int nf, int ls, int fs, int ps, const C* tw) {
+    const int total = ln.np * ln.nl * nf;
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+        const int q = fdiv(idx, ln.dnl), l = idx - q * ln.nl;   // q = plane * nf + f
+        int p = 0, f = q;
+        if (ln.np > 1) { p = q / nf; f = q - p * nf; }
+        C* base = sm + p * ln.plane + (l & 1) + (l >> 1) * ls + f * fs;
+        C v[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = base[m * ps];
+        bfly<R, -1>(v);
+        if (tw) {
+#pragma unroll
+            for (int m = 1; m < R; ++m) v[m] = cmul(v[m], tw[f * m]);
+        }
+#pragma unroll
+        for (int m = 0; m < R; ++m) base[m * ps] = v[m];
+    }
+}
+template <typename C>
+__device__ __forceinline__ void dft_step(int R, C* sm, const Lines& ln, int nf, int ls, int fs, int ps, const C* tw) {
+    if (R == 1) return;
+    switch (R) {
+        case 2: dft_pass<2>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 3: dft_pass<3>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 4: dft_pass<4>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 5: dft_pass<5>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 6: dft_pass<6>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 7: dft_pass<7>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 8: dft_pass<8>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 9: dft_pass<9>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 10: dft_pass<10>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 12: dft_pass<12>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 14: dft_pass<14>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 15: dft_pass<15>(sm, ln, nf, ls, fs, ps, tw); break;
+        case 16: dft_pass<16>(sm, ln, nf, ls, fs, ps, tw); break;
+        default: break;
+    }
+    __syncthreads();
+}
+template <typename C> __device__ __forceinline__ C swapc(C a) { return mk<C>(a.y, a.x); }
+
+// Shared tables of the preconditioned phases, behind the FFT tile. Positions: after a forward split
+// N = N1 N2 position N1 k2 + k1 holds frequency k2 + N2 k1 (see fft_ct.cu).
+template <typename R> struct PreTab {
+    using C = cplx<R>;
+    C *tile, *twx, *twt, *twist, *ew;
+    R* cosk;
+};
+template <typename R> __device__ __forceinline__ PreTab<R> pre_tables(const TeamPre<R>& q, int L, int Nt, unsigned char* sm) {
+    PreTab<R> p;
+    using C = cplx<R>;
+    p.tile = reinterpret_cast<C*>(sm);
+    p.twx = p.tile + q.tile;
+    p.twt = p.twx + L;
+    p.twist = p.twt + Nt;
+    p.ew = p.twist + Nt;
+    p.cosk = reinterpret_cast<R*>(p.ew + Nt);
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        p.twx[i] = __ldg(q.twx + i);
+        p.cosk[i] = __ldg(q.cosk + (i / q.x1 + q.x2 * (i % q.x1)));
+    }
+    for (int i = threadIdx.x; i < Nt; i += blockDim.x) {
+        p.twt[i] = __ldg(q.twt + i);
+        p.twist[i] = __ldg(q.twist + i);
+        p.ew[i] = __ldg(q.eitw + (i / q.t1 + q.t2 * (i % q.t1)));
+    }
+    __syncthreads();
+    return p;
+}
+__device__ __forceinline__ int row_stride(int L) { return L | 1; }   // odd: rows fall in distinct banks
+
+// Planes of the tile -> zhat: forward FFTs along x, then y, and the spectra out, band-major. Plane p is task
+// t0 + p * T (slice task / 2, band task % 2).
+template <typename R>
+__device__ __forceinline__ void plane_forward(const TeamPre<R>& q, const PreTab<R>& p, const BChainDev& g, int t0, int T,
+                                              int np, cplx<R>* z) {
+    const int L = g.L, RS = row_stride(L);
+    const Lines ln{np, q.plane, 2 * L, q.d2L};
+    __syncthreads();
+    dft_step(q.x2, p.tile, ln, q.x1, 2 * RS, 2, 2 * q.x1, p.twx);
+    dft_step(q.x1, p.tile, ln, q.x2, 2 * RS, 2 * q.x1, 2, (const cplx<R>*)nullptr);
+    dft_step(q.x2, p.tile, ln, q.x1, 2, 2 * RS, 2 * RS * q.x1, p.twx);
+    dft_step(q.x1, p.tile, ln, q.x2, 2, 2 * RS * q.x1, 2 * RS, (const cplx<R>*)nullptr);
+    for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
+        const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), x = j - y * L;
+        z[(int64_t)(t0 + pl * T) * g.LL * 2 + 2 * j + (e & 1)] = p.tile[pl * q.plane + (y * RS + x) * 2 + (e & 1)];
+    }
+    __syncthreads();
+}
+
+// One team's solve of right-hand side k of chain g; false when a barrier gave up.
+template <typename R, bool PRE, bool CLU>
+__device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>& c, const BChainDev& g, int k, int pair,
+                                         const PreTab<R>& pt, unsigned long long* red) {
+    constexpr bool kMixed = sizeof(R) == 4;
+    using C = cplx<R>;
+    const int64_t off = (g.off + (int64_t)k * g.V) * 4;   // complex entries
+    const int n = 2 * (int)g.V;
+    const int per = ((n + tm.T - 1) / tm.T + 31) & ~31;
+    const int i0 = min(tm.rank * per, n), i1 = min(i0 + per, n);
+    const double2 *b = a.b + off;
+    double2 *x64 = a.x64 + off, *t64 = a.t64 + off;
+    C *r = a.r + off, *t = a.t + off, *pold = a.pA + off, *pnew = kMixed && !PRE ? a.pB + off : a.pA + off;
+    C* x;
+    if constexpr (kMixed) x = a.x + off;
+    else x = x64;
+    C* z = PRE ? a.z + off : nullptr;
+    const R* phi;
+    if constexpr (kMixed) phi = g.phi32;
+    else phi = g.phi64;
+    auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](double) {}); };
+    auto ld64 = [](const double2* v) { return [v](int j) { return ld_it<double>(v, j); }; };
+    auto ldr = [](const C* v) { return [v](int j) { return ld_it<R>(v, j); }; };
+
+    // ---- start: r = b - A x (or b), zero directions, norms ----------------------------------------
+    if (a.use_x0) {
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true>(g, a.cf64, g.phi64, i, ld64(x64)));
+        if (!sync()) return false;
+    }
+    {
+        Sum2<double> sb, sr;
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            const It<double> bb = ld_it<double>(b, i);
+            It<double> rr = bb;
+            if (a.use_x0) {
+                rr = axpy_it<double>(-1.0, d_item<double, false>(g, a.cf64, g.phi64, i, ld64(t64)), bb);
+            } else {
+                st_it<double>(x64, i, It<double>{});
+                st_it<double>(t64, i, It<double>{});   // D^dagger x of the zero start
+            }
+            It<R> rl;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rr.s[s].x, (R)rr.s[s].y);
+            st_it<R>(r, i, rl);
+            if constexpr (kMixed) st_it<R>(x, i, It<R>{});
+            // the first direction is r (or z): the on-the-fly and the inverse-FFT forms add 0 * p
+            st_it<R>(pold, i, !kMixed && !PRE ? rl : It<R>{});
+            sq_it(sb, bb);
+            sq_it(sr, rr);
+        }
+        if (!sync_sum<CLU>(tm, c, red, sb, [&](double v) { c.b2 = v; })) return false;
+        if (!sync_sum<CLU>(tm, c, red, sr, [&](double v) {
+                c.r2 = c.r2true = c.r2max = c.rr = v;
+                c.alpha = c.beta = (R)0;
+                c.it = c.n_ru = c.hold = 0;
+                c.wait = 4;
+                c.nonfinite = !(isfinite(c.b2) && isfinite(v));
+                c.active = !c.nonfinite && c.b2 > 0.0 && v > a.tol2 * c.b2;
+            }))
+            return false;
+    }
+
+    // this block's (slice, band) planes, tasks rank, rank + T, ..., as many at a time as the tile holds
+    auto each_round = [&](const auto& f) {
+        const int own = tm.rank < 2 * g.Nt ? (2 * g.Nt - tm.rank + tm.T - 1) / tm.T : 0;
+        for (int j = 0; j < own; j += a.pre.np) f(tm.rank + j * tm.T, min(a.pre.np, own - j));
+    };
+    // f(item, place in the tile) for the sites of planes t0, t0 + T, ...
+    auto each_site = [&](int t0, int np, const auto& f) {
+        const int RS = row_stride(g.L);
+        for (int e = threadIdx.x; e < np * g.LL; e += blockDim.x) {
+            const int pl = fdiv(e, g.dLL), j = e - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * g.L;
+            const int task = t0 + pl * tm.T;
+            f(2 * ((task >> 1) * g.LL + j) + (task & 1), pl * a.pre.plane + (y * RS + xx) * 2);
+        }
+    };
+    // spectra of r's planes
+    auto forward = [&]() {
+        each_round([&](int t0, int np) {
+            each_site(t0, np, [&](int i, int at) {
+                const It<R> v = ld_it<R>(r, i);
+                pt.tile[at] = v.s[0];
+                pt.tile[at + 1] = v.s[1];
+            });
+            plane_forward<R>(a.pre, pt, g, t0, tm.T, np, z);
+        });
+    };
+    // tau pass in place on z; this thread's part of <r, z> (before the transforms' scale)
+    auto tau = [&]() {
+        const TeamPre<R>& q = a.pre;
+        const int w2 = 2 * q.W, ng = (g.LL + q.W - 1) / q.W;
+        const Lines ln{1, 0, w2, q.dw2};
+        __shared__ R base_s[kTeamTau];
+        Sum2<R> acc;
+        for (int task = tm.rank; task < 2 * ng; task += tm.T) {
+            const int band = task & 1, j0 = (task >> 1) * q.W;
+            for (int p = threadIdx.x; p < q.W; p += blockDim.x) {
+                const int j = min(j0 + p, g.LL - 1), y = fdiv(j, g.dL), xx = j - y * g.L;
+                base_s[p] = q.c0[band] + q.chx[band] * pt.cosk[xx] + q.chy[band] * pt.cosk[y];
+            }
+            C* zp = z + ((int64_t)band * g.LL + j0) * 2;
+            const int64_t step = (int64_t)4 * g.LL;
+            const int live = 2 * min(q.W, g.LL - j0);
+            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
+                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
+                pt.tile[e] = l < live ? cmulconj(pt.twist[ts], zp[ts * step + l]) : mk<C>(0, 0);
+            }
+            __syncthreads();
+            dft_step(q.t2, pt.tile, ln, q.t1, 2, w2, w2 * q.t1, pt.twt);
+            dft_step(q.t1, pt.tile, ln, q.t2, 2, w2 * q.t1, w2, (const C*)nullptr);
+            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
+                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
+                const C w = pt.ew[ts];
+                const R re = w.x + base_s[l >> 1];
+                const R ph = (R)1 / (re * re + w.y * w.y);
+                const C v = pt.tile[e];
+                acc.add(ph, v.x);
+                acc.add(ph, v.y);
+                pt.tile[e] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
+            }
+            __syncthreads();
+            dft_step(q.t1, pt.tile, ln, q.t2, 2, w2 * q.t1, w2, pt.twt);
+            dft_step(q.t2, pt.tile, ln, q.t1, 2, w2, w2 * q.t1, (const C*)nullptr);
+            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
+                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
+                if (l < live) zp[ts * step + l] = cmul(swapc(pt.tile[e]), pt.twist[ts]);
+            }
+            __syncthreads();
+        }
+        return acc;
+    };
+    // p = z + beta p by inverse FFTs of z's planes
+    auto inverse = [&]() {
+        const TeamPre<R>& q = a.pre;
+        const R be = c.beta, sc = (R)q.scale;
+        const int L = g.L, RS = row_stride(L);
+        each_round([&](int t0, int np) {
+            const Lines ln{np, q.plane, 2 * L, q.d2L};
+            for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
+                const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * L;
+                pt.tile[pl * q.plane + (y * RS + xx) * 2 + (e & 1)] =
+                    swapc(z[(int64_t)(t0 + pl * tm.T) * g.LL * 2 + 2 * j + (e & 1)]);
+            }
+            __syncthreads();
+            dft_step(q.x1, pt.tile, ln, q.x2, 2, 2 * RS * q.x1, 2 * RS, pt.twx);
+            dft_step(q.x2, pt.tile, ln, q.x1, 2, 2 * RS, 2 * RS * q.x1, (const C*)nullptr);
+            dft_step(q.x1, pt.tile, ln, q.x2, 2 * RS, 2 * q.x1, 2, pt.twx);
+            dft_step(q.x2, pt.tile, ln, q.x1, 2 * RS, 2, 2 * q.x1, (const C*)nullptr);
+            each_site(t0, np, [&](int i, int at) {
+                It<R> v;
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const C d = pt.tile[at + s];
+                    v.s[s] = mk<C>(sc * d.y, sc * d.x);
+                }
+                st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), v));
+            });
+            __syncthreads();
+        });
+        return sync();
+    };
+    if constexpr (PRE) {
+        if (c.active) {   // first direction p = z, rr = <r, z>
+            forward();
+            if (!sync()) return false;
+            if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
+                    c.rr = v * a.pre.scale;
+                    if (!isfinite(v)) c.nonfinite = 1;
+                }))
+                return false;
+            if (!inverse()) return false;
+        }
+    }
+
+    while (c.active && !c.nonfinite) {
+        // ---- t_ = D^dagger p; alpha = rr / <p, A p> ----
+        Sum2<R> acc;
+        if constexpr (kMixed && !PRE) {
+            const R be = c.beta;
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+                It<R> pc;
+                const It<R> o = d_item<R, true>(
+                    g, a.cf, phi, i, [&](int j) { return axpy_it<R>(be, ld_it<R>(pold, j), ld_it<R>(r, j)); }, &pc);
+                st_it<R>(pnew, i, pc);
+                st_it<R>(t, i, o);
+                sq_it(acc, o);
+            }
+        } else {
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+                const It<R> o = d_item<R, true>(g, a.cf, phi, i, ldr(pold));
+                st_it<R>(t, i, o);
+                sq_it(acc, o);
+            }
+        }
+        if (!sync_sum<CLU>(tm, c, red, acc, [&](double pAp) {
+                c.alpha = (R)((pAp > 0.0 && isfinite(pAp)) ? quot(c.rr, pAp) : 0.0);
+                if (!isfinite(pAp)) c.nonfinite = 1;
+            }))
+            return false;
+        // ---- q = D t_, x += alpha p, r -= alpha q, ||r||^2 (PRE: and the spectrum of r) ----
+        acc = Sum2<R>();
+        const R al = c.alpha;
+        auto update = [&](int i) {
+            const It<R> q = d_item<R, false>(g, a.cf, phi, i, ldr(t));
+            st_it<R>(x, i, axpy_it<R>(al, ld_it<R>(pnew, i), ld_it<R>(x, i)));
+            const It<R> rn = axpy_it<R>(-al, q, ld_it<R>(r, i));
+            st_it<R>(r, i, rn);
+            sq_it(acc, rn);
+            return rn;
+        };
+        if constexpr (PRE) {
+            each_round([&](int t0, int np) {
+                each_site(t0, np, [&](int i, int at) {
+                    const It<R> v = update(i);
+                    pt.tile[at] = v.s[0];
+                    pt.tile[at + 1] = v.s[1];
+                });
+                plane_forward<R>(a.pre, pt, g, t0, tm.T, np, z);
+            });
+        } else {
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) update(i);
+        }
+        if (!sync_sum<CLU>(tm, c, red, acc, [&](double v) {
+                c.r2 = v;
+                if (!isfinite(v)) c.nonfinite = 1;
+                if constexpr (!PRE) {
+                    c.beta = (R)(c.rr > 0.0 ? quot(v, c.rr) : 0.0);
+                    c.rr = v;
+                }
+                c.last = ++c.it >= a.maxit;
+                // Near the rounding floor of the true residual, an update after every iteration that meets
+                // the tolerance would put its noise back into the recurrence each time and hardly ever stop:
+                // after one that misses, some iterations pass before the next.
+                c.met = v <= a.tol2 * c.b2 && c.it >= c.hold;
+                c.ru = c.met || (kMixed && v < a.delta2 * c.r2max) || c.last;
+            }))
+            return false;
+        if (c.nonfinite) break;
+        if constexpr (kMixed && !PRE) { C* s = pold; pold = pnew; pnew = s; }
+        const bool ru = c.ru;
+        if (ru) {
+            // ---- reliable update: x64 += x, r = b - A x64 in FP64 ----
+            if constexpr (kMixed) {
+                for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+                    const It<R> lo = ld_it<R>(x, i);
+                    It<double> hi = ld_it<double>(x64, i);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        hi.s[s].x += (double)lo.s[s].x;
+                        hi.s[s].y += (double)lo.s[s].y;
+                    }
+                    st_it<double>(x64, i, hi);
+                    st_it<R>(x, i, It<R>{});
+                }
+                if (!sync()) return false;
+            }
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true>(g, a.cf64, g.phi64, i, ld64(x64)));
+            if (!sync()) return false;
+            Sum2<double> acc64;
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+                const It<double> rd =
+                    axpy_it<double>(-1.0, d_item<double, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i));
+                It<R> rl;
+#pragma unroll
+                for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rd.s[s].x, (R)rd.s[s].y);
+                st_it<R>(r, i, rl);
+                sq_it(acc64, rd);
+            }
+            if (!sync_sum<CLU>(tm, c, red, acc64, [&](double v) {
+                    c.r2true = v;
+                    ++c.n_ru;
+                    if (!isfinite(v)) c.nonfinite = 1;
+                    else if (v <= a.tol2 * c.b2) c.active = 0;
+                    else {
+                        c.r2max = v;
+                        if constexpr (!PRE) c.rr = v;
+                        if (c.met) {
+                            c.hold = c.it + c.wait;
+                            c.wait = 8;
+                        }
+                    }
+                }))
+                return false;
+            if (c.nonfinite || !c.active || c.last) break;
+        }
+        if constexpr (PRE) {
+            if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
+                    v *= a.pre.scale;
+                    c.beta = (R)(c.rr > 0.0 ? quot(v, c.rr) : 0.0);
+                    c.rr = v;
+                    if (!isfinite(v)) c.nonfinite = 1;
+                }))
+                return false;
+            if (ru) {
+                // beta belongs to the recurrence (the spectrum that was in z): taken from the new residual,
+                // which near the floor is larger, it would blow the old direction up
+                forward();
+                if (!sync()) return false;
+                if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
+                        c.rr = v * a.pre.scale;
+                        if (!isfinite(v)) c.nonfinite = 1;
+                    }))
+                    return false;
+            }
+            if (c.nonfinite) break;
+            if (!inverse()) return false;
+        } else if constexpr (!kMixed) {
+            const R be = c.beta;
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
+                st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), ld_it<R>(r, i)));
+            if (!sync()) return false;
+        }
+    }
+    if (tm.rank == 0 && threadIdx.x == 0) {
+        const int f = (c.active && !c.nonfinite ? 1 : 0) | (c.nonfinite ? 2 : 0);
+        if (a.fail && f) atomicOr(a.fail, f);
+        if (a.stat) a.stat[pair] = TeamStat{c.r2true, c.b2, c.it, c.n_ru, f, 0};
+    }
+    return true;
+}
+
+// Registers: 128 for the preconditioned kernels and for FP64 (the FP64 radix steps take 196), 80 for
+// complex64 CG, three blocks per SM: its phases wait on L2.
+template <typename R, bool PRE, bool CLU> struct TeamBounds {
+    static constexpr int threads = CLU && !(PRE && sizeof(R) == 8) ? 512 : 256;
+    static constexpr int blocks = CLU ? 1 : sizeof(R) == 4 && !PRE ? 3 : 2;
+};
+template <typename R, bool PRE, bool CLU>
+__global__ void __launch_bounds__(TeamBounds<R, PRE, CLU>::threads, TeamBounds<R, PRE, CLU>::blocks)
+k_team(const __grid_constant__ TeamArgs<R> a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long red[TeamBounds<R, PRE, CLU>::threads];
+    __shared__ unsigned long long cpart[2 * 16];
+    __shared__ BChainDev g;
+    __shared__ Ctl<R> ctl;
+    Team tm;
+    tm.part = a.part;
+    tm.cpart = cpart;
+    tm.never = a.test_timeout != 0;
+    tm.shared_sm = a.pairs != nullptr;
+    tm.flags = a.flags;
+    tm.timeout_ns = a.timeout_ns;
+    PreTab<R> pt;
+    if constexpr (PRE) pt = pre_tables<R>(a.pre, a.one.L, a.one.Nt, smem);
+    // entries [mine.x, mine.x + mine.y) of the table of pairs, in turn
+    const int2 mine = a.pairs ? a.blk[blockIdx.x] : make_int2(blockIdx.x / a.T, 1);
+    for (int e = mine.x; e < mine.x + mine.y; ++e) {
+        TeamPair tp{0, e, e * a.T, a.T};
+        if (a.pairs) tp = a.pairs[e];
+        __syncthreads();
+        if (threadIdx.x == 0) g = a.pairs ? a.ch[tp.chain] : a.one;
+        __syncthreads();
+        tm.b0 = tp.b0;
+        tm.T = tp.T;
+        tm.rank = blockIdx.x - tp.b0;
+        tm.cnt = a.bar + e;
+        tm.epoch = 0;
+        if (!team_run<R, PRE, CLU>(a, tm, ctl, g, tp.k, tp.chain * a.K + tp.k, pt, red)) return;
+    }
+}
+
+// ---- host --------------------------------------------------------------------------------------------
+static FastDiv fast_div(int d) {   // n / d for 0 <= n < 2^31, d >= 2
+    FastDiv f;
+    int s = 1;
+    while ((int64_t(1) << s) < d) ++s;
+    f.m = (unsigned)((uint64_t(1) << (31 + s)) / (unsigned)d + 1);
+    f.s = (unsigned)(s - 1);
+    return f;
+}
+
+void team_geometry(BChainDev* d, const Lat& lat) {
+    d->L = lat.L;
+    d->Nt = lat.Nt;
+    d->LL = lat.L * lat.L;
+    d->V = lat.V;
+    d->dL = fast_div(lat.L);
+    d->dLL = fast_div(lat.L * lat.L);
+}
+
+// N = n1 n2 with both factors among dft_step's radices, their sum (the work per point) least; up to 10
+// points in one step: a step costs its latency, not its work, at the sizes that take few points
+static bool split(int n, int* n1, int* n2) {
+    static const int radix[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};
+    if (n <= 10) {
+        *n1 = n;
+        *n2 = 1;
+        return true;
+    }
+    int best = 1 << 30;
+    for (int a : radix)
+        for (int b : radix)
+            if (a * b == n && a >= b && a + b < best) {
+                best = a + b;
+                *n1 = a;
+                *n2 = b;
+            }
+    return best < (1 << 30);
+}
+
+template <typename R> static const cplx<R>* plan_tw(const FftPlan* p);
+template <> const float2* plan_tw<float>(const FftPlan* p) { return p->tw32; }
+template <> const double2* plan_tw<double>(const FftPlan* p) { return p->tw64; }
+
+// Tables and splits of the preconditioned phases; false when the lattice has no two-factor split.
+template <typename R> static bool pre_setup(hmc_ctx* ctx, const Lat& lat, TeamPre<R>* q) {
+    const FftPlan *px = get_plan(ctx, lat.L), *ptau = get_plan(ctx, lat.Nt);
+    const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
+    if (!px || !ptau || !pc || !split(lat.L, &q->x1, &q->x2) || !split(lat.Nt, &q->t1, &q->t2)) return false;
+    q->twx = plan_tw<R>(px);
+    q->twt = plan_tw<R>(ptau);
+    if constexpr (sizeof(R) == 4) {
+        q->cosk = pc->cosk32;
+        q->eitw = pc->eitw32;
+        q->twist = pc->twist32;
+    } else {
+        q->cosk = pc->cosk;
+        q->eitw = pc->eitw;
+        q->twist = pc->twist;
+    }
+    const double dt = ctx->p.dtau;
+    for (int s = 0; s < 2; ++s) {
+        q->c0[s] = (R)(-1.0 - dt * ctx->p.mu[s]);
+        q->chx[s] = (R)(-2.0 * dt * ctx->p.t_h[s]);
+        q->chy[s] = (R)(-2.0 * dt * ctx->p.t_v[s]);
+    }
+    q->d2L = fast_div(2 * lat.L);
+    q->scale = 1.0 / ((double)lat.L * lat.L * lat.Nt);   // the unnormalised transforms both ways
+    q->plane = lat.L * (lat.L | 1) * 2;
+    return true;
+}
+
+// Planes in the shared tile at a time and tau tiles for teams of T blocks, within `most` bytes; returns the
+// dynamic shared memory, 0 when not even one plane fits.
+template <typename R> static size_t pre_tiles(TeamPre<R>* q, const Lat& lat, int T, size_t most) {
+    const int own = (2 * lat.Nt + T - 1) / T, LL = lat.L * lat.L;
+    const size_t tables = (size_t)(lat.L + 3 * lat.Nt) * sizeof(cplx<R>) + (size_t)lat.L * sizeof(R);
+    const int room = most > tables ? (int)((most - tables) / sizeof(cplx<R>)) : 0;
+    q->np = std::min(own, room / q->plane);
+    // as many tau tiles as blocks
+    q->W = std::min({kTeamTau, (2 * LL + T - 1) / T, room / (2 * lat.Nt)});
+    if (q->np < 1 || q->W < 1) return 0;
+    q->dw2 = fast_div(2 * q->W);
+    q->tile = std::max(q->np * q->plane, lat.Nt * 2 * q->W);
+    return tables + (size_t)q->tile * sizeof(cplx<R>);
+}
+
+template <typename R, bool PRE, bool CLU> static int set_attr(hmc_ctx* ctx) {
+    static PerDevice attr;
+    uint64_t bit;
+    if (!attr.pending(&bit)) return HMC_OK;
+    if (PRE)
+        HMC_CUDA(ctx, cudaFuncSetAttribute(k_team<R, PRE, CLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTeamSmem));
+    if (CLU) HMC_CUDA(ctx, cudaFuncSetAttribute(k_team<R, PRE, CLU>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    attr.mark(bit);
+    return HMC_OK;
+}
+
+// resident blocks of k_team<R, PRE, false> with `smem` bytes of dynamic shared memory
+template <typename R, bool PRE> static int capacity(hmc_ctx* ctx, size_t smem, int* cap) {
+    int rc;
+    if ((rc = set_attr<R, PRE, false>(ctx))) return rc;
+    const int id = (sizeof(R) == 8 ? 2 : 0) + (PRE ? 1 : 0);
+    for (const TeamCap& c : ctx->team_caps)
+        if (c.id == id && c.smem == smem) {
+            *cap = c.blocks;
+            return HMC_OK;
+        }
+    int bps = 0;
+    HMC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_team<R, PRE, false>,
+                                                                TeamBounds<R, PRE, false>::threads, smem));
+    *cap = bps * ctx->num_sms;
+    ctx->team_caps.push_back(TeamCap{id, smem, *cap});
+    return HMC_OK;
+}
+
+// Cooperative launch, or one cluster per right-hand side (CLU), through the attribute form, which stream
+// capture records as such a kernel node.
+template <typename R, bool PRE, bool CLU>
+static int launch(hmc_ctx* ctx, const TeamArgs<R>& a, int grid, size_t smem, int npairs) {
+    int rc;
+    if ((rc = set_attr<R, PRE, CLU>(ctx))) return rc;
+    if (!CLU) HMC_CUDA(ctx, cudaMemsetAsync(a.bar, 0, npairs * sizeof(unsigned), ctx->stream));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(TeamBounds<R, PRE, CLU>::threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    if (CLU) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = a.T;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    HMC_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_team<R, PRE, CLU>, a));
+    HMC_LAUNCH(ctx, "k_team");
+    return HMC_OK;
+}
+
+int team_batch_capacity(hmc_ctx* ctx, int* cap) { return capacity<float, false>(ctx, 0, cap); }
+
+int team_launch_batch(hmc_ctx* ctx, const TeamArgs<float>& a, int grid, int npairs) {
+    return launch<float, false, false>(ctx, a, grid, 0, npairs);
+}
+
+// clusters of T blocks of k_team<R, PRE, true> that are resident at a time
+template <typename R, bool PRE> static int clusters(hmc_ctx* ctx, int T, size_t smem, int* cap) {
+    int rc;
+    if ((rc = set_attr<R, PRE, true>(ctx))) return rc;
+    const int id = 4 + 8 * T + (sizeof(R) == 8 ? 2 : 0) + (PRE ? 1 : 0);
+    for (const TeamCap& c : ctx->team_caps)
+        if (c.id == id && c.smem == smem) {
+            *cap = c.blocks;
+            return HMC_OK;
+        }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)T);
+    cfg.blockDim = dim3(TeamBounds<R, PRE, true>::threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = T;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    HMC_CUDA(ctx, cudaOccupancyMaxActiveClusters(cap, k_team<R, PRE, true>, &cfg));
+    ctx->team_caps.push_back(TeamCap{id, smem, *cap});
+    return HMC_OK;
+}
+
+// How a solve runs: clusters of T blocks, or teams of T blocks of a cooperative launch; T = 0: neither.
+struct TeamPlan {
+    int T = 0;
+    bool cluster = false;
+    size_t smem = 0;
+};
+template <typename R>
+static int make_plan(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond, TeamPre<R>* pre, TeamPlan* plan) {
+    if (precond && !pre_setup<R>(ctx, lat, pre)) return HMC_OK;
+    const int64_t n = 2 * lat.V;
+    int cap = 0, rc;
+    // A cluster where its threads have few items each, measured against a team of a cooperative launch
+    // (microseconds an iteration, one right-hand side): CG in complex64 5.5 : 7.0 at 16 x 16 x 16 (8192 items,
+    // one each) but 7.3 : 6.8 at 16 x 16 x 32; PCG 18.4 : 19.9 and 23.1 : 18.9 there; PCG in FP64, whose pipe
+    // wants more SMs, 29.6 : 32.7 at 8 x 8 x 16 but 47.9 : 42.3 at 10 x 10 x 20; CG in FP64 16.4 : 13.9 at
+    // 6 x 6 x 12. A right-hand side of one block needs no barrier beyond the block's (3.4 : 4.8 at 4 x 4 x 8).
+    if constexpr (sizeof(R) == 4) {
+        if (!ctx->p.test_wait_timeout && n > (precond ? 0 : 512)) {
+            for (int T = 16; T >= 2; T /= 2) {
+                if (n > (precond ? 512 : 768) * (int64_t)T) break;
+                if (n <= 256 * (int64_t)T && T > 2 && (!precond || 2 * lat.Nt <= T / 2)) continue;   // half as many do
+                if (precond && !(plan->smem = pre_tiles<R>(pre, lat, T, kTeamSmem))) continue;
+                if ((rc = precond ? clusters<R, true>(ctx, T, plan->smem, &cap) : clusters<R, false>(ctx, T, 0, &cap)))
+                    return rc;
+                if (cap < nrhs) continue;   // the others would run one after another
+                plan->T = T;
+                plan->cluster = true;
+                return HMC_OK;
+            }
+        }
+    } else {
+        if (!ctx->p.test_wait_timeout && precond && n <= 2048) {
+            for (int T = 16; T >= 8; T /= 2) {
+                if (!(plan->smem = pre_tiles<R>(pre, lat, T, kTeamSmem))) continue;
+                if ((rc = clusters<R, true>(ctx, T, plan->smem, &cap))) return rc;
+                if (cap < nrhs) continue;
+                plan->T = T;
+                plan->cluster = true;
+                return HMC_OK;
+            }
+        }
+    }
+    if (precond) {
+        // shared memory for two resident blocks if a plane fits in half an SM's
+        for (const int most : {kTeamSmem / 2, kTeamSmem}) {
+            if (!pre_tiles<R>(pre, lat, 1 << 20, most)) continue;   // one plane
+            if ((rc = capacity<R, true>(ctx, most, &cap))) return rc;
+            const int tasks = 2 * lat.Nt, avail = cap / nrhs;
+            if (avail < 1) return HMC_OK;
+            const int rounds = (tasks + avail - 1) / avail;
+            // one block an SM and a last round that leaves SMs idle: 1162 us an iteration at 60 x 60 x 120 in FP64,
+            // 1103 by the separate kernels
+            if (most == kTeamSmem && 5 * (int64_t)tasks < 4 * (int64_t)rounds * avail) return HMC_OK;
+            plan->T = (tasks + rounds - 1) / rounds;
+            plan->smem = pre_tiles<R>(pre, lat, plan->T, most);
+            return HMC_OK;
+        }
+        return HMC_OK;
+    }
+    if ((rc = capacity<R, false>(ctx, 0, &cap))) return rc;
+    plan->T = (int)std::min<int64_t>(cap / nrhs, (n + 255) / 256);
+    return HMC_OK;
+}
+
+template <typename R>
+static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2* b, double2* x, int nrhs, double tol,
+                 int maxit, int precond, hmc_cg_stats* st, bool use_x0, bool* y_ready, bool* done) {
+    *done = false;
+    TeamArgs<R> a{};
+    TeamPlan plan;
+    int rc;
+    if ((rc = make_plan<R>(ctx, lat, nrhs, precond, &a.pre, &plan))) return rc;
+    const int T = plan.T;
+    if (T < 1 || 2 * (int64_t)T * nrhs + nrhs > ctx->part_cap) return HMC_OK;
+    *done = true;
+    team_geometry(&a.one, lat);
+    a.one.off = 0;
+    a.one.phi64 = phi;
+    a.one.phi32 = ctx->d_phi32;
+    a.T = T;
+    a.K = nrhs;
+    a.cf = make_coef<R>(ctx->p);
+    a.cf64 = make_coef<double>(ctx->p);
+    a.b = b;
+    a.x64 = x;
+    a.t64 = ctx->d_z64;
+    if constexpr (sizeof(R) == 4) {
+        if ((rc = launch_phi_to32(ctx, phi, ctx->d_phi32, 3 * lat.V))) return rc;
+        a.x = ctx->d_x32;
+        a.r = ctx->d_r32;
+        a.pA = ctx->d_p32;
+        a.pB = ctx->d_p32b;
+        a.t = ctx->d_q32;
+        a.z = ctx->d_z32;
+    } else {
+        a.r = ctx->d_r64;
+        a.pA = ctx->d_p64;
+        a.t = ctx->d_q64;
+        a.z = ctx->d_p64b;
+    }
+    a.bar = reinterpret_cast<unsigned*>(ctx->d_part);
+    a.part = reinterpret_cast<unsigned long long*>(ctx->d_part) + nrhs;
+    a.flags = ctx->d_flags;
+    // statistics in the scalars of the separate kernels, which this solve does not use
+    static_assert(sizeof(TeamStat) <= sizeof(CgScalars), "statistics fit");
+    a.stat = reinterpret_cast<TeamStat*>(ctx->d_cg);
+    a.tol2 = tol * tol;
+    a.delta2 = 1e-6;
+    a.maxit = maxit;
+    a.use_x0 = use_x0 ? 1 : 0;
+    a.test_timeout = ctx->p.test_wait_timeout;
+    // wait_spin_limit counts the strip operator's polls, microseconds of a batched solve; here it only
+    // shortens the wait that a timeout test lets run out
+    a.timeout_ns = a.test_timeout && ctx->p.wait_spin_limit > 0 ? (long long)ctx->p.wait_spin_limit * 1000LL
+                                                                : 2000000000LL;
+    const int grid = T * nrhs;
+    if (plan.cluster && precond) rc = launch<R, true, true>(ctx, a, grid, plan.smem, nrhs);
+    else if (plan.cluster) {
+        if constexpr (sizeof(R) == 4) rc = launch<R, false, true>(ctx, a, grid, 0, nrhs);
+    } else
+        rc = precond ? launch<R, true, false>(ctx, a, grid, plan.smem, nrhs) : launch<R, false, false>(ctx, a, grid, 0, nrhs);
+    if (rc) return rc;
+    HMC_CUDA(ctx, cudaMemcpyAsync(ctx->h_cg, a.stat, nrhs * sizeof(TeamStat), cudaMemcpyDeviceToHost, ctx->stream));
+    if ((rc = check_device_flags(ctx))) return rc;   // synchronises
+    double worst = 0.0;
+    int iters = 0, n_ru = 0, f = 0;
+    for (int k = 0; k < nrhs; ++k) {
+        const TeamStat& s = reinterpret_cast<const TeamStat*>(ctx->h_cg)[k];
+        const double rel = s.b2 > 0.0 ? std::sqrt(s.r2true / s.b2) : 0.0;
+        if (!(rel <= worst)) worst = rel;
+        iters = std::max(iters, s.iters);
+        n_ru = std::max(n_ru, s.n_ru);
+        f |= s.flags;
+    }
+    if (st) {
+        st->iterations = iters;
+        st->reliable_updates = n_ru;
+        st->converged = f == 0;
+        st->true_rel_resid = worst;
+    }
+    if (f & 2) return fail(ctx, HMC_ERR_NONFINITE, "cg_solve: non-finite residual norm");
+    if (f & 1) return fail(ctx, HMC_ERR_NOCONV, "cg_solve: no convergence in " + std::to_string(maxit) + " iterations");
+    // every right-hand side stopped at a true residual of its final x, whose t_ = D^dagger x is in d_z64
+    if (y_ready) *y_ready = true;
+    return HMC_OK;
+}
+
+// Where one launch is the faster way (microseconds an iteration, one launch : the kernels of cg.cu):
+//  CG, complex64   strip lattices 73 : 83 at 80 x 80 x 160, 73 : 82 at 64 x 64 x 128 with 2 right-hand sides, but
+//                  152 : 137 with 2 at 80 x 80 x 160: past about a million sites the strip operator's traffic
+//                  counts; other lattices 394 : 412 at 70 x 70 x 140 with 8
+//  CG, complex128  2991 : 4300 at 80 x 80 x 160 with 8
+//  PCG, complex64  lattices with compiled FFT passes 82 : 93 at 40 x 40 x 80 with 3, but 229 : 182 with 8; others
+//                  (no compiled length) 1316 : 2805 at 70 x 70 x 140 with 8
+//  PCG, complex128 3441 : 4328 at 64 x 64 x 128 with 4
+static bool worth_it(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond) {
+    const int64_t sites = (int64_t)nrhs * lat.V;
+    if (sites > (int64_t)1 << 23) return false;   // the largest measured
+    if (ctx->p.solver_mode != HMC_SOLVER_MIXED) return true;
+    if (precond) return sites <= 400000 || !(fftc_supported(lat.L) && fftc_can(lat.Nt, 4 * (int64_t)lat.L * lat.L));
+    return sites <= 1250000 || !strip_supported(lat);
+}
+
+int team_solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2* b, double2* x, int nrhs, double tol,
+               int maxit, int precond, hmc_cg_stats* st, bool use_x0, bool* y_ready, bool* done) {
+    *done = false;
+    if (!worth_it(ctx, lat, nrhs, precond)) return HMC_OK;
+    if (ctx->p.solver_mode == HMC_SOLVER_MIXED)
+        return solve<float>(ctx, lat, phi, b, x, nrhs, tol, maxit, precond, st, use_x0, y_ready, done);
+    return solve<double>(ctx, lat, phi, b, x, nrhs, tol, maxit, precond, st, use_x0, y_ready, done);
+}
+
+}  // namespace hmc
