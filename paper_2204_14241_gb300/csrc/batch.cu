@@ -24,10 +24,10 @@ __global__ void k_phi_to32_b(const BChainDev* __restrict__ ch) {
 // ---- host ----------------------------------------------------------------------------------------
 void batch_free(hmc_ctx* ctx) {
     BatchWork& w = ctx->batch;
-    void* ps[] = {w.pairs, w.blk, w.part, w.bar, w.hist, w.fail};
+    void* ps[] = {w.pairs, w.blk, w.part, w.bar, w.hist, w.fail, w.metric};
     for (void* p : ps)
         if (p) cudaFree(p);
-    w.pairs = nullptr; w.blk = nullptr; w.part = nullptr; w.bar = nullptr; w.hist = nullptr; w.fail = nullptr;
+    w.pairs = nullptr; w.blk = nullptr; w.part = nullptr; w.bar = nullptr; w.hist = nullptr; w.fail = nullptr; w.metric = nullptr;
     w.K = 0;
     w.kcap = 0;
 }
@@ -46,6 +46,7 @@ int batch_alloc(hmc_ctx* ctx) {
     HMC_CUDA(ctx, cudaMalloc((void**)&w.bar, np * sizeof(unsigned)));
     HMC_CUDA(ctx, cudaMalloc((void**)&w.hist, HMC_MAX_SOLVES * np * sizeof(TeamStat)));
     HMC_CUDA(ctx, cudaMalloc((void**)&w.fail, sizeof(int)));
+    if ((rc = metric_batch_alloc(ctx))) return rc;
     w.kcap = ctx->kmax;
     w.K = 0;
     w.hch.resize(ctx->chains.size());

@@ -761,12 +761,15 @@ static int fft3_real_field(hmc_ctx* ctx, const Lat& lat, double2* v, int dir) {
 
 int metric_op(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in,
               double* out, double eps, double* scalar_dev) {
+    bool done = false;
+    int rc = metric_real(ctx, lat, op, sig, in, out, eps, scalar_dev, &done);
+    if (rc || done) return rc;
+    // extents without a two-factor split, or planes past an SM's shared memory: complex transforms axis by axis
     const int64_t n = 3 * lat.V;
     const unsigned nb = (unsigned)((n + 255) / 256);
     double2* v = ctx->d_fft;
     k_pack_real<<<nb, 256, 0, ctx->stream>>>(in, v, n);
     HMC_LAUNCH(ctx, "k_pack_real");
-    int rc;
     if ((rc = fft3_real_field(ctx, lat, v, -1))) return rc;
     if (op == HMC_METRIC_KINETIC || op == HMC_METRIC_MNORM) {
         if (nb > ctx->part_cap) return fail(ctx, HMC_ERR_ARG, "metric: reduction buffer too small");

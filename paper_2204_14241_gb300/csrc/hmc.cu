@@ -804,6 +804,7 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
     // its statistics on the device (slot = solve index) and nothing in it waits for the host, so
     // with batch_graph the whole leapfrog is captured once and replayed as a CUDA graph
     if ((rc = batched_begin(ctx, K, phis.data()))) return rc;
+    if ((rc = metric_batch_begin(ctx, (const double* const*)in->sigma_hat, (double* const*)in->phi))) return rc;
     const int mode = ctx->p.initial_guess;
     double2* hist[kMaxGuess + 1] = {ctx->d_X};
     for (int j = 1; j <= mode; ++j) hist[j] = ctx->d_Xhist[j - 1];
@@ -869,7 +870,8 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
         HMC_LAUNCH(ctx, "k_axpy");
         for (int i = 1; i <= in->n_leap; ++i) {
             if ((r2 = mark(kPhaseMetric))) return r2;
-            for (int c = 0; c < nc; ++c)
+            if (ctx->batch.metric_ok && (r2 = metric_batch_drift(ctx, eps))) return r2;
+            for (int c = 0; c < nc && !ctx->batch.metric_ok; ++c)
                 if ((r2 = metric_op(ctx, ctx->chains[c].lat, HMC_METRIC_VELOCITY, (const double*)in->sigma_hat[c],
                                     bvec(ctx->d_pi, c), (double*)in->phi[c], eps, nullptr)))
                     return r2;

@@ -93,6 +93,10 @@ struct BatchWork {
     BChainDev* ch = nullptr;    // chain table (n_chains entries)
     TeamStat* hist = nullptr;   // per-solve statistics of every pair, HMC_MAX_SOLVES solves of a trajectory
     int* fail = nullptr;        // failure flags of every solve of the trajectory
+    void* metric = nullptr;     // transform table of the drift (metric.cu), every chain
+    std::vector<char> hmetric;  // its host copy
+    bool metric_ok = false;     // every chain's lattice has the real transforms
+    int maxL = 0, maxNt = 0;
     std::vector<BChainDev> hch; // host copy of the chain table of the current trajectory
 };
 
@@ -298,6 +302,14 @@ int launch_pcg_xy_forward(hmc_ctx* ctx, const Lat& lat, float2* x, float2* r, co
                           int* nblk_r2, int* nblk_rz);
 int launch_pcg_xy_inverse(hmc_ctx* ctx, const Lat& lat, const float2* zhat, const float2* pold, float2* pnew,
                           int nrhs, const CgScalars* cgs);
+// metric.cu: the same on real transforms; *done = false where the lattice rules them out
+int metric_real(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in, double* out, double eps,
+                double* scalar_dev, bool* done);
+// the drift phi += eps F^-1(sigma F pi) of every chain of a batch (pi in ctx->d_pi), three launches:
+// metric_batch_begin uploads a trajectory's table (and sets batch.metric_ok), metric_batch_drift enqueues one
+int metric_batch_alloc(hmc_ctx* ctx);
+int metric_batch_begin(hmc_ctx* ctx, const double* const* sig, double* const* phi);
+int metric_batch_drift(hmc_ctx* ctx, double eps);
 int metric_op(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in,
               double* out, double eps, double* scalar_dev);
 

@@ -33,7 +33,7 @@
 #include <cmath>
 #include <type_traits>
 
-#include "dft.cuh"
+#include "dft_smem.cuh"
 #include "fft_ct.h"
 #include "internal.h"
 #include "team.h"
@@ -80,8 +80,6 @@ __device__ __forceinline__ float flip(float v, int neg) {
 __device__ __forceinline__ double flip(double v, int neg) {
     return __hiloint2double(__double2hiint(v) ^ (neg << 31), __double2loint(v));
 }
-
-__device__ __forceinline__ int fdiv(int n, FastDiv d) { return (int)(__umulhi((unsigned)n, d.m) >> d.s); }
 
 // Item i of D v (DAG = false) or D^dagger v: the stencil of site_op (common.cuh) for one band, the
 // vector read through ld(item).
@@ -325,59 +323,8 @@ __device__ __forceinline__ bool sync_sum(Team& tm, C& ctl, unsigned long long* r
 }
 
 // ---- FFTs of the preconditioned phases ---------------------------------------------------------------
-// All R-point DFTs of one step over lines of single components in shared memory, forward sign. The tile
-// holds planes of `nl` lines, `plane` entries apart; line l of a plane starts at (l & 1) + (l >> 1) * ls, the
-// points of DFT f at f * fs + m * ps; with tw, output m is multiplied by tw[f m]. Inverse steps run the same
-// code on data with re and im exchanged.
-struct Lines {
-    int np, plane, nl;   // planes, entries between them, lines of a plane
-    FastDiv dnl;
-};
-template <int R, typename C>
-__device__ __noinline__ void dft_pass(C* sm, const Lines ln, int nf, int ls, int fs, int ps, const C* tw) {
-    const int total = ln.np * ln.nl * nf;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int q = fdiv(idx, ln.dnl), l = idx - q * ln.nl;   // q = plane * nf + f
-        int p = 0, f = q;
-        if (ln.np > 1) { p = q / nf; f = q - p * nf; }
-        C* base = sm + p * ln.plane + (l & 1) + (l >> 1) * ls + f * fs;
-        C v[R];
-#pragma unroll
-        for (int m = 0; m < R; ++m) v[m] = base[m * ps];
-        bfly<R, -1>(v);
-        if (tw) {
-#pragma unroll
-            for (int m = 1; m < R; ++m) v[m] = cmul(v[m], tw[f * m]);
-        }
-#pragma unroll
-        for (int m = 0; m < R; ++m) base[m * ps] = v[m];
-    }
-}
-template <typename C>
-__device__ __forceinline__ void dft_step(int R, C* sm, const Lines& ln, int nf, int ls, int fs, int ps, const C* tw) {
-    if (R == 1) return;
-    switch (R) {
-        case 2: dft_pass<2>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 3: dft_pass<3>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 4: dft_pass<4>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 5: dft_pass<5>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 6: dft_pass<6>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 7: dft_pass<7>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 8: dft_pass<8>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 9: dft_pass<9>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 10: dft_pass<10>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 12: dft_pass<12>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 14: dft_pass<14>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 15: dft_pass<15>(sm, ln, nf, ls, fs, ps, tw); break;
-        case 16: dft_pass<16>(sm, ln, nf, ls, fs, ps, tw); break;
-        default: break;
-    }
-    __syncthreads();
-}
-template <typename C> __device__ __forceinline__ C swapc(C a) { return mk<C>(a.y, a.x); }
-
-// Shared tables of the preconditioned phases, behind the FFT tile. Positions: after a forward split
-// N = N1 N2 position N1 k2 + k1 holds frequency k2 + N2 k1 (see fft_ct.cu).
+// Shared tables of the preconditioned phases, behind the FFT tile; cosk and ew by position after the
+// forward steps.
 template <typename R> struct PreTab {
     using C = cplx<R>;
     C *tile, *twx, *twt, *twist, *ew;
@@ -394,12 +341,12 @@ template <typename R> __device__ __forceinline__ PreTab<R> pre_tables(const Team
     p.cosk = reinterpret_cast<R*>(p.ew + Nt);
     for (int i = threadIdx.x; i < L; i += blockDim.x) {
         p.twx[i] = __ldg(q.twx + i);
-        p.cosk[i] = __ldg(q.cosk + (i / q.x1 + q.x2 * (i % q.x1)));
+        p.cosk[i] = __ldg(q.cosk + dft_freq(i, q.x1, q.x2));
     }
     for (int i = threadIdx.x; i < Nt; i += blockDim.x) {
         p.twt[i] = __ldg(q.twt + i);
         p.twist[i] = __ldg(q.twist + i);
-        p.ew[i] = __ldg(q.eitw + (i / q.t1 + q.t2 * (i % q.t1)));
+        p.ew[i] = __ldg(q.eitw + dft_freq(i, q.t1, q.t2));
     }
     __syncthreads();
     return p;
@@ -412,12 +359,10 @@ template <typename R>
 __device__ __forceinline__ void plane_forward(const TeamPre<R>& q, const PreTab<R>& p, const BChainDev& g, int t0, int T,
                                               int np, cplx<R>* z) {
     const int L = g.L, RS = row_stride(L);
-    const Lines ln{np, q.plane, 2 * L, q.d2L};
+    const Lines rows{np, q.plane, 2 * L, q.d2L, 1, 2 * RS}, cols{np, q.plane, 2 * L, q.d2L, 1, 2};
     __syncthreads();
-    dft_step(q.x2, p.tile, ln, q.x1, 2 * RS, 2, 2 * q.x1, p.twx);
-    dft_step(q.x1, p.tile, ln, q.x2, 2 * RS, 2 * q.x1, 2, (const cplx<R>*)nullptr);
-    dft_step(q.x2, p.tile, ln, q.x1, 2, 2 * RS, 2 * RS * q.x1, p.twx);
-    dft_step(q.x1, p.tile, ln, q.x2, 2, 2 * RS * q.x1, 2 * RS, (const cplx<R>*)nullptr);
+    dft_forward(p.tile, rows, q.x1, q.x2, 2, p.twx);
+    dft_forward(p.tile, cols, q.x1, q.x2, 2 * RS, p.twx);
     for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
         const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), x = j - y * L;
         z[(int64_t)(t0 + pl * T) * g.LL * 2 + 2 * j + (e & 1)] = p.tile[pl * q.plane + (y * RS + x) * 2 + (e & 1)];
@@ -516,7 +461,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     auto tau = [&]() {
         const TeamPre<R>& q = a.pre;
         const int w2 = 2 * q.W, ng = (g.LL + q.W - 1) / q.W;
-        const Lines ln{1, 0, w2, q.dw2};
+        const Lines ln{1, 0, w2, q.dw2, 1, 2};
         __shared__ R base_s[kTeamTau];
         Sum2<R> acc;
         for (int task = tm.rank; task < 2 * ng; task += tm.T) {
@@ -533,8 +478,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 pt.tile[e] = l < live ? cmulconj(pt.twist[ts], zp[ts * step + l]) : mk<C>(0, 0);
             }
             __syncthreads();
-            dft_step(q.t2, pt.tile, ln, q.t1, 2, w2, w2 * q.t1, pt.twt);
-            dft_step(q.t1, pt.tile, ln, q.t2, 2, w2 * q.t1, w2, (const C*)nullptr);
+            dft_forward(pt.tile, ln, q.t1, q.t2, w2, pt.twt);
             for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
                 const int ts = fdiv(e, q.dw2), l = e - ts * w2;
                 const C w = pt.ew[ts];
@@ -546,8 +490,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 pt.tile[e] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
             }
             __syncthreads();
-            dft_step(q.t1, pt.tile, ln, q.t2, 2, w2 * q.t1, w2, pt.twt);
-            dft_step(q.t2, pt.tile, ln, q.t1, 2, w2, w2 * q.t1, (const C*)nullptr);
+            dft_inverse(pt.tile, ln, q.t1, q.t2, w2, pt.twt);
             for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
                 const int ts = fdiv(e, q.dw2), l = e - ts * w2;
                 if (l < live) zp[ts * step + l] = cmul(swapc(pt.tile[e]), pt.twist[ts]);
@@ -562,17 +505,15 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         const R be = c.beta, sc = (R)q.scale;
         const int L = g.L, RS = row_stride(L);
         each_round([&](int t0, int np) {
-            const Lines ln{np, q.plane, 2 * L, q.d2L};
+            const Lines rows{np, q.plane, 2 * L, q.d2L, 1, 2 * RS}, cols{np, q.plane, 2 * L, q.d2L, 1, 2};
             for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
                 const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * L;
                 pt.tile[pl * q.plane + (y * RS + xx) * 2 + (e & 1)] =
                     swapc(z[(int64_t)(t0 + pl * tm.T) * g.LL * 2 + 2 * j + (e & 1)]);
             }
             __syncthreads();
-            dft_step(q.x1, pt.tile, ln, q.x2, 2, 2 * RS * q.x1, 2 * RS, pt.twx);
-            dft_step(q.x2, pt.tile, ln, q.x1, 2, 2 * RS, 2 * RS * q.x1, (const C*)nullptr);
-            dft_step(q.x1, pt.tile, ln, q.x2, 2 * RS, 2 * q.x1, 2, pt.twx);
-            dft_step(q.x2, pt.tile, ln, q.x1, 2 * RS, 2, 2 * q.x1, (const C*)nullptr);
+            dft_inverse(pt.tile, cols, q.x1, q.x2, 2 * RS, pt.twx);
+            dft_inverse(pt.tile, rows, q.x1, q.x2, 2, pt.twx);
             each_site(t0, np, [&](int i, int at) {
                 It<R> v;
 #pragma unroll
@@ -787,15 +728,6 @@ k_team(const __grid_constant__ TeamArgs<R> a) {
 }
 
 // ---- host --------------------------------------------------------------------------------------------
-static FastDiv fast_div(int d) {   // n / d for 0 <= n < 2^31, d >= 2
-    FastDiv f;
-    int s = 1;
-    while ((int64_t(1) << s) < d) ++s;
-    f.m = (unsigned)((uint64_t(1) << (31 + s)) / (unsigned)d + 1);
-    f.s = (unsigned)(s - 1);
-    return f;
-}
-
 void team_geometry(BChainDev* d, const Lat& lat) {
     d->L = lat.L;
     d->Nt = lat.Nt;
@@ -803,26 +735,6 @@ void team_geometry(BChainDev* d, const Lat& lat) {
     d->V = lat.V;
     d->dL = fast_div(lat.L);
     d->dLL = fast_div(lat.L * lat.L);
-}
-
-// N = n1 n2 with both factors among dft_step's radices, their sum (the work per point) least; up to 10
-// points in one step: a step costs its latency, not its work, at the sizes that take few points
-static bool split(int n, int* n1, int* n2) {
-    static const int radix[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};
-    if (n <= 10) {
-        *n1 = n;
-        *n2 = 1;
-        return true;
-    }
-    int best = 1 << 30;
-    for (int a : radix)
-        for (int b : radix)
-            if (a * b == n && a >= b && a + b < best) {
-                best = a + b;
-                *n1 = a;
-                *n2 = b;
-            }
-    return best < (1 << 30);
 }
 
 template <typename R> static const cplx<R>* plan_tw(const FftPlan* p);
@@ -833,7 +745,7 @@ template <> const double2* plan_tw<double>(const FftPlan* p) { return p->tw64; }
 template <typename R> static bool pre_setup(hmc_ctx* ctx, const Lat& lat, TeamPre<R>* q) {
     const FftPlan *px = get_plan(ctx, lat.L), *ptau = get_plan(ctx, lat.Nt);
     const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
-    if (!px || !ptau || !pc || !split(lat.L, &q->x1, &q->x2) || !split(lat.Nt, &q->t1, &q->t2)) return false;
+    if (!px || !ptau || !pc || !dft_split(lat.L, &q->x1, &q->x2) || !dft_split(lat.Nt, &q->t1, &q->t2)) return false;
     q->twx = plan_tw<R>(px);
     q->twt = plan_tw<R>(ptau);
     if constexpr (sizeof(R) == 4) {
