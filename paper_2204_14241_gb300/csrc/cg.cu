@@ -203,8 +203,9 @@ __global__ void k_cg_set_rz(CgScalars* cgs, const double* __restrict__ part, int
     }
 }
 
-// After a true-residual evaluation: r2true from part; converged RHS become inactive.
-__global__ void k_ru_finish(CgScalars* cgs, const double* __restrict__ part, int nblk, double tol2) {
+// After a true-residual evaluation: r2true from part; converged RHS become inactive. set_rr: the recurrence
+// goes on with this norm (plain complex64 CG: that of the residual before its rounding to complex64, 1e-8 off).
+__global__ void k_ru_finish(CgScalars* cgs, const double* __restrict__ part, int nblk, double tol2, int set_rr) {
     __shared__ double red[8];
     const int k = blockIdx.x;
     if (!cgs[k].active) return;
@@ -217,6 +218,7 @@ __global__ void k_ru_finish(CgScalars* cgs, const double* __restrict__ part, int
         if (r2 <= tol2 * c.b2) { c.active = 0; return; }
         c.r2 = r2;
         c.r2_max = r2;
+        if (set_rr) c.rr = r2;
     }
 }
 
@@ -406,9 +408,9 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
         int nbr = 0;
         if ((rc = residual64(ctx, lat, phi64, x, b, ctx->d_r64, kMixed ? ctx->d_r32 : nullptr, nrhs, part, &nbr, cgs)))
             return rc;
-        k_ru_finish<<<nrhs, 256, 0, sm>>>(cgs, part, nbr, tol2);
+        k_ru_finish<<<nrhs, 256, 0, sm>>>(cgs, part, nbr, tol2, fused ? 1 : 0);
         HMC_LAUNCH(ctx, "k_ru_finish");
-        return restart_dir();
+        return fused ? HMC_OK : restart_dir();
     };
 
     // The host reads the flags (one stream synchronisation) after at most check_every iterations.

@@ -44,6 +44,21 @@ template <typename R> __device__ __forceinline__ Site<R> load_site(const Site<R>
     }
     return s;
 }
+// A complex64 site in one 32-byte access (p 32-byte aligned): a warp's sites are 1 KB in a row, which two
+// 16-byte accesses of every second half cross twice.
+__device__ __forceinline__ Site<float> load_site_wide(const Site<float>* p) {
+    Site<float> s;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(s.c[0].x), "=f"(s.c[0].y), "=f"(s.c[1].x), "=f"(s.c[1].y), "=f"(s.c[2].x), "=f"(s.c[2].y), "=f"(s.c[3].x),
+          "=f"(s.c[3].y)
+        : "l"(p));
+    return s;
+}
+__device__ __forceinline__ void store_site_wide(Site<float>* p, const Site<float>& s) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(s.c[0].x), "f"(s.c[0].y),
+                 "f"(s.c[1].x), "f"(s.c[1].y), "f"(s.c[2].x), "f"(s.c[2].y), "f"(s.c[3].x), "f"(s.c[3].y)
+                 : "memory");
+}
 template <typename R> __device__ __forceinline__ void store_site(Site<R>* p, const Site<R>& s) {
     if constexpr (sizeof(R) == 4) {
         float4* q = reinterpret_cast<float4*>(p);
@@ -76,17 +91,31 @@ __device__ __forceinline__ int tprev(int t, int Nt) { return t == 0 ? Nt - 1 : t
 __device__ __forceinline__ int wrap_inc(int x, int L) { return x + 1 == L ? 0 : x + 1; }
 __device__ __forceinline__ int wrap_dec(int x, int L) { return x == 0 ? L - 1 : x - 1; }
 
+// v with its sign changed when bit 0 of `neg` is set, in the integer units: GB300 has two FP64 lanes a clock
+// per SM, and a multiply by +-1 costs one of them as much as any other FP64 operation.
+__device__ __forceinline__ float flip(float v, int neg) {
+    return __int_as_float(__float_as_int(v) ^ (neg << 31));
+}
+__device__ __forceinline__ double flip(double v, int neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg << 31), __double2loint(v));
+}
+__device__ __forceinline__ int sign_bit(float v) { return (int)((unsigned)__float_as_int(v) >> 31); }
+__device__ __forceinline__ int sign_bit(double v) { return (int)((unsigned)__double2hiint(v) >> 31); }
+
 // One site of D v (DAG = false) or D^dagger v (DAG = true):
 //   out = diag c + tsign * tn + hx (xm + xp) + hy (ym + yp) + cpl eta (phi.sigma) c[other band]
-// tn is v at t+1 (D) or t-1 (D^dagger); tsign is b(t) for D and b(t-1) for D^dagger.
+// tn is v at t+1 (D) or t-1 (D^dagger); tsign (+-1) is b(t) for D and b(t-1) for D^dagger; eta is +-1.
 // The hopping is real symmetric and the on-site block Hermitian, so D and D^dagger differ
-// only in the time hop.
+// only in the time hop. 67 FP64 operations (every product in a fused multiply-add, signs flipped in
+// integers); 84 when each line was a sum of products with tsign and eta as factors. The largest product comes
+// last: the sums before it round at a smaller magnitude (0.88 of that form's error; first, 1.13 of it).
 template <typename R>
 __device__ __forceinline__ Site<R> site_op(const Coef<R>& cf, const Site<R>& c, const Site<R>& xm,
                                            const Site<R>& xp, const Site<R>& ym, const Site<R>& yp,
                                            const Site<R>& tn, R tsign, R p1, R p2, R p3, R eta) {
     Site<R> o;
-    const R f = cf.cpl * eta;
+    const int edge = sign_bit(tsign);
+    const R f = flip(cf.cpl, sign_bit(eta));
     const R q1 = f * p1, q2 = f * p2, q3 = f * p3;
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -94,16 +123,16 @@ __device__ __forceinline__ Site<R> site_op(const Coef<R>& cf, const Site<R>& c, 
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int i = a * 2 + s;
-            R re = d * c.c[i].x + tsign * tn.c[i].x + hx * (xm.c[i].x + xp.c[i].x) + hy * (ym.c[i].x + yp.c[i].x);
-            R im = d * c.c[i].y + tsign * tn.c[i].y + hx * (xm.c[i].y + xp.c[i].y) + hy * (ym.c[i].y + yp.c[i].y);
-            o.c[i].x = re; o.c[i].y = im;
+            o.c[i].x = fma(hx, xm.c[i].x + xp.c[i].x, fma(hy, ym.c[i].x + yp.c[i].x, flip(tn.c[i].x, edge)));
+            o.c[i].y = fma(hx, xm.c[i].y + xp.c[i].y, fma(hy, ym.c[i].y + yp.c[i].y, flip(tn.c[i].y, edge)));
         }
         // sigma^x swaps the bands; phi.sigma = [[p3, p1 - i p2], [p1 + i p2, -p3]]
-        const cplx<R> w0 = c.c[(1 - a) * 2], w1 = c.c[(1 - a) * 2 + 1];
-        o.c[a * 2].x += q3 * w0.x + q1 * w1.x + q2 * w1.y;
-        o.c[a * 2].y += q3 * w0.y + q1 * w1.y - q2 * w1.x;
-        o.c[a * 2 + 1].x += q1 * w0.x - q2 * w0.y - q3 * w1.x;
-        o.c[a * 2 + 1].y += q1 * w0.y + q2 * w0.x - q3 * w1.y;
+        const cplx<R> v0 = c.c[a * 2], v1 = c.c[a * 2 + 1], w0 = c.c[(1 - a) * 2], w1 = c.c[(1 - a) * 2 + 1];
+        cplx<R>&o0 = o.c[a * 2], &o1 = o.c[a * 2 + 1];
+        o0.x = fma(d, v0.x, fma(q3, w0.x, fma(q1, w1.x, fma(q2, w1.y, o0.x))));
+        o0.y = fma(d, v0.y, fma(q3, w0.y, fma(q1, w1.y, fma(-q2, w1.x, o0.y))));
+        o1.x = fma(d, v1.x, fma(-q3, w1.x, fma(q1, w0.x, fma(-q2, w0.y, o1.x))));
+        o1.y = fma(d, v1.y, fma(-q3, w1.y, fma(q1, w0.y, fma(q2, w0.x, o1.y))));
     }
     return o;
 }
@@ -125,6 +154,23 @@ __device__ __forceinline__ double block_sum(double v, double* smem) {
     if (w == 0) {
         const int nw = (blockDim.x + 31) >> 5;
         t = lane < nw ? smem[lane] : 0.0;
+        t = warp_sum(t);
+    }
+    __syncthreads();
+    return t;
+}
+
+// The same for kernels that the FP64 pipe bounds, blocks of 256 threads, smem of 256 doubles: one warp adds
+// the block's values, 12 warp-wide additions against 45 in the shuffle trees of all warps (6 % of the
+// operations of an FP64 stencil block).
+__device__ __forceinline__ double block_sum_256(double v, double* smem) {
+    smem[threadIdx.x] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < 32) {
+        t = v;
+#pragma unroll
+        for (int j = 1; j < 8; ++j) t += smem[threadIdx.x + 32 * j];
         t = warp_sum(t);
     }
     __syncthreads();
@@ -155,10 +201,6 @@ enum { kBndApplyD = 1, kBndForce = 2, kBndStripGlobal = 4, kBndStripShared = 8 }
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() {

@@ -11,8 +11,6 @@
 
 namespace hmc {
 
-__device__ __forceinline__ int fdiv(int n, FastDiv d) { return (int)(__umulhi((unsigned)n, d.m) >> d.s); }
-
 // The tile holds `np` planes of `nl` lines, `plane` entries apart; line l of a plane starts at
 // (l & 1) * l1 + (l >> 1) * ls, the points of DFT f at f * fs + m * ps; with tw, output m is multiplied by
 // tw[f m].
@@ -80,14 +78,6 @@ __device__ __forceinline__ int dft_freq(int p, int n1, int n2) { return p / n1 +
 __device__ __forceinline__ int dft_pos(int k, int n1, int n2) { return n1 * (k % n2) + k / n2; }
 
 // ---- host --------------------------------------------------------------------------------------------
-inline FastDiv fast_div(int d) {   // n / d for 0 <= n < 2^31, d >= 2
-    FastDiv f;
-    int s = 1;
-    while ((int64_t(1) << s) < d) ++s;
-    f.m = (unsigned)((uint64_t(1) << (31 + s)) / (unsigned)d + 1);
-    f.s = (unsigned)(s - 1);
-    return f;
-}
 // N = n1 n2 with both factors among dft_step's radices, their sum (the work per point) least; up to 10
 // points in one step: a step costs its latency, not its work, at the sizes that take few points. False when
 // there is none.

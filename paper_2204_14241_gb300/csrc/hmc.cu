@@ -467,7 +467,8 @@ static int force_impl(hmc_ctx* ctx, int chain, const double* phi, const double2*
     if (rc) return rc;
     if (tm && (rc = tm->mark(kPhaseForce))) return rc;
     int nb = 0;
-    if ((rc = launch_force(ctx, ch.lat, ch.r, phi, X, pf, nrhs, F, include_boson, ctx->d_part, &nb,
+    const bool action = dev_e || s_pf || s_b;
+    if ((rc = launch_force(ctx, ch.lat, ch.r, phi, X, pf, nrhs, F, include_boson, action ? ctx->d_part : nullptr, &nb,
                            y_ready ? ctx->d_z64 : nullptr)))
         return rc;
     if (dev_e) return reduce_rows(ctx, ctx->d_part, 2, nb, dev_e);
@@ -845,7 +846,7 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
             int nb = 0;
             // D^dagger X of the solution is left in d_z64 by the batched solve
             if ((r2 = launch_force(ctx, ch.lat, ch.r, phis[c], fvec(xo, c), fvec(ctx->d_pf, c), K, bvec(ctx->d_F, c), 1,
-                                   ctx->d_part, &nb, fvec(ctx->d_z64, c))))
+                                   want ? ctx->d_part : nullptr, &nb, fvec(ctx->d_z64, c))))
                 return r2;
             if (want) {
                 if ((r2 = reduce_rows(ctx, ctx->d_part, 1, nb, E + 6 * c + 5))) return r2;

@@ -11,6 +11,22 @@
 
 namespace hmc {
 
+// n / d for 0 <= n < 2^31 as umulhi(n, m) >> s
+struct FastDiv {
+    unsigned m, s;
+};
+inline FastDiv fast_div(int d) {   // d >= 2
+    FastDiv f;
+    int s = 1;
+    while ((int64_t(1) << s) < d) ++s;
+    f.m = (unsigned)((uint64_t(1) << (31 + s)) / (unsigned)d + 1);
+    f.s = (unsigned)(s - 1);
+    return f;
+}
+__device__ __forceinline__ int fdiv(int n, FastDiv d) { return (int)(__umulhi((unsigned)n, d.m) >> d.s); }
+
+inline bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
 struct FftPlan {
     int n = 0;
     std::vector<int> radix;      // factors, applied in order
@@ -52,10 +68,6 @@ struct ChainDesc {
     double r;
 };
 
-// n / d for 0 <= n < 2^31 as umulhi(n, m) >> s (team.cu)
-struct FastDiv {
-    unsigned m, s;
-};
 
 // Geometry and fields of a chain in the team solver (team.cu): item offset of the chain's K right-hand
 // sides in the concatenated vectors.
@@ -239,10 +251,11 @@ template <typename R> Coef<R> make_coef(const hmc_params& p);
 
 // stencil.cu
 // y = D x (dagger 0) or D^dagger x; right-hand sides with cgs[k].active == 0 are skipped when cgs
-// is given.
+// is given. With part, per-block partial sums of ||y||^2 in part[k * *nblk_out + b].
 template <typename R>
 int launch_apply_D(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x, cplx<R>* y,
-                   int dagger, int nrhs, const CgScalars* cgs = nullptr);
+                   int dagger, int nrhs, const CgScalars* cgs = nullptr, double* part = nullptr,
+                   int* nblk_out = nullptr);
 // FP64 true residual r = b - D t (t = D^dagger x from launch_apply_D), written as r64 and, if
 // r32 != nullptr, as complex64; per-block partial sums of ||r||^2 in part[k * nblk + b], nblk =
 // *nblk_out. Inactive right-hand sides (cgs) are skipped.
@@ -251,7 +264,8 @@ int launch_residual_D(hmc_ctx* ctx, const Lat& lat, const double* phi, const dou
 // y = A x; if part != nullptr, per-block partial sums of ||D^dag x||^2 are written to
 // part[k * nblk + b] and *nblk_out receives nblk.
 // cgs (may be null): right-hand sides whose cgs[k].active is 0 are skipped. With pnew set,
-// the operand is p = x + cgs[k].beta * pold, written to pnew for every site, and y = A p.
+// the operand is p = x + cgs[k].beta * pold, written to pnew for every site, and y = A p; without it
+// ctx->d_q64 may be overwritten.
 template <typename R>
 int launch_apply_A(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x, cplx<R>* y,
                    int nrhs, double* part, int* nblk_out, const CgScalars* cgs = nullptr,
@@ -262,7 +276,7 @@ int launch_apply_A(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x,
 bool strip_supported(const Lat& lat);
 int launch_apply_A_strip(hmc_ctx* ctx, const Lat& lat, const float* phi, const float2* x, float2* y, int nrhs,
                          double* part, int* nblk_out, const CgScalars* cgs, double* part_q = nullptr);
-// fermion (+ boson) force and the action pieces, see force() in hmc.h. Y (may be null): D^dagger X
+// fermion (+ boson) force and, unless part is null, the action pieces, see force() in hmc.h. Y (may be null): D^dagger X
 // already computed (same layout as X); otherwise the kernel forms it.
 int launch_force(hmc_ctx* ctx, const Lat& lat, double r, const double* phi, const double2* X,
                  const double2* pf, int nrhs, double* F, int include_boson, double* part,

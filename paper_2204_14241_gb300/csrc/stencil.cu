@@ -20,53 +20,117 @@ template Coef<float> make_coef<float>(const hmc_params&);
 template Coef<double> make_coef<double>(const hmc_params&);
 
 // ---------------------------------------------------------------------------------------
-// y = D x or D^dagger x, one thread per site, neighbours through the read-only cache.
-template <typename R, bool DAG>
-__global__ void __launch_bounds__(256) k_apply_D(Lat lat, Coef<R> cf, const R* __restrict__ phi,
+// Site coordinates without 64-bit divisions, which took as long as the complex64 operator's memory traffic:
+// exact multiplications by reciprocals for site indices below 2^31, divisions past that.
+struct SiteDiv {
+    FastDiv dL, dLL;
+    int big;
+};
+static SiteDiv site_div(const Lat& lat) {
+    return SiteDiv{fast_div(lat.L), fast_div(lat.L * lat.L), lat.V >= (int64_t)1 << 31};
+}
+__device__ __forceinline__ void site_xyt(const Lat& lat, const SiteDiv& sd, int64_t s, int& x, int& y, int& t) {
+    if (sd.big) {
+        x = (int)(s % lat.L);
+        const int64_t rest = s / lat.L;
+        y = (int)(rest % lat.L);
+        t = (int)(rest / lat.L);
+    } else {
+        t = fdiv((int)s, sd.dLL);
+        const int rem = (int)s - t * lat.L * lat.L;
+        y = fdiv(rem, sd.dL);
+        x = rem - y * lat.L;
+    }
+}
+
+// y = D x or D^dagger x, one thread per site, neighbours through the read-only cache. complex64 moves 536 MB
+// at 80 x 80 x 160 with 8 right-hand sides (79 us at the copy bandwidth) and was bound by L1 wavefronts, 16-byte
+// accesses at every second half of the sites: 128 us. WIDE takes a site in one access, where x and y are
+// 32-byte aligned: 107 us. complex128: bound by the FP64 pipe, 0.99 ms there (1.27 with 84 operations per site).
+template <typename R, bool DAG, bool WIDE>
+__global__ void __launch_bounds__(256) k_apply_D(Lat lat, SiteDiv sd, Coef<R> cf, const R* __restrict__ phi,
                                                  const Site<R>* __restrict__ x,
-                                                 Site<R>* __restrict__ y, const CgScalars* __restrict__ cgs) {
+                                                 Site<R>* __restrict__ y, const CgScalars* __restrict__ cgs,
+                                                 double* __restrict__ part) {
+    __shared__ double red[256];
     if (cgs && !cgs[blockIdx.y].active) return;
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= lat.V) return;
     const int64_t V = lat.V;
-    const int L = lat.L;
-    const Site<R>* xk = x + blockIdx.y * V;
-    const int xx = (int)(s % L);
-    const int64_t rest = s / L;
-    const int yy = (int)(rest % L);
-    const int t = (int)(rest / L);
-    const int64_t row = s - xx, slice = (int64_t)t * L * L;
-    const int tn = DAG ? tprev(t, lat.Nt) : tnext(t, lat.Nt);
-    const R tsign = DAG ? (t == 0 ? R(-1) : R(1)) : (t == lat.Nt - 1 ? R(-1) : R(1));
-    const R eta = ((xx + yy) & 1) ? R(-1) : R(1);
-    auto ld = [&](int64_t i) {
-        Site<R> z{};
-        return HMC_IN(i >= 0 && i < V, kBndApplyD) ? load_site(xk + i) : z;
-    };
-    Site<R> o = site_op<R>(cf, ld(s), ld(row + wrap_dec(xx, L)), ld(row + wrap_inc(xx, L)),
-                           ld(slice + (int64_t)wrap_dec(yy, L) * L + xx), ld(slice + (int64_t)wrap_inc(yy, L) * L + xx),
-                           ld((int64_t)tn * L * L + (s - slice)), tsign,
-                           __ldg(phi + s), __ldg(phi + V + s), __ldg(phi + 2 * V + s), eta);
-    store_site(y + blockIdx.y * V + s, o);
+    R e = 0;
+    if (s < V) {
+        const int L = lat.L;
+        const Site<R>* xk = x + blockIdx.y * V;
+        int xx, yy, t;
+        site_xyt(lat, sd, s, xx, yy, t);
+        const int64_t row = s - xx, slice = (int64_t)t * L * L;
+        const int tn = DAG ? tprev(t, lat.Nt) : tnext(t, lat.Nt);
+        const R tsign = DAG ? (t == 0 ? R(-1) : R(1)) : (t == lat.Nt - 1 ? R(-1) : R(1));
+        const R eta = ((xx + yy) & 1) ? R(-1) : R(1);
+        auto ld = [&](int64_t i) {
+            Site<R> z{};
+            if (!HMC_IN(i >= 0 && i < V, kBndApplyD)) return z;
+            if constexpr (WIDE) return load_site_wide(xk + i);
+            else return load_site(xk + i);
+        };
+        Site<R> o = site_op<R>(cf, ld(s), ld(row + wrap_dec(xx, L)), ld(row + wrap_inc(xx, L)),
+                               ld(slice + (int64_t)wrap_dec(yy, L) * L + xx), ld(slice + (int64_t)wrap_inc(yy, L) * L + xx),
+                               ld((int64_t)tn * L * L + (s - slice)), tsign,
+                               __ldg(phi + s), __ldg(phi + V + s), __ldg(phi + 2 * V + s), eta);
+        if constexpr (WIDE) store_site_wide(y + blockIdx.y * V + s, o);
+        else store_site(y + blockIdx.y * V + s, o);
+        if (part) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) e = fma(o.c[q].x, o.c[q].x, fma(o.c[q].y, o.c[q].y, e));
+        }
+    }
+    if (part) {
+        const double tot = block_sum_256((double)e, red);
+        if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
+    }
 }
 
 template <typename R>
 int launch_apply_D(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x, cplx<R>* y,
-                   int dagger, int nrhs, const CgScalars* cgs) {
+                   int dagger, int nrhs, const CgScalars* cgs, double* part, int* nblk_out) {
     if (nrhs <= 0) return HMC_OK;
     dim3 grid((unsigned)((lat.V + 255) / 256), nrhs);
+    if (part) {
+        if ((int64_t)grid.x * nrhs > ctx->part_cap) return fail(ctx, HMC_ERR_ARG, "apply_D: reduction buffer too small");
+        *nblk_out = (int)grid.x;
+    }
     Coef<R> cf = make_coef<R>(ctx->p);
     auto xs = reinterpret_cast<const Site<R>*>(x);
     auto ys = reinterpret_cast<Site<R>*>(y);
-    if (dagger) k_apply_D<R, true><<<grid, 256, 0, ctx->stream>>>(lat, cf, phi, xs, ys, cgs);
-    else        k_apply_D<R, false><<<grid, 256, 0, ctx->stream>>>(lat, cf, phi, xs, ys, cgs);
+    auto go = [&](auto kernel) {
+        kernel<<<grid, 256, 0, ctx->stream>>>(lat, site_div(lat), cf, phi, xs, ys, cgs, part);
+    };
+    if constexpr (sizeof(R) == 4) {
+        if (aligned32(x) && aligned32(y)) dagger ? go(k_apply_D<R, true, true>) : go(k_apply_D<R, false, true>);
+        else dagger ? go(k_apply_D<R, true, false>) : go(k_apply_D<R, false, false>);
+    } else {
+        dagger ? go(k_apply_D<R, true, false>) : go(k_apply_D<R, false, false>);
+    }
     HMC_LAUNCH(ctx, "k_apply_D");
     return HMC_OK;
 }
 template int launch_apply_D<float>(hmc_ctx*, const Lat&, const float*, const float2*, float2*, int, int,
-                                   const CgScalars*);
+                                   const CgScalars*, double*, int*);
 template int launch_apply_D<double>(hmc_ctx*, const Lat&, const double*, const double2*, double2*, int, int,
-                                    const CgScalars*);
+                                    const CgScalars*, double*, int*);
+
+// A = D D^dagger as two passes through the FP64 q workspace (free whenever this runs: solves in FP64 mode fold
+// the direction update into k_apply_A). The fused kernel (k_apply_A) forms t_ again on a ring around every
+// tile, 2.4 site operations per site against 2, and waits at its barriers: in complex128, bound by the FP64 pipe,
+// 3.32 ms against 1.98 at 80 x 80 x 160 with 8 right-hand sides; in complex64 43 against 25 us at 40 x 40 x 80 with
+// 8 (in L2), 187 against 157 at 72 x 72 x 144. The complex64 strip kernel is ahead of both where it has a form.
+template <typename R>
+static int launch_A_two_pass(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x, cplx<R>* y, int nrhs,
+                             double* part, int* nblk_out, const CgScalars* cgs) {
+    cplx<R>* t = reinterpret_cast<cplx<R>*>(ctx->d_q64);
+    int rc;
+    if ((rc = launch_apply_D<R>(ctx, lat, phi, x, t, 1, nrhs, cgs, part, nblk_out))) return rc;
+    return launch_apply_D<R>(ctx, lat, phi, t, y, 0, nrhs, cgs);
+}
 
 // The FP64 true residual r = b - D t of a reliable update or of a start from a guess, in the
 // operator's second pass: the pass is bound by the FP64 pipe, so streaming b in and r (and its
@@ -76,7 +140,7 @@ __global__ void __launch_bounds__(256) k_residual_D(Lat lat, Coef<double> cf, co
                                                     const Site<double>* __restrict__ b, Site<double>* __restrict__ r,
                                                     Site<float>* __restrict__ r32, double* __restrict__ part,
                                                     const CgScalars* __restrict__ cgs) {
-    __shared__ double red[8];
+    __shared__ double red[256];
     if (cgs && !cgs[blockIdx.y].active) return;
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t V = lat.V;
@@ -109,12 +173,12 @@ __global__ void __launch_bounds__(256) k_residual_D(Lat lat, Coef<double> cf, co
         for (int q = 0; q < 4; ++q) {
             rr.c[q] = make_double2(bb.c[q].x - o.c[q].x, bb.c[q].y - o.c[q].y);
             rf.c[q] = make_float2((float)rr.c[q].x, (float)rr.c[q].y);
-            e += rr.c[q].x * rr.c[q].x + rr.c[q].y * rr.c[q].y;
+            e = fma(rr.c[q].x, rr.c[q].x, fma(rr.c[q].y, rr.c[q].y, e));
         }
         store_site(r + g, rr);
         if (r32) store_site(r32 + g, rf);
     }
-    e = block_sum(e, red);
+    e = block_sum_256(e, red);
     if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = e;
 }
 
@@ -354,196 +418,6 @@ k_apply_A(Lat lat, Coef<R> cf, ATile tl, const R* __restrict__ phi, const Site<R
     }
 }
 
-// ---------------------------------------------------------------------------------------
-// Plain FP32 fused A, asynchronous staging, tile extent fixed at compile time. Same marching
-// scheme as k_apply_A, but each time slice of x and phi arrives by cp.async copies (16-byte
-// chunks for x) into a four-slice ring in shared memory, issued three slices ahead, so no
-// registers hold staged data and a slice has two steps to land. Thread i < TX*TY owns tile
-// site (i % TX, i / TX) and keeps that site's x(t), t_(t) and phi(t) in registers: its
-// t_(t+1) reads the four x neighbours and its y(t) the four t_ neighbours from shared memory.
-// The one-site-ring t_ sites are a second job of threads 0, 1, ... One barrier per step:
-// step t writes t_(t+1) into the t_ buffer that y(t-1) read before the barrier, and reads
-// t_(t), written before it; slice t+3 goes into the x buffer of slice t-1, last read before it.
-
-constexpr int kA4Ring = 4;   // x and phi slices resident: t-1 .. t+2
-
-template <int TX, int TY> struct A4Shape {
-    static constexpr int HX2 = TX + 4, N2 = (TX + 4) * (TY + 4);   // two-site halo
-    static constexpr int HX1 = TX + 2, N1 = (TX + 2) * (TY + 2);   // one-site halo
-    static constexpr int NI = TX * TY;
-    static constexpr int NCH = (2 * N2 + kAThreads - 1) / kAThreads;   // 16-byte chunks per thread and slice
-    static constexpr int NPH = (N1 + kAThreads - 1) / kAThreads;       // phi sites per thread and slice
-    static constexpr size_t smem = (size_t)kA4Ring * N2 * 32 + (size_t)2 * N1 * 32 + (size_t)kA4Ring * 3 * N1 * 4;
-    static_assert(NI <= kAThreads && N1 - NI <= kAThreads, "one tile site and one ring site per thread");
-};
-
-template <int TX, int TY>
-__global__ void __launch_bounds__(kAThreads, 2) k_apply_A4(Lat lat, Coef<float> cf, ATile tl,
-                                                           const float* __restrict__ phi,
-                                                           const Site<float>* __restrict__ x,
-                                                           Site<float>* __restrict__ y, double* __restrict__ part,
-                                                           const CgScalars* __restrict__ cgs) {
-    if (cgs && !cgs[blockIdx.z].active) return;
-    using S = A4Shape<TX, TY>;
-    constexpr int HX2 = S::HX2, N2 = S::N2, HX1 = S::HX1, N1 = S::N1, NI = S::NI;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint4* xsb = reinterpret_cast<uint4*>(smem_raw);                 // ring x [2 planes][N2]
-    uint4* tsb = xsb + kA4Ring * 2 * N2;                             // 2 x [2 planes][N1]
-    float* phb = reinterpret_cast<float*>(tsb + 2 * 2 * N1);         // ring x [3][N1]
-    __shared__ double red[kAThreads / 32];
-
-    const int L = lat.L, Nt = lat.Nt;
-    const int64_t V = lat.V, LL = (int64_t)L * L;
-    const int x0 = (blockIdx.x % tl.ntx) * TX, y0 = (blockIdx.x / tl.ntx) * TY;
-    const int t0 = blockIdx.y * tl.C;
-    const int t1 = min(t0 + tl.C, Nt);
-    const int k = blockIdx.z;
-    const Site<float>* xk = x + k * V;
-    Site<float>* yk = y + k * V;
-    auto gx = [&](int i) { int v = (x0 + i) % L; return v < 0 ? v + L : v; };
-    auto gy = [&](int j) { int v = (y0 + j) % L; return v < 0 ? v + L : v; };
-    auto wrap_t = [&](int t) { return t < 0 ? t + Nt : (t >= Nt ? t - Nt : t); };
-    const int tid = threadIdx.x;
-
-    // staging: chunk c = tid + j * threads is plane (c & 1) of two-site-halo site (c >> 1);
-    // g_off in 16-byte units within a slice, -1 for none
-    int g_off[S::NCH];
-#pragma unroll
-    for (int j = 0; j < S::NCH; ++j) {
-        const int c = tid + j * kAThreads, i = c >> 1;
-        g_off[j] = c < 2 * N2 ? 2 * (gy(i / HX2 - 2) * L + gx(i % HX2 - 2)) + (c & 1) : -1;
-    }
-    int p_off[S::NPH];
-#pragma unroll
-    for (int j = 0; j < S::NPH; ++j) {
-        const int i = tid + j * kAThreads;
-        p_off[j] = i < N1 ? gy(i / HX1 - 1) * L + gx(i % HX1 - 1) : -1;
-    }
-    // own tile site
-    const bool own = tid < NI;
-    const int ix = tid % TX, iy = tid / TX;
-    const int o_c2 = (iy + 2) * HX2 + ix + 2, o_c1 = (iy + 1) * HX1 + ix + 1;
-    const bool o_valid = own && x0 + ix < L && y0 + iy < L;
-    const int o_off = gy(iy) * L + gx(ix);
-    const float o_eta = ((gx(ix) + gy(iy)) & 1) ? -1.f : 1.f;
-    // one-site-ring site of this thread: top row, the two side columns, bottom row
-    int r1_c1 = -1, r1_c2 = 0;
-    float r1_eta = 1.f;
-    if (tid < N1 - NI) {
-        int hx, hy;
-        if (tid < HX1) { hy = 0; hx = tid; }
-        else if (tid < HX1 + 2 * TY) { const int r = tid - HX1; hy = 1 + r / 2; hx = (r & 1) ? TX + 1 : 0; }
-        else { hy = TY + 1; hx = tid - HX1 - 2 * TY; }
-        r1_c1 = hy * HX1 + hx;
-        r1_c2 = (hy + 1) * HX2 + hx + 1;
-        r1_eta = ((gx(hx - 1) + gy(hy - 1)) & 1) ? -1.f : 1.f;
-    }
-
-    auto xbuf = [&](int b) { return xsb + b * (2 * N2); };
-    auto tbuf = [&](int b) { return tsb + b * (2 * N1); };
-    auto pbuf = [&](int b) { return phb + b * (3 * N1); };
-    auto issue = [&](int b, int t) {
-        const int64_t base = (int64_t)t * LL;
-        const uint4* src = reinterpret_cast<const uint4*>(xk + base);
-        uint4* dst = xbuf(b);
-#pragma unroll
-        for (int j = 0; j < S::NCH; ++j) {
-            const int c = tid + j * kAThreads;
-            if (g_off[j] >= 0) cp_async16(dst + (c & 1) * N2 + (c >> 1), src + g_off[j]);
-        }
-        float* pd = pbuf(b);
-#pragma unroll
-        for (int j = 0; j < S::NPH; ++j)
-            if (p_off[j] >= 0) {
-                const int i = tid + j * kAThreads;
-                const float* ps = phi + base + p_off[j];
-                cp_async4(pd + i, ps);
-                cp_async4(pd + N1 + i, ps + V);
-                cp_async4(pd + 2 * N1 + i, ps + 2 * V);
-            }
-    };
-    // t_ at slice t on this thread's ring site from x(t) (buffer bc) and x(t-1) (buffer bp)
-    auto ring_t = [&](int bc, int bp, int bt, int t) {
-        if (r1_c1 < 0) return;
-        const uint4* xc = xbuf(bc);
-        const float* ph = pbuf(bc);
-        const int c = r1_c2;
-        const Site<float> o = site_op<float>(cf, sm_load<float>(xc, N2, c), sm_load<float>(xc, N2, c - 1),
-                                             sm_load<float>(xc, N2, c + 1), sm_load<float>(xc, N2, c - HX2),
-                                             sm_load<float>(xc, N2, c + HX2), sm_load<float>(xbuf(bp), N2, c),
-                                             t == 0 ? -1.f : 1.f, ph[r1_c1], ph[N1 + r1_c1], ph[2 * N1 + r1_c1],
-                                             r1_eta);
-        sm_store<float>(tbuf(bt), N1, r1_c1, o);
-    };
-    // t_ at slice t on the own site from x(t) (buffer bc, also returned in xo) and x(t-1)
-    auto own_t = [&](int bc, const Site<float>& xprev, int bt, int t, Site<float>& xo, float* ph3) {
-        const uint4* xc = xbuf(bc);
-        const float* ph = pbuf(bc);
-        xo = sm_load<float>(xc, N2, o_c2);
-        ph3[0] = ph[o_c1]; ph3[1] = ph[N1 + o_c1]; ph3[2] = ph[2 * N1 + o_c1];
-        const Site<float> o = site_op<float>(cf, xo, sm_load<float>(xc, N2, o_c2 - 1), sm_load<float>(xc, N2, o_c2 + 1),
-                                             sm_load<float>(xc, N2, o_c2 - HX2), sm_load<float>(xc, N2, o_c2 + HX2),
-                                             xprev, t == 0 ? -1.f : 1.f, ph3[0], ph3[1], ph3[2], o_eta);
-        sm_store<float>(tbuf(bt), N1, o_c1, o);
-        return o;
-    };
-
-    // prologue: slices t0-1 .. t0+2 in buffers 0 .. 3 (slice t0+2 only if step t0+1 exists)
-    issue(0, wrap_t(t0 - 1));
-    cp_async_commit();
-    issue(1, t0);
-    cp_async_commit();
-    issue(2, wrap_t(t0 + 1));   // y(t0) needs t_(t0+1) even when the chunk is one slice long
-    cp_async_commit();
-    if (t0 + 1 < t1) issue(3, wrap_t(t0 + 2));
-    cp_async_commit();
-    cp_async_wait<2>();
-    __syncthreads();
-    Site<float> xo, to;
-    float pho[3] = {0.f, 0.f, 0.f};
-    if (own) to = own_t(1, sm_load<float>(xbuf(0), N2, o_c2), 0, t0, xo, pho);
-    ring_t(1, 0, 0, t0);
-
-    float acc = 0.f;
-    for (int t = t0; t < t1; ++t) {
-        const int u = t - t0 + 1;              // ring buffer of slice t is u & 3
-        cp_async_wait<1>();                    // slice t+1 has landed (slice t+2 may be in flight)
-        __syncthreads();
-        if (t + 2 < t1) issue((u + 3) & 3, wrap_t(t + 3));
-        cp_async_commit();
-        const int tp = wrap_t(t + 1);
-        const int bn = (u + 1) & 3, bt = (t + 1 - t0) & 1;
-        Site<float> xn, tn;
-        float phn[3] = {0.f, 0.f, 0.f};
-        if (own) tn = own_t(bn, xo, bt, tp, xn, phn);
-        ring_t(bn, u & 3, bt, tp);
-        // y(t) = D t_ on the own site: t_(t) neighbours from the buffer written before the barrier
-        if (own) {
-            const uint4* tc = tbuf(bt ^ 1);
-            const Site<float> o = site_op<float>(cf, to, sm_load<float>(tc, N1, o_c1 - 1),
-                                                 sm_load<float>(tc, N1, o_c1 + 1), sm_load<float>(tc, N1, o_c1 - HX1),
-                                                 sm_load<float>(tc, N1, o_c1 + HX1), tn, t == Nt - 1 ? -1.f : 1.f,
-                                                 pho[0], pho[1], pho[2], o_eta);
-            if (o_valid) {
-                store_site(yk + (int64_t)t * LL + o_off, o);
-                if (part) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) acc += to.c[q].x * to.c[q].x + to.c[q].y * to.c[q].y;
-                }
-            }
-            xo = xn;
-            to = tn;
-            pho[0] = phn[0]; pho[1] = phn[1]; pho[2] = phn[2];
-        }
-    }
-    cp_async_wait<0>();
-    if (part) {
-        const double tot = block_sum((double)acc, red);
-        if (threadIdx.x == 0)
-            part[(int64_t)k * (gridDim.x * gridDim.y) + blockIdx.y * gridDim.x + blockIdx.x] = tot;
-    }
-}
-
 static int largest_divisor_le(int L, int cap) {
     for (int d = cap < L ? cap : L; d >= 1; --d)
         if (L % d == 0) return d;
@@ -594,27 +468,13 @@ static ATile make_atile(const Lat& lat, int TX, int TY, int C) {
     return t;
 }
 
-// One launch of the fused A on tile tl: the plain FP32 operator takes the asynchronous-staging
-// kernel where the tile fits it, everything else the register-prefetch kernel.
+// One launch of the fused A with the direction update on tile tl.
 template <typename R>
 static void go_apply_A(hmc_ctx* ctx, const Lat& lat, const ATile& tl, int nrhs, const R* phi, const Site<R>* x,
                        Site<R>* y, double* part, const CgScalars* cgs, const Site<R>* pold, Site<R>* pnew) {
     const dim3 grid(tl.ntx * tl.nty, tl.nchunk, nrhs);
-    const Coef<R> cf = make_coef<R>(ctx->p);
-    if (pnew) {
-        k_apply_A<R, true><<<grid, kAThreads, a_smem_bytes<R>(tl), ctx->stream>>>(lat, cf, tl, phi, x, y, part, cgs,
-                                                                                  pold, pnew);
-        return;
-    }
-    if constexpr (sizeof(R) == 4) {
-        if (tl.TX == 16 && tl.TY == 16) {
-            k_apply_A4<16, 16><<<grid, kAThreads, A4Shape<16, 16>::smem, ctx->stream>>>(lat, cf, tl, phi, x, y, part,
-                                                                                        cgs);
-            return;
-        }
-    }
-    k_apply_A<R, false><<<grid, kAThreads, a_smem_bytes<R>(tl), ctx->stream>>>(lat, cf, tl, phi, x, y, part, cgs,
-                                                                               nullptr, nullptr);
+    k_apply_A<R, true><<<grid, kAThreads, a_smem_bytes<R>(tl), ctx->stream>>>(lat, make_coef<R>(ctx->p), tl, phi, x, y,
+                                                                              part, cgs, pold, pnew);
 }
 
 // Times every valid (TX, TY, C) on the call's own buffers (the launch is idempotent: y, pnew
@@ -675,20 +535,18 @@ int launch_apply_A(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x,
                    const cplx<R>* pold, cplx<R>* pnew) {
     if (nrhs <= 0) return HMC_OK;
     if (pnew && (!cgs || !pold || pold == pnew)) return fail(ctx, HMC_ERR_ARG, "apply_A: bad direction-update buffers");
-    if constexpr (sizeof(R) == 4) {
-        if (!pnew && strip_supported(lat))
-            return launch_apply_A_strip(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
+    if (!pnew) {
+        if constexpr (sizeof(R) == 4) {
+            // (the strip kernel stores whole sites: y 32-byte aligned)
+            if (strip_supported(lat) && aligned32(y))
+                return launch_apply_A_strip(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
+        }
+        return launch_A_two_pass<R>(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
     }
     static PerDevice attr;
     uint64_t bit;
     if (attr.pending(&bit)) {
         HMC_CUDA(ctx, cudaFuncSetAttribute(k_apply_A<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        HMC_CUDA(ctx, cudaFuncSetAttribute(k_apply_A<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        if constexpr (sizeof(R) == 4)
-        {
-            HMC_CUDA(ctx, cudaFuncSetAttribute(k_apply_A4<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)A4Shape<16, 16>::smem));
-        }
         attr.mark(bit);
     }
     const int prec = sizeof(R) == 8 ? HMC_FP64 : HMC_FP32;
@@ -880,16 +738,20 @@ __device__ __forceinline__ void boson_site(const Lat& lat, const BosonCoef& bc,
 // Force: F = -dS_B/dphi (optional) + sum_k 2 dtau g eta Re[X^dag (sigma^x (x) sigma^a) Y],
 // Y = D^dagger X computed on the fly, or read from Yin when a solve's last true-residual
 // evaluation left it (the same stencil on the same X, so the same bits, without the FP64 work).
-// Partials: [0, nblk) = sum_k 2 Re<pf, X> - |Y|^2, [nblk, 2 nblk) = S_B density.
+// With ACT, partials: [0, nblk) = sum_k 2 Re<pf, X> - |Y|^2, [nblk, 2 nblk) = S_B density; pf is read for
+// them only. The FP64 pipe bounds it: 24 operations per site and right-hand side for the force and 16 for
+// the action, every product in a fused multiply-add (about 60 as sums of complex products). 80 x 80 x 160 with
+// 8 right-hand sides and Y given: 1.14 ms before, 0.42 without and 0.62 with the action.
+template <bool ACT>
 __global__ void __launch_bounds__(256) k_force(Lat lat, Coef<double> cf, BosonCoef bc,
                                                const double* __restrict__ phi,
                                                const Site<double>* __restrict__ X,
                                                const Site<double>* __restrict__ pf, int nrhs,
                                                double* __restrict__ F, int include_boson,
                                                double* __restrict__ part, const Site<double>* __restrict__ Yin) {
-    __shared__ double red[8];
+    __shared__ double red[256];
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double spf = 0.0, sb = 0.0;
+    double px = 0.0, y2 = 0.0, sb = 0.0;
     if (s < lat.V) {
         const int64_t V = lat.V;
         const int L = lat.L;
@@ -916,21 +778,23 @@ __global__ void __launch_bounds__(256) k_force(Lat lat, Coef<double> cf, BosonCo
             const Site<double> Y = Yin ? ld(Yin + k * V, s)
                                        : site_op<double>(cf, xc, ld(Xk, sxm), ld(Xk, sxp), ld(Xk, sym), ld(Xk, syp),
                                                          ld(Xk, stm), tsign, p1, p2, p3, eta);
-            const Site<double> pk = load_site(pf + k * V + s);
 #pragma unroll
             for (int a = 0; a < 2; ++a) {
                 const double2 x0 = xc.c[a * 2], x1 = xc.c[a * 2 + 1];
                 const double2 y0 = Y.c[(1 - a) * 2], y1 = Y.c[(1 - a) * 2 + 1];
-                const double2 z01 = cmulconj(x0, y1), z10 = cmulconj(x1, y0);
-                const double2 z00 = cmulconj(x0, y0), z11 = cmulconj(x1, y1);
-                acc[0] += z01.x + z10.x;          // sigma^1
-                acc[1] += z01.y - z10.y;          // sigma^2: Re(-i z01 + i z10)
-                acc[2] += z00.x - z11.x;          // sigma^3
+                // sigma^1: Re(conj x0 y1 + conj x1 y0); sigma^2: Im(conj x0 y1 - conj x1 y0);
+                // sigma^3: Re(conj x0 y0 - conj x1 y1)
+                acc[0] = fma(x0.x, y1.x, fma(x0.y, y1.y, fma(x1.x, y0.x, fma(x1.y, y0.y, acc[0]))));
+                acc[1] = fma(x0.x, y1.y, fma(-x0.y, y1.x, fma(-x1.x, y0.y, fma(x1.y, y0.x, acc[1]))));
+                acc[2] = fma(x0.x, y0.x, fma(x0.y, y0.y, fma(-x1.x, y1.x, fma(-x1.y, y1.y, acc[2]))));
             }
+            if constexpr (ACT) {
+                const Site<double> pk = load_site(pf + k * V + s);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                spf += 2.0 * (pk.c[q].x * xc.c[q].x + pk.c[q].y * xc.c[q].y)
-                       - (Y.c[q].x * Y.c[q].x + Y.c[q].y * Y.c[q].y);
+                for (int q = 0; q < 4; ++q) {
+                    px = fma(pk.c[q].x, xc.c[q].x, fma(pk.c[q].y, xc.c[q].y, px));
+                    y2 = fma(Y.c[q].x, Y.c[q].x, fma(Y.c[q].y, Y.c[q].y, y2));
+                }
             }
         }
         const double f = 2.0 * cf.cpl * eta;
@@ -939,11 +803,13 @@ __global__ void __launch_bounds__(256) k_force(Lat lat, Coef<double> cf, BosonCo
 #pragma unroll
         for (int a = 0; a < 3; ++a) F[a * V + s] = f * acc[a] + Fb[a];
     }
-    const double a = block_sum(spf, red);
-    const double b = block_sum(sb, red);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = a;
-        part[gridDim.x + blockIdx.x] = b;
+    if constexpr (ACT) {
+        const double a = block_sum_256(2.0 * px - y2, red);
+        const double b = block_sum_256(sb, red);
+        if (threadIdx.x == 0) {
+            part[blockIdx.x] = a;
+            part[gridDim.x + blockIdx.x] = b;
+        }
     }
 }
 
@@ -961,12 +827,16 @@ int launch_force(hmc_ctx* ctx, const Lat& lat, double r, const double* phi, cons
                  int* nblk_out, const double2* Y) {
     const int nblk = (int)((lat.V + 255) / 256);
     if (2 * (int64_t)nblk > ctx->part_cap) return fail(ctx, HMC_ERR_ARG, "force: reduction buffer too small");
-    k_force<<<nblk, 256, 0, ctx->stream>>>(lat, make_coef<double>(ctx->p), boson_coef(ctx->p, r), phi,
-                                           reinterpret_cast<const Site<double>*>(X),
-                                           reinterpret_cast<const Site<double>*>(pf), nrhs, F,
-                                           include_boson, part, reinterpret_cast<const Site<double>*>(Y));
+    auto go = [&](auto kernel) {
+        kernel<<<nblk, 256, 0, ctx->stream>>>(lat, make_coef<double>(ctx->p), boson_coef(ctx->p, r), phi,
+                                              reinterpret_cast<const Site<double>*>(X),
+                                              reinterpret_cast<const Site<double>*>(pf), nrhs, F, include_boson, part,
+                                              reinterpret_cast<const Site<double>*>(Y));
+    };
+    if (part) go(k_force<true>);
+    else go(k_force<false>);
     HMC_LAUNCH(ctx, "k_force");
-    *nblk_out = nblk;
+    if (nblk_out) *nblk_out = nblk;
     return HMC_OK;
 }
 

@@ -72,15 +72,6 @@ template <typename R> __device__ __forceinline__ It<R> axpy_it(R a, const It<R>&
     return o;
 }
 
-// v with its sign changed when bit 0 of `neg` is set (integer units: an FP64 multiply costs a slot of
-// the pipe that bounds the FP64 phases)
-__device__ __forceinline__ float flip(float v, int neg) {
-    return __int_as_float(__float_as_int(v) ^ (neg << 31));
-}
-__device__ __forceinline__ double flip(double v, int neg) {
-    return __hiloint2double(__double2hiint(v) ^ (neg << 31), __double2loint(v));
-}
-
 // Item i of D v (DAG = false) or D^dagger v: the stencil of site_op (common.cuh) for one band, the
 // vector read through ld(item).
 template <typename R, bool DAG, typename Ld>
@@ -100,18 +91,14 @@ __device__ __forceinline__ It<R> d_item(const BChainDev& g, const Coef<R>& cf, c
     It<R> o;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        o.s[q].x = fma(d, c.s[q].x, flip(tn.s[q].x, edge));
-        o.s[q].y = fma(d, c.s[q].y, flip(tn.s[q].y, edge));
-        o.s[q].x = fma(hx, xm.s[q].x + xp.s[q].x, o.s[q].x);
-        o.s[q].y = fma(hx, xm.s[q].y + xp.s[q].y, o.s[q].y);
-        o.s[q].x = fma(hy, ym.s[q].x + yp.s[q].x, o.s[q].x);
-        o.s[q].y = fma(hy, ym.s[q].y + yp.s[q].y, o.s[q].y);
+        o.s[q].x = fma(hx, xm.s[q].x + xp.s[q].x, fma(hy, ym.s[q].x + yp.s[q].x, flip(tn.s[q].x, edge)));
+        o.s[q].y = fma(hx, xm.s[q].y + xp.s[q].y, fma(hy, ym.s[q].y + yp.s[q].y, flip(tn.s[q].y, edge)));
     }
     const cplx<R> w0 = w.s[0], w1 = w.s[1];
-    o.s[0].x = fma(q3, w0.x, fma(q1, w1.x, fma(q2, w1.y, o.s[0].x)));
-    o.s[0].y = fma(q3, w0.y, fma(q1, w1.y, fma(-q2, w1.x, o.s[0].y)));
-    o.s[1].x = fma(-q3, w1.x, fma(q1, w0.x, fma(-q2, w0.y, o.s[1].x)));
-    o.s[1].y = fma(-q3, w1.y, fma(q1, w0.y, fma(q2, w0.x, o.s[1].y)));
+    o.s[0].x = fma(d, c.s[0].x, fma(q3, w0.x, fma(q1, w1.x, fma(q2, w1.y, o.s[0].x))));
+    o.s[0].y = fma(d, c.s[0].y, fma(q3, w0.y, fma(q1, w1.y, fma(-q2, w1.x, o.s[0].y))));
+    o.s[1].x = fma(d, c.s[1].x, fma(-q3, w1.x, fma(q1, w0.x, fma(-q2, w0.y, o.s[1].x))));
+    o.s[1].y = fma(d, c.s[1].y, fma(-q3, w1.y, fma(q1, w0.y, fma(q2, w0.x, o.s[1].y))));
     if (centre) *centre = c;
     return o;
 }
