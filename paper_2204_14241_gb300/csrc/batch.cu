@@ -2,8 +2,13 @@
 // of a context is a team of the solver in team.cu (mixed precision, plain CG). The vectors of all pairs
 // are concatenated, chain c's K right-hand sides at item offset off_c ([c][k][site], 4 complex per item).
 //
-// Blocks are dealt to the pairs by volume, so that all pairs take about the same time per iteration;
-// when there are more pairs than resident blocks, one-block teams solve several pairs in turn.
+// The pairs in flight keep their vectors in L2 (x, r, two directions, t_ and phi: 172 bytes a site) where all of
+// them fit: a team each, with blocks by volume, so that all take about the same time per iteration. Past that,
+// 128 pairs of the 64-chain batch (270 MB) streamed from memory in every iteration; there, teams of equal size take
+// the pairs from a queue, largest first, as many teams as fit: a 64-chain trajectory 196 -> 154 ms. (With
+// a set that fits the queue's last pairs leave teams idle: 24 chains, 101 MB, 53 ms in flight, 57 to 63 queued.) A
+// pair's result does not depend on the team that takes it: queued teams have the same number of blocks and so
+// the same order of sums.
 #include <algorithm>
 #include <cmath>
 #include <numeric>
@@ -12,6 +17,8 @@
 #include "team.h"
 
 namespace hmc {
+
+constexpr int64_t kBatchAll = 112 << 20, kBatchQueued = 60 << 20;   // bytes in flight: all pairs at most; queued
 
 // FP32 copies of every chain's phi: block column blockIdx.y is a chain
 __global__ void k_phi_to32_b(const BChainDev* __restrict__ ch) {
@@ -24,10 +31,10 @@ __global__ void k_phi_to32_b(const BChainDev* __restrict__ ch) {
 // ---- host ----------------------------------------------------------------------------------------
 void batch_free(hmc_ctx* ctx) {
     BatchWork& w = ctx->batch;
-    void* ps[] = {w.pairs, w.blk, w.part, w.bar, w.hist, w.fail, w.metric};
+    void* ps[] = {w.pairs, w.blk, w.team, w.next, w.part, w.bar, w.hist, w.fail, w.metric};
     for (void* p : ps)
         if (p) cudaFree(p);
-    w.pairs = nullptr; w.blk = nullptr; w.part = nullptr; w.bar = nullptr; w.hist = nullptr; w.fail = nullptr; w.metric = nullptr;
+    w.pairs = nullptr; w.blk = nullptr; w.team = nullptr; w.next = nullptr; w.part = nullptr; w.bar = nullptr; w.hist = nullptr; w.fail = nullptr; w.metric = nullptr;
     w.K = 0;
     w.kcap = 0;
 }
@@ -41,9 +48,11 @@ int batch_alloc(hmc_ctx* ctx) {
     if ((rc = team_batch_capacity(ctx, &w.cap))) return rc;
     if (w.cap < 1) return fail(ctx, HMC_ERR_CUDA, "batched solve: kernel does not fit on an SM");
     HMC_CUDA(ctx, cudaMalloc(&w.pairs, np * sizeof(TeamPair)));
-    HMC_CUDA(ctx, cudaMalloc((void**)&w.blk, w.cap * sizeof(int2)));
+    HMC_CUDA(ctx, cudaMalloc((void**)&w.blk, w.cap * sizeof(int)));
+    HMC_CUDA(ctx, cudaMalloc((void**)&w.team, w.cap * sizeof(int2)));
+    HMC_CUDA(ctx, cudaMalloc((void**)&w.next, w.cap * sizeof(int)));
     HMC_CUDA(ctx, cudaMalloc((void**)&w.part, 2 * (size_t)w.cap * sizeof(unsigned long long)));
-    HMC_CUDA(ctx, cudaMalloc((void**)&w.bar, np * sizeof(unsigned)));
+    HMC_CUDA(ctx, cudaMalloc((void**)&w.bar, (w.cap + 1) * sizeof(unsigned)));
     HMC_CUDA(ctx, cudaMalloc((void**)&w.hist, HMC_MAX_SOLVES * np * sizeof(TeamStat)));
     HMC_CUDA(ctx, cudaMalloc((void**)&w.fail, sizeof(int)));
     if ((rc = metric_batch_alloc(ctx))) return rc;
@@ -63,51 +72,42 @@ static int batch_setup(hmc_ctx* ctx, int K) {
     std::vector<int> order(np);
     std::iota(order.begin(), order.end(), 0);
     auto vol = [&](int p) { return ctx->chains[p / K].lat.V; };
-    std::vector<TeamPair> pairs(np);   // indexed by pair
-    std::vector<int2> blk;
-    std::vector<int> table;            // pair of each table entry
-    if (np <= w.cap) {
-        // T blocks per pair: one each, then one more to the pair with the most items per block while a
-        // thread of it still has more than one
-        std::vector<int> T(np, 1);
+    const int64_t bytes = 172 * ctx->vtot / nc;   // of a pair, on average
+    std::vector<int> T;
+    w.queued = np > w.cap || np * bytes > kBatchAll;
+    if (w.queued) std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return vol(a) > vol(b); });
+    std::vector<TeamPair> pairs;
+    for (int p : order) pairs.push_back(TeamPair{p / K, p % K});
+    if (w.queued) {
+        // no more blocks than leave a thread of the largest pair one item
+        const int n = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)np, (int64_t)w.cap, kBatchQueued / bytes}));
+        T.assign(n, (int)std::max<int64_t>(1, std::min<int64_t>(w.cap / n, (2 * vol(order[0]) + 255) / 256)));
+    } else {
+        // one block each, then one more to the pair with the most items per block while a thread of it still
+        // has more than one
+        T.assign(np, 1);
         std::vector<std::pair<double, int>> heap;
-        for (int p = 0; p < np; ++p) heap.push_back({2.0 * vol(p), p});
+        for (int e = 0; e < np; ++e) heap.push_back({2.0 * vol(order[e]), e});
         std::make_heap(heap.begin(), heap.end());
         for (int left = w.cap - np; left > 0 && heap.front().first > 256; --left) {
             std::pop_heap(heap.begin(), heap.end());
-            const int p = heap.back().second;
-            heap.back().first = 2.0 * vol(p) / ++T[p];
+            const int e = heap.back().second;
+            heap.back().first = 2.0 * vol(order[e]) / ++T[e];
             std::push_heap(heap.begin(), heap.end());
         }
-        for (int p = 0; p < np; ++p) {
-            pairs[p] = TeamPair{p / K, p % K, (int)blk.size(), T[p]};
-            for (int j = 0; j < T[p]; ++j) blk.push_back(make_int2(p, 1));
-            table.push_back(p);
-        }
-    } else {
-        // largest first to the block with the least so far
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return vol(a) > vol(b); });
-        std::vector<int64_t> load(w.cap, 0);
-        std::vector<std::vector<int>> own(w.cap);
-        for (int p : order) {
-            const int j = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-            load[j] += vol(p);
-            own[j].push_back(p);
-        }
-        for (int j = 0; j < w.cap; ++j) {
-            blk.push_back(make_int2((int)table.size(), (int)own[j].size()));
-            for (int p : own[j]) {
-                pairs[p] = TeamPair{p / K, p % K, j, 1};
-                table.push_back(p);
-            }
-        }
     }
-    std::vector<TeamPair> tab;
-    for (int p : table) tab.push_back(pairs[p]);
-    HMC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // the tables may be in use by earlier work
-    HMC_CUDA(ctx, cudaMemcpy(w.pairs, tab.data(), tab.size() * sizeof(TeamPair), cudaMemcpyHostToDevice));
-    HMC_CUDA(ctx, cudaMemcpy(w.blk, blk.data(), blk.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    std::vector<int> blk;
+    std::vector<int2> team;
+    for (int j = 0; j < (int)T.size(); ++j) {
+        team.push_back(make_int2((int)blk.size(), T[j]));
+        blk.insert(blk.end(), T[j], j);
+    }
+    w.teams = (int)team.size();
     w.grid = (int)blk.size();
+    HMC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // the tables may be in use by earlier work
+    HMC_CUDA(ctx, cudaMemcpy(w.pairs, pairs.data(), pairs.size() * sizeof(TeamPair), cudaMemcpyHostToDevice));
+    HMC_CUDA(ctx, cudaMemcpy(w.blk, blk.data(), blk.size() * sizeof(int), cudaMemcpyHostToDevice));
+    HMC_CUDA(ctx, cudaMemcpy(w.team, team.data(), team.size() * sizeof(int2), cudaMemcpyHostToDevice));
     w.K = K;
     return HMC_OK;
 }
@@ -139,7 +139,12 @@ int batched_solve(hmc_ctx* ctx, int K, const double2* b, double2* x, bool use_x0
     HMC_LAUNCH(ctx, "k_phi_to32_b");
     TeamArgs<float> a{};
     a.pairs = reinterpret_cast<const TeamPair*>(w.pairs);
+    a.npairs = nc * K;
+    a.next = w.next;
+    a.nteams = w.teams;
     a.blk = w.blk;
+    a.team = w.team;
+    a.queue = w.queued ? reinterpret_cast<int*>(w.bar) + w.teams : nullptr;
     a.ch = w.ch;
     a.K = K;
     a.cf = make_coef<float>(ctx->p);
@@ -163,7 +168,7 @@ int batched_solve(hmc_ctx* ctx, int K, const double2* b, double2* x, bool use_x0
     a.use_x0 = use_x0 ? 1 : 0;
     a.test_timeout = ctx->p.test_wait_timeout;
     a.timeout_ns = ctx->p.wait_spin_limit > 0 ? (long long)ctx->p.wait_spin_limit * 1000LL : 2000000000LL;
-    return team_launch_batch(ctx, a, w.grid, nc * K);
+    return team_launch_batch(ctx, a, w.grid);
 }
 
 int batched_collect(hmc_ctx* ctx, int K, int nsolves, int* iterations, double* worst_resid, int* reliable_updates) {

@@ -96,12 +96,15 @@ struct TeamCap {   // resident blocks of one team kernel
 
 // Device state of the batched solve, built on first use for a right-hand-side count.
 struct BatchWork {
-    int K = 0, grid = 0;
+    int K = 0, teams = 0, grid = 0;
+    bool queued = false;        // teams take pairs from a queue
     int kcap = 0, cap = 0;      // right-hand sides and resident blocks allocated for at hmc_init
-    void* pairs = nullptr;      // TeamPair table, each team's pairs together
-    int2* blk = nullptr;        // per block: first pair of its team, number of pairs
+    void* pairs = nullptr;      // TeamPair queue, largest first
+    int* blk = nullptr;         // team of each block
+    int2* team = nullptr;       // first block and blocks of each team
+    int* next = nullptr;        // the entry each team takes next
     unsigned long long* part = nullptr;   // partial sums
-    unsigned* bar = nullptr;    // an arrival counter per pair
+    unsigned* bar = nullptr;    // an arrival counter per team, then the queue's
     BChainDev* ch = nullptr;    // chain table (n_chains entries)
     TeamStat* hist = nullptr;   // per-solve statistics of every pair, HMC_MAX_SOLVES solves of a trajectory
     int* fail = nullptr;        // failure flags of every solve of the trajectory

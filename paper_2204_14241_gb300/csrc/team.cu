@@ -9,7 +9,7 @@
 //
 // Small lattices are bound by latency, a launch or a barrier after every few microseconds of work: with a
 // launch per step and the host reading flags an iteration took 27 to 60 us (CG, PCG) whatever the size, here
-// 5 to 7 and 14 to 30 up to some 30000 sites. From about 10^5 sites memory bounds complex64 and the FP64 pipe
+// 4 to 8 and 13 to 30 up to some 30000 sites. From about 10^5 sites memory bounds complex64 and the FP64 pipe
 // complex128.
 //
 // Work is dealt in items, one band's two spin components of one site (16 bytes in complex64): a block
@@ -25,7 +25,7 @@
 // and take the same decisions: no scalar kernel, no flag to read back, no host in the loop.
 // Vectors that other blocks write are read with plain loads: the barrier's acquire drops the SM's L1
 // lines, and within a phase L1 then serves the neighbours (read through L2 instead, 14 site loads per site
-// in the first phase, and with FP64 sums, an iteration of the 64-chain batch took 0.37 ms; now 0.17).
+// in the first phase, and with FP64 sums, an iteration of the 64-chain batch took 0.37 ms against 0.17).
 //
 // A cooperative team's barrier spins on a counter with a time limit; a block that gives up sets the device
 // error word and returns.
@@ -158,15 +158,45 @@ template <typename R> __device__ __forceinline__ void sq_it(Sum2<R>& a, const It
     }
 }
 
-// a / b to an ulp or so: two Newton steps on the FP32 quotient (FP64 latency is what a scalar costs here: a
-// full division takes three times as long), or the division where FP32 does not reach
-__device__ __forceinline__ double quot(double a, double b) {
-    const float bf = (float)b, af = (float)a;
-    if (!(fabsf(bf) > 1e-30f && fabsf(bf) < 1e30f && fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return a / b;
-    const double y = (double)(1.0f / bf);
-    double q = a * y;
-    q = fma(fma(-q, b, a), y, q);
-    return fma(fma(-q, b, a), y, q);
+// Scalars of the recurrence: FP64, or an FP32 pair (48 bits) in complex64, where they end in an FP32 alpha or
+// beta: one thread works on them while the rest wait, and an FP64 operation takes 65 clocks, a division 570.
+template <typename R> struct Num;
+template <> struct Num<double> {
+    double v;
+    __device__ __forceinline__ Num() {}
+    __device__ __forceinline__ Num(double x) : v(x) {}
+    __device__ __forceinline__ Num(const Sum2<double>& a) : v(a.v) {}
+    __device__ __forceinline__ double get() const { return v; }
+    __device__ __forceinline__ bool finite() const { return isfinite(v); }
+    __device__ __forceinline__ bool positive() const { return v > 0.0; }
+    __device__ __forceinline__ Num times(const Num& s) const { return Num(v * s.v); }
+};
+template <> struct Num<float> {
+    float hi, lo;
+    __device__ __forceinline__ Num() {}
+    __device__ __forceinline__ Num(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
+    __device__ __forceinline__ Num(const Sum2<float>& a) {
+        hi = __fadd_rn(a.hi, a.lo);
+        lo = __fadd_rn(__fsub_rn(a.hi, hi), a.lo);
+    }
+    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ bool finite() const { return isfinite(hi); }
+    __device__ __forceinline__ bool positive() const { return hi > 0.f; }
+    __device__ __forceinline__ Num times(const Num& s) const {
+        Num o;
+        o.hi = __fmul_rn(hi, s.hi);
+        o.lo = __fmaf_rn(hi, s.hi, -o.hi) + __fmaf_rn(hi, s.lo, __fmul_rn(lo, s.hi));
+        return o;
+    }
+};
+__device__ __forceinline__ double quot(const Num<double>& a, const Num<double>& b) { return a.v / b.v; }
+// a / b rounded to FP32: the FP32 quotient and its remainder's, or FP64 where FP32 does not reach
+__device__ __forceinline__ float quot(const Num<float>& a, const Num<float>& b) {
+    if (!(fabsf(b.hi) > 1e-30f && fabsf(b.hi) < 1e30f && fabsf(a.hi) > 1e-30f && fabsf(a.hi) < 1e30f))
+        return (float)(a.get() / b.get());
+    const float q = a.hi / b.hi;
+    const float rem = __fmaf_rn(-q, b.hi, a.hi) + __fmaf_rn(-q, b.lo, a.lo);
+    return q + rem / b.hi;
 }
 
 struct NoSum {   // a barrier without a sum
@@ -178,10 +208,11 @@ struct NoSum {   // a barrier without a sum
 };
 
 // ---- team ------------------------------------------------------------------------------------------
-// Scalars of a solve, in shared memory: written by one thread, so that no other spends the FP64 pipe's
-// time on them (a double division by all 256 threads takes 0.7 us of it).
+// A solve's state, in shared memory, written by one thread.
 template <typename R> struct Ctl {
-    double rr, b2, r2, r2true, r2max;
+    double b2, r2true;         // ||b||^2, the last true ||r||^2
+    double stop, ru_below;     // tol^2 ||b||^2; ||r||^2 at which a reliable update is due
+    Num<R> rr;
     R alpha, beta;
     int it, n_ru, hold, wait;
     int active, nonfinite, met, ru, last;
@@ -291,18 +322,26 @@ __device__ __forceinline__ bool sync_sum(Team& tm, C& ctl, unsigned long long* r
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         __syncwarp();
         if (!std::is_same<S, NoSum>::value) {
+            // eight loads in flight: one after the other they took 0.7 thousand clocks each
             acc = S();
-            for (int b = lane; b < tm.T; b += 32) {
-                S o;
-                o.from(__ldcg(row + b));
-                acc.plus(o);
+            for (int b = lane; b < tm.T; b += 256) {
+                unsigned long long v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = b + 32 * j < tm.T ? __ldcg(row + b + 32 * j) : 0ull;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if (32 * j >= tm.T) break;
+                    S o;
+                    o.from(v[j]);
+                    acc.plus(o);
+                }
             }
             warp_plus(acc, 16);
         }
     }
     if (w == 0 && lane == 0) {
         ctl.ok = ok ? 1 : 0;
-        if (ok) fin(acc.get());
+        if (ok) fin(acc);
     }
     __syncthreads();
     tm.never = false;
@@ -377,7 +416,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     const R* phi;
     if constexpr (kMixed) phi = g.phi32;
     else phi = g.phi64;
-    auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](double) {}); };
+    auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](const NoSum&) {}); };
     auto ld64 = [](const double2* v) { return [v](int j) { return ld_it<double>(v, j); }; };
     auto ldr = [](const C* v) { return [v](int j) { return ld_it<R>(v, j); }; };
 
@@ -407,14 +446,17 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             sq_it(sb, bb);
             sq_it(sr, rr);
         }
-        if (!sync_sum<CLU>(tm, c, red, sb, [&](double v) { c.b2 = v; })) return false;
-        if (!sync_sum<CLU>(tm, c, red, sr, [&](double v) {
-                c.r2 = c.r2true = c.r2max = c.rr = v;
+        if (!sync_sum<CLU>(tm, c, red, sb, [&](const Sum2<double>& v) { c.b2 = v.v; })) return false;
+        if (!sync_sum<CLU>(tm, c, red, sr, [&](const Sum2<double>& v) {
+                c.r2true = v.v;
+                c.rr = Num<R>(v.v);
                 c.alpha = c.beta = (R)0;
                 c.it = c.n_ru = c.hold = 0;
                 c.wait = 4;
-                c.nonfinite = !(isfinite(c.b2) && isfinite(v));
-                c.active = !c.nonfinite && c.b2 > 0.0 && v > a.tol2 * c.b2;
+                c.stop = a.tol2 * c.b2;
+                c.ru_below = kMixed ? fmax(c.stop, a.delta2 * v.v) : c.stop;
+                c.nonfinite = !(isfinite(c.b2) && isfinite(v.v));
+                c.active = !c.nonfinite && c.b2 > 0.0 && v.v > c.stop;
             }))
             return false;
     }
@@ -514,13 +556,14 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         });
         return sync();
     };
+    const Num<R> scale(PRE ? a.pre.scale : 1.0);
     if constexpr (PRE) {
         if (c.active) {   // first direction p = z, rr = <r, z>
             forward();
             if (!sync()) return false;
-            if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
-                    c.rr = v * a.pre.scale;
-                    if (!isfinite(v)) c.nonfinite = 1;
+            if (!sync_sum<CLU>(tm, c, red, tau(), [&](const Sum2<R>& v) {
+                    c.rr = Num<R>(v).times(scale);
+                    if (!c.rr.finite()) c.nonfinite = 1;
                 }))
                 return false;
             if (!inverse()) return false;
@@ -547,9 +590,10 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 sq_it(acc, o);
             }
         }
-        if (!sync_sum<CLU>(tm, c, red, acc, [&](double pAp) {
-                c.alpha = (R)((pAp > 0.0 && isfinite(pAp)) ? quot(c.rr, pAp) : 0.0);
-                if (!isfinite(pAp)) c.nonfinite = 1;
+        if (!sync_sum<CLU>(tm, c, red, acc, [&](const Sum2<R>& v) {
+                const Num<R> pAp(v);
+                c.alpha = (pAp.positive() && pAp.finite()) ? quot(c.rr, pAp) : (R)0;
+                if (!pAp.finite()) c.nonfinite = 1;
             }))
             return false;
         // ---- q = D t_, x += alpha p, r -= alpha q, ||r||^2 (PRE: and the spectrum of r) ----
@@ -575,19 +619,21 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         } else {
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) update(i);
         }
-        if (!sync_sum<CLU>(tm, c, red, acc, [&](double v) {
-                c.r2 = v;
-                if (!isfinite(v)) c.nonfinite = 1;
+        if (!sync_sum<CLU>(tm, c, red, acc, [&](const Sum2<R>& sum) {
+                const Num<R> r2(sum);
+                const double v = r2.get();
+                if (!r2.finite()) c.nonfinite = 1;
                 if constexpr (!PRE) {
-                    c.beta = (R)(c.rr > 0.0 ? quot(v, c.rr) : 0.0);
-                    c.rr = v;
+                    c.beta = c.rr.positive() ? quot(r2, c.rr) : (R)0;
+                    c.rr = r2;
                 }
                 c.last = ++c.it >= a.maxit;
                 // Near the rounding floor of the true residual, an update after every iteration that meets
                 // the tolerance would put its noise back into the recurrence each time and hardly ever stop:
                 // after one that misses, some iterations pass before the next.
-                c.met = v <= a.tol2 * c.b2 && c.it >= c.hold;
-                c.ru = c.met || (kMixed && v < a.delta2 * c.r2max) || c.last;
+                c.ru = v <= c.ru_below && (c.it >= c.hold || v > c.stop);
+                c.met = c.ru && v <= c.stop;
+                if (c.last) c.ru = 1;
             }))
             return false;
         if (c.nonfinite) break;
@@ -621,14 +667,15 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 st_it<R>(r, i, rl);
                 sq_it(acc64, rd);
             }
-            if (!sync_sum<CLU>(tm, c, red, acc64, [&](double v) {
+            if (!sync_sum<CLU>(tm, c, red, acc64, [&](const Sum2<double>& sum) {
+                    const double v = sum.v;
                     c.r2true = v;
                     ++c.n_ru;
                     if (!isfinite(v)) c.nonfinite = 1;
-                    else if (v <= a.tol2 * c.b2) c.active = 0;
+                    else if (v <= c.stop) c.active = 0;
                     else {
-                        c.r2max = v;
-                        if constexpr (!PRE) c.rr = v;
+                        if (kMixed) c.ru_below = fmax(c.stop, a.delta2 * v);
+                        if constexpr (!PRE) c.rr = Num<R>(v);
                         if (c.met) {
                             c.hold = c.it + c.wait;
                             c.wait = 8;
@@ -639,11 +686,11 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             if (c.nonfinite || !c.active || c.last) break;
         }
         if constexpr (PRE) {
-            if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
-                    v *= a.pre.scale;
-                    c.beta = (R)(c.rr > 0.0 ? quot(v, c.rr) : 0.0);
-                    c.rr = v;
-                    if (!isfinite(v)) c.nonfinite = 1;
+            if (!sync_sum<CLU>(tm, c, red, tau(), [&](const Sum2<R>& v) {
+                    const Num<R> rz = Num<R>(v).times(scale);
+                    c.beta = c.rr.positive() ? quot(rz, c.rr) : (R)0;
+                    c.rr = rz;
+                    if (!rz.finite()) c.nonfinite = 1;
                 }))
                 return false;
             if (ru) {
@@ -651,9 +698,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 // which near the floor is larger, it would blow the old direction up
                 forward();
                 if (!sync()) return false;
-                if (!sync_sum<CLU>(tm, c, red, tau(), [&](double v) {
-                        c.rr = v * a.pre.scale;
-                        if (!isfinite(v)) c.nonfinite = 1;
+                if (!sync_sum<CLU>(tm, c, red, tau(), [&](const Sum2<R>& v) {
+                        c.rr = Num<R>(v).times(scale);
+                        if (!c.rr.finite()) c.nonfinite = 1;
                     }))
                     return false;
             }
@@ -697,20 +744,34 @@ k_team(const __grid_constant__ TeamArgs<R> a) {
     tm.timeout_ns = a.timeout_ns;
     PreTab<R> pt;
     if constexpr (PRE) pt = pre_tables<R>(a.pre, a.one.L, a.one.Nt, smem);
-    // entries [mine.x, mine.x + mine.y) of the table of pairs, in turn
-    const int2 mine = a.pairs ? a.blk[blockIdx.x] : make_int2(blockIdx.x / a.T, 1);
-    for (int e = mine.x; e < mine.x + mine.y; ++e) {
-        TeamPair tp{0, e, e * a.T, a.T};
-        if (a.pairs) tp = a.pairs[e];
+    const int team = a.pairs ? a.blk[blockIdx.x] : blockIdx.x / a.T;
+    tm.b0 = a.pairs ? a.team[team].x : team * a.T;
+    tm.T = a.pairs ? a.team[team].y : a.T;
+    tm.rank = blockIdx.x - tm.b0;
+    tm.cnt = a.bar + team;
+    tm.epoch = 0;
+    if (!a.pairs) {   // one right-hand side per team
+        if (threadIdx.x == 0) g = a.one;
         __syncthreads();
-        if (threadIdx.x == 0) g = a.pairs ? a.ch[tp.chain] : a.one;
-        __syncthreads();
-        tm.b0 = tp.b0;
-        tm.T = tp.T;
-        tm.rank = blockIdx.x - tp.b0;
-        tm.cnt = a.bar + e;
-        tm.epoch = 0;
-        if (!team_run<R, PRE, CLU>(a, tm, ctl, g, tp.k, tp.chain * a.K + tp.k, pt, red)) return;
+        team_run<R, PRE, CLU>(a, tm, ctl, g, team, team, pt, red);
+        return;
+    }
+    // a batch: team j solves pair j, or (queue) teams take the next pair until there is none
+    if constexpr (!PRE && !CLU && sizeof(R) == 4) {
+        __shared__ int entry;
+        int e = team;
+        do {
+            if (a.queue) {
+                if (tm.rank == 0 && threadIdx.x == 0) __stcg(a.next + team, atomicAdd(a.queue, 1));
+                if (!sync_sum<CLU>(tm, ctl, red, NoSum(), [&](const NoSum&) { entry = __ldcg(a.next + team); })) return;
+                e = entry;
+            }
+            if (e >= a.npairs) return;
+            const TeamPair tp = a.pairs[e];
+            if (threadIdx.x == 0) g = a.ch[tp.chain];
+            __syncthreads();
+            if (!team_run<R, PRE, CLU>(a, tm, ctl, g, tp.k, tp.chain * a.K + tp.k, pt, red)) return;
+        } while (a.queue);
     }
 }
 
@@ -803,10 +864,11 @@ template <typename R, bool PRE> static int capacity(hmc_ctx* ctx, size_t smem, i
 // Cooperative launch, or one cluster per right-hand side (CLU), through the attribute form, which stream
 // capture records as such a kernel node.
 template <typename R, bool PRE, bool CLU>
-static int launch(hmc_ctx* ctx, const TeamArgs<R>& a, int grid, size_t smem, int npairs) {
+static int launch(hmc_ctx* ctx, const TeamArgs<R>& a, int grid, size_t smem) {
     int rc;
     if ((rc = set_attr<R, PRE, CLU>(ctx))) return rc;
-    if (!CLU) HMC_CUDA(ctx, cudaMemsetAsync(a.bar, 0, npairs * sizeof(unsigned), ctx->stream));
+    // the teams' arrival counters and, behind them, the queue of a batch
+    if (!CLU) HMC_CUDA(ctx, cudaMemsetAsync(a.bar, 0, ((a.pairs ? a.nteams : grid / a.T) + 1) * sizeof(unsigned), ctx->stream));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(TeamBounds<R, PRE, CLU>::threads);
@@ -830,8 +892,8 @@ static int launch(hmc_ctx* ctx, const TeamArgs<R>& a, int grid, size_t smem, int
 
 int team_batch_capacity(hmc_ctx* ctx, int* cap) { return capacity<float, false>(ctx, 0, cap); }
 
-int team_launch_batch(hmc_ctx* ctx, const TeamArgs<float>& a, int grid, int npairs) {
-    return launch<float, false, false>(ctx, a, grid, 0, npairs);
+int team_launch_batch(hmc_ctx* ctx, const TeamArgs<float>& a, int grid) {
+    return launch<float, false, false>(ctx, a, grid, 0);
 }
 
 // clusters of T blocks of k_team<R, PRE, true> that are resident at a time
@@ -919,6 +981,13 @@ static int make_plan(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond, TeamPr
         return HMC_OK;
     }
     if ((rc = capacity<R, false>(ctx, 0, &cap))) return rc;
+    if (sizeof(R) == 8 && n > 256 && n * nrhs <= 131072 && cap >= nrhs) {
+        // A block's items take their SM's FP64 pipe 16 clocks a warp and operation: two warps of items a block, one
+        // block an SM (11.6 us an iteration at 8 x 8 x 16 to 16 x 16 x 16, against 14.8 with 256 items a block;
+        // past that size two blocks an SM are ahead, 359 : 403 at 80 x 80 x 160)
+        plan->T = (int)std::min<int64_t>(std::max(1, std::min(cap, ctx->num_sms) / nrhs), (n + 63) / 64);
+        return HMC_OK;
+    }
     plan->T = (int)std::min<int64_t>(cap / nrhs, (n + 255) / 256);
     return HMC_OK;
 }
@@ -932,7 +1001,7 @@ static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2*
     int rc;
     if ((rc = make_plan<R>(ctx, lat, nrhs, precond, &a.pre, &plan))) return rc;
     const int T = plan.T;
-    if (T < 1 || 2 * (int64_t)T * nrhs + nrhs > ctx->part_cap) return HMC_OK;
+    if (T < 1 || 2 * (int64_t)T * nrhs + nrhs + 1 > ctx->part_cap) return HMC_OK;
     *done = true;
     team_geometry(&a.one, lat);
     a.one.off = 0;
@@ -960,7 +1029,7 @@ static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2*
         a.z = ctx->d_p64b;
     }
     a.bar = reinterpret_cast<unsigned*>(ctx->d_part);
-    a.part = reinterpret_cast<unsigned long long*>(ctx->d_part) + nrhs;
+    a.part = reinterpret_cast<unsigned long long*>(ctx->d_part) + nrhs + 1;
     a.flags = ctx->d_flags;
     // statistics in the scalars of the separate kernels, which this solve does not use
     static_assert(sizeof(TeamStat) <= sizeof(CgScalars), "statistics fit");
@@ -975,11 +1044,11 @@ static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2*
     a.timeout_ns = a.test_timeout && ctx->p.wait_spin_limit > 0 ? (long long)ctx->p.wait_spin_limit * 1000LL
                                                                 : 2000000000LL;
     const int grid = T * nrhs;
-    if (plan.cluster && precond) rc = launch<R, true, true>(ctx, a, grid, plan.smem, nrhs);
+    if (plan.cluster && precond) rc = launch<R, true, true>(ctx, a, grid, plan.smem);
     else if (plan.cluster) {
-        if constexpr (sizeof(R) == 4) rc = launch<R, false, true>(ctx, a, grid, 0, nrhs);
+        if constexpr (sizeof(R) == 4) rc = launch<R, false, true>(ctx, a, grid, 0);
     } else
-        rc = precond ? launch<R, true, false>(ctx, a, grid, plan.smem, nrhs) : launch<R, false, false>(ctx, a, grid, 0, nrhs);
+        rc = precond ? launch<R, true, false>(ctx, a, grid, plan.smem) : launch<R, false, false>(ctx, a, grid, 0);
     if (rc) return rc;
     HMC_CUDA(ctx, cudaMemcpyAsync(ctx->h_cg, a.stat, nrhs * sizeof(TeamStat), cudaMemcpyDeviceToHost, ctx->stream));
     if ((rc = check_device_flags(ctx))) return rc;   // synchronises

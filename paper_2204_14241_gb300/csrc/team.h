@@ -8,10 +8,9 @@ namespace hmc {
 constexpr int kTeamSmem = 216 * 1024;   // dynamic shared memory of a preconditioned block, at most
 constexpr int kTeamTau = 64;      // most sites of a tau tile
 
-// One (chain, right-hand side) pair of a batched solve and its blocks.
+// One (chain, right-hand side) pair of a batched solve.
 struct TeamPair {
     int chain, k;
-    int b0, T;
 };
 
 // Preconditioner tables (device) and splits L = x1 x2, Nt = t1 t2 of the PCG phases.
@@ -28,8 +27,11 @@ template <typename R> struct TeamPre {
 };
 
 template <typename R> struct TeamArgs {
-    const TeamPair* pairs;     // batched: table of pairs; otherwise null, T blocks per right-hand side of `one`
-    const int2* blk;           // batched: per block the first table entry and the number of entries it solves
+    const TeamPair* pairs;     // batched: the queue, npairs entries; otherwise null, a right-hand side of `one` per team
+    int npairs, nteams;
+    const int* blk;            // batched: the team of each block
+    const int2* team;          // batched: first block and blocks of each team
+    int *queue, *next;         // batched: entries taken (null: team j solves pair j); the entry each team takes next
     const BChainDev* ch;
     BChainDev one;
     int T, K;
@@ -38,7 +40,7 @@ template <typename R> struct TeamArgs {
     const double2* b;
     double2 *x64, *t64;        // solution; its D^dagger image at the last true residual
     cplx<R> *x, *r, *pA, *pB, *t, *z;   // x: FP32 iterate (mixed); pB: second direction (mixed CG); z: PCG
-    unsigned* bar;             // an arrival counter per table entry, zeroed before the launch
+    unsigned* bar;             // an arrival counter per team, and one word behind them, zeroed before the launch
     unsigned long long* part;  // [2][blocks] partial sums
     int* flags;                // device error word
     int* fail;                 // OR of the pairs' failure flags (may be null)
@@ -51,7 +53,7 @@ template <typename R> struct TeamArgs {
 
 void team_geometry(BChainDev* d, const Lat& lat);
 int team_batch_capacity(hmc_ctx* ctx, int* cap);
-int team_launch_batch(hmc_ctx* ctx, const TeamArgs<float>& a, int grid, int npairs);
+int team_launch_batch(hmc_ctx* ctx, const TeamArgs<float>& a, int grid);
 // Solves all right-hand sides in one launch (cg_run's contract); *done = false where the size, the
 // lattice's factors or the workspace rule that out and nothing was launched.
 int team_solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2* b, double2* x, int nrhs, double tol,
