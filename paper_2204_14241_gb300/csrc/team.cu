@@ -72,17 +72,41 @@ template <typename R> __device__ __forceinline__ It<R> axpy_it(R a, const It<R>&
     return o;
 }
 
+// Two orders of a vector's items. Site-major, the public layout: 2 s + band. Band-major (BM), the vectors of the
+// preconditioned solver: (2 t + band) L^2 + y L + x, so that a (slice, band) plane is one run.
+__device__ __forceinline__ int to_bm(const BChainDev& g, int i) {
+    const int s = i >> 1, t = fdiv(s, g.dLL);
+    return (2 * t + (i & 1)) * g.LL + (s - t * g.LL);
+}
+__device__ __forceinline__ int from_bm(const BChainDev& g, int i) {
+    const int q = fdiv(i, g.dLL);
+    return 2 * ((q >> 1) * g.LL + (i - q * g.LL)) + (q & 1);
+}
+
 // Item i of D v (DAG = false) or D^dagger v: the stencil of site_op (common.cuh) for one band, the
 // vector read through ld(item).
-template <typename R, bool DAG, typename Ld>
+template <typename R, bool DAG, bool BM, typename Ld>
 __device__ __forceinline__ It<R> d_item(const BChainDev& g, const Coef<R>& cf, const R* __restrict__ phi, int i,
                                         const Ld& ld, It<R>* centre = nullptr) {
-    const int band = i & 1, s = i >> 1;
-    const int t = fdiv(s, g.dLL), rem = s - t * g.LL, y = fdiv(rem, g.dL), x = rem - y * g.L;
     const int L = g.L, LL = g.LL, hop = 2 * ((int)g.V - LL);
-    const It<R> c = ld(i), w = ld(i ^ 1);
-    const It<R> xm = ld(x ? i - 2 : i + 2 * (L - 1)), xp = ld(x + 1 < L ? i + 2 : i - 2 * (L - 1));
-    const It<R> ym = ld(y ? i - 2 * L : i + 2 * (LL - L)), yp = ld(y + 1 < L ? i + 2 * L : i - 2 * (LL - L));
+    int band, s, t, rem;
+    if (BM) {
+        const int q = fdiv(i, g.dLL);
+        band = q & 1;
+        t = q >> 1;
+        rem = i - q * LL;
+        s = t * LL + rem;
+    } else {
+        band = i & 1;
+        s = i >> 1;
+        t = fdiv(s, g.dLL);
+        rem = s - t * LL;
+    }
+    const int y = fdiv(rem, g.dL), x = rem - y * L;
+    constexpr int u = BM ? 1 : 2;   // items per step along x
+    const It<R> c = ld(i), w = ld(BM ? (band ? i - LL : i + LL) : i ^ 1);
+    const It<R> xm = ld(x ? i - u : i + u * (L - 1)), xp = ld(x + 1 < L ? i + u : i - u * (L - 1));
+    const It<R> ym = ld(y ? i - u * L : i + u * (LL - L)), yp = ld(y + 1 < L ? i + u * L : i - u * (LL - L));
     const int edge = DAG ? (t == 0) : (t + 1 == g.Nt);   // the time hop crosses the antiperiodic boundary
     const It<R> tn = ld(DAG ? (edge ? i + hop : i - 2 * LL) : (edge ? i - hop : i + 2 * LL));
     const R f = flip(cf.cpl, (x + y) & 1);
@@ -389,9 +413,12 @@ __device__ __forceinline__ void plane_forward(const TeamPre<R>& q, const PreTab<
     __syncthreads();
     dft_forward(p.tile, rows, q.x1, q.x2, 2, p.twx);
     dft_forward(p.tile, cols, q.x1, q.x2, 2 * RS, p.twx);
-    for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
-        const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), x = j - y * L;
-        z[(int64_t)(t0 + pl * T) * g.LL * 2 + 2 * j + (e & 1)] = p.tile[pl * q.plane + (y * RS + x) * 2 + (e & 1)];
+    for (int e = threadIdx.x; e < np * g.LL; e += blockDim.x) {
+        const int pl = fdiv(e, g.dLL), j = e - pl * g.LL, y = fdiv(j, g.dL), at = pl * q.plane + (y * RS + j - y * L) * 2;
+        It<R> v;
+        v.s[0] = p.tile[at];
+        v.s[1] = p.tile[at + 1];
+        st_it<R>(z, (t0 + pl * T) * g.LL + j, v);
     }
     __syncthreads();
 }
@@ -417,12 +444,13 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     if constexpr (kMixed) phi = g.phi32;
     else phi = g.phi64;
     auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](const NoSum&) {}); };
+    auto in = [&](int i) { return PRE ? to_bm(g, i) : i; };   // from the public layout to the solver's
     auto ld64 = [](const double2* v) { return [v](int j) { return ld_it<double>(v, j); }; };
     auto ldr = [](const C* v) { return [v](int j) { return ld_it<R>(v, j); }; };
 
     // ---- start: r = b - A x (or b), zero directions, norms ----------------------------------------
     if (a.use_x0) {
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true>(g, a.cf64, g.phi64, i, ld64(x64)));
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
         if (!sync()) return false;
     }
     {
@@ -431,7 +459,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             const It<double> bb = ld_it<double>(b, i);
             It<double> rr = bb;
             if (a.use_x0) {
-                rr = axpy_it<double>(-1.0, d_item<double, false>(g, a.cf64, g.phi64, i, ld64(t64)), bb);
+                rr = axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), bb);
             } else {
                 st_it<double>(x64, i, It<double>{});
                 st_it<double>(t64, i, It<double>{});   // D^dagger x of the zero start
@@ -439,10 +467,11 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             It<R> rl;
 #pragma unroll
             for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rr.s[s].x, (R)rr.s[s].y);
-            st_it<R>(r, i, rl);
-            if constexpr (kMixed) st_it<R>(x, i, It<R>{});
+            const int o = in(i);
+            st_it<R>(r, o, rl);
+            if constexpr (kMixed) st_it<R>(x, o, It<R>{});
             // the first direction is r (or z): the on-the-fly and the inverse-FFT forms add 0 * p
-            st_it<R>(pold, i, !kMixed && !PRE ? rl : It<R>{});
+            st_it<R>(pold, o, !kMixed && !PRE ? rl : It<R>{});
             sq_it(sb, bb);
             sq_it(sr, rr);
         }
@@ -471,8 +500,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         const int RS = row_stride(g.L);
         for (int e = threadIdx.x; e < np * g.LL; e += blockDim.x) {
             const int pl = fdiv(e, g.dLL), j = e - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * g.L;
-            const int task = t0 + pl * tm.T;
-            f(2 * ((task >> 1) * g.LL + j) + (task & 1), pl * a.pre.plane + (y * RS + xx) * 2);
+            f((t0 + pl * tm.T) * g.LL + j, pl * a.pre.plane + (y * RS + xx) * 2);
         }
     };
     // spectra of r's planes
@@ -500,29 +528,39 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 base_s[p] = q.c0[band] + q.chx[band] * pt.cosk[xx] + q.chy[band] * pt.cosk[y];
             }
             C* zp = z + ((int64_t)band * g.LL + j0) * 2;
-            const int64_t step = (int64_t)4 * g.LL;
-            const int live = 2 * min(q.W, g.LL - j0);
-            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
-                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
-                pt.tile[e] = l < live ? cmulconj(pt.twist[ts], zp[ts * step + l]) : mk<C>(0, 0);
+            const int step = 2 * g.LL, live = min(q.W, g.LL - j0), ne = g.Nt * q.W;   // items
+            for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+                const int ts = fdiv(e, q.dW), l = e - ts * q.W;
+                const C w = pt.twist[ts];
+                It<R> v{};
+                if (l < live) v = ld_it<R>(zp, (int64_t)ts * step + l);
+                pt.tile[2 * e] = cmulconj(w, v.s[0]);
+                pt.tile[2 * e + 1] = cmulconj(w, v.s[1]);
             }
             __syncthreads();
             dft_forward(pt.tile, ln, q.t1, q.t2, w2, pt.twt);
-            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
-                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
+            for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+                const int ts = fdiv(e, q.dW), l = e - ts * q.W;
                 const C w = pt.ew[ts];
-                const R re = w.x + base_s[l >> 1];
+                const R re = w.x + base_s[l];
                 const R ph = (R)1 / (re * re + w.y * w.y);
-                const C v = pt.tile[e];
-                acc.add(ph, v.x);
-                acc.add(ph, v.y);
-                pt.tile[e] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const C v = pt.tile[2 * e + s];
+                    acc.add(ph, v.x);
+                    acc.add(ph, v.y);
+                    pt.tile[2 * e + s] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
+                }
             }
             __syncthreads();
             dft_inverse(pt.tile, ln, q.t1, q.t2, w2, pt.twt);
-            for (int e = threadIdx.x; e < g.Nt * w2; e += blockDim.x) {
-                const int ts = fdiv(e, q.dw2), l = e - ts * w2;
-                if (l < live) zp[ts * step + l] = cmul(swapc(pt.tile[e]), pt.twist[ts]);
+            for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+                const int ts = fdiv(e, q.dW), l = e - ts * q.W;
+                const C w = pt.twist[ts];
+                It<R> v;
+                v.s[0] = cmul(swapc(pt.tile[2 * e]), w);
+                v.s[1] = cmul(swapc(pt.tile[2 * e + 1]), w);
+                if (l < live) st_it<R>(zp, (int64_t)ts * step + l, v);
             }
             __syncthreads();
         }
@@ -535,11 +573,11 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         const int L = g.L, RS = row_stride(L);
         each_round([&](int t0, int np) {
             const Lines rows{np, q.plane, 2 * L, q.d2L, 1, 2 * RS}, cols{np, q.plane, 2 * L, q.d2L, 1, 2};
-            for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
-                const int s = e >> 1, pl = fdiv(s, g.dLL), j = s - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * L;
-                pt.tile[pl * q.plane + (y * RS + xx) * 2 + (e & 1)] =
-                    swapc(z[(int64_t)(t0 + pl * tm.T) * g.LL * 2 + 2 * j + (e & 1)]);
-            }
+            each_site(t0, np, [&](int i, int at) {
+                const It<R> v = ld_it<R>(z, i);
+                pt.tile[at] = swapc(v.s[0]);
+                pt.tile[at + 1] = swapc(v.s[1]);
+            });
             __syncthreads();
             dft_inverse(pt.tile, cols, q.x1, q.x2, 2 * RS, pt.twx);
             dft_inverse(pt.tile, rows, q.x1, q.x2, 2, pt.twx);
@@ -577,7 +615,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             const R be = c.beta;
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 It<R> pc;
-                const It<R> o = d_item<R, true>(
+                const It<R> o = d_item<R, true, PRE>(
                     g, a.cf, phi, i, [&](int j) { return axpy_it<R>(be, ld_it<R>(pold, j), ld_it<R>(r, j)); }, &pc);
                 st_it<R>(pnew, i, pc);
                 st_it<R>(t, i, o);
@@ -585,7 +623,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             }
         } else {
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-                const It<R> o = d_item<R, true>(g, a.cf, phi, i, ldr(pold));
+                const It<R> o = d_item<R, true, PRE>(g, a.cf, phi, i, ldr(pold));
                 st_it<R>(t, i, o);
                 sq_it(acc, o);
             }
@@ -600,8 +638,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         acc = Sum2<R>();
         const R al = c.alpha;
         auto update = [&](int i) {
-            const It<R> q = d_item<R, false>(g, a.cf, phi, i, ldr(t));
-            st_it<R>(x, i, axpy_it<R>(al, ld_it<R>(pnew, i), ld_it<R>(x, i)));
+            const It<R> q = d_item<R, false, PRE>(g, a.cf, phi, i, ldr(t));
+            const int o = PRE && !kMixed ? from_bm(g, i) : i;   // FP64 iterates in the caller's x
+            st_it<R>(x, o, axpy_it<R>(al, ld_it<R>(pnew, i), ld_it<R>(x, o)));
             const It<R> rn = axpy_it<R>(-al, q, ld_it<R>(r, i));
             st_it<R>(r, i, rn);
             sq_it(acc, rn);
@@ -643,7 +682,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             // ---- reliable update: x64 += x, r = b - A x64 in FP64 ----
             if constexpr (kMixed) {
                 for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-                    const It<R> lo = ld_it<R>(x, i);
+                    const It<R> lo = ld_it<R>(x, in(i));
                     It<double> hi = ld_it<double>(x64, i);
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
@@ -651,20 +690,20 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                         hi.s[s].y += (double)lo.s[s].y;
                     }
                     st_it<double>(x64, i, hi);
-                    st_it<R>(x, i, It<R>{});
+                    st_it<R>(x, in(i), It<R>{});
                 }
                 if (!sync()) return false;
             }
-            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true>(g, a.cf64, g.phi64, i, ld64(x64)));
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
             if (!sync()) return false;
             Sum2<double> acc64;
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 const It<double> rd =
-                    axpy_it<double>(-1.0, d_item<double, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i));
+                    axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i));
                 It<R> rl;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rd.s[s].x, (R)rd.s[s].y);
-                st_it<R>(r, i, rl);
+                st_it<R>(r, in(i), rl);
                 sq_it(acc64, rd);
             }
             if (!sync_sum<CLU>(tm, c, red, acc64, [&](const Sum2<double>& sum) {
@@ -825,9 +864,10 @@ template <typename R> static size_t pre_tiles(TeamPre<R>* q, const Lat& lat, int
     const int room = most > tables ? (int)((most - tables) / sizeof(cplx<R>)) : 0;
     q->np = std::min(own, room / q->plane);
     // as many tau tiles as blocks
-    q->W = std::min({kTeamTau, (2 * LL + T - 1) / T, room / (2 * lat.Nt)});
-    if (q->np < 1 || q->W < 1) return 0;
+    q->W = std::min({kTeamTau, std::max(2, (2 * LL + T - 1) / T), room / (2 * lat.Nt)});
+    if (q->np < 1 || q->W < 2) return 0;
     q->dw2 = fast_div(2 * q->W);
+    q->dW = fast_div(q->W);
     q->tile = std::max(q->np * q->plane, lat.Nt * 2 * q->W);
     return tables + (size_t)q->tile * sizeof(cplx<R>);
 }

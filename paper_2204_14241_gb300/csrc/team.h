@@ -21,7 +21,7 @@ template <typename R> struct TeamPre {
     double scale;
     int x1, x2, t1, t2;
     int W;                     // sites of a tau tile
-    FastDiv d2L, dw2;          // by 2 L and 2 W
+    FastDiv d2L, dw2, dW;      // by 2 L, 2 W and W
     int plane, np;             // complex entries of a plane in the shared FFT tile, planes at a time
     int tile;                  // entries of the tile
 };
