@@ -15,7 +15,7 @@ template <> struct CT<float> { using T = float2; };
 template <> struct CT<double> { using T = double2; };
 template <typename R> using cplx = typename CT<R>::T;
 
-template <typename C> __host__ __device__ __forceinline__ C mk(double re, double im) {
+template <typename C, typename A, typename B> __host__ __device__ __forceinline__ C mk(A re, B im) {
     C c; c.x = re; c.y = im; return c;
 }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { a.x += b.x; a.y += b.y; return a; }

@@ -56,6 +56,14 @@ template <typename C, typename T> __device__ __forceinline__ C mulcs(C a, T c, T
     return o;
 }
 
+// a * (DIR i)^q: a product with these twiddles would keep its multiplications by 0
+template <int DIR, typename C> __device__ __forceinline__ C turn(C a, int q) {
+    q &= 3;
+    if (q == 0) return a;
+    if (q == 2) return mk<C>(-a.x, -a.y);
+    return (q == 1) == (DIR > 0) ? mk<C>(-a.y, a.x) : mk<C>(a.y, -a.x);
+}
+
 // Prime-size DFTs on registers: v[p] <- sum_q v[q] w^{pq}, w = e^{DIR 2 pi i / R}.
 template <int R, int DIR, typename C>
 __device__ __forceinline__ void bfly_prime(C* v) {
@@ -142,7 +150,9 @@ __device__ __forceinline__ void bfly_split(C* v) {
         bfly_prime<R2, DIR>(w);
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2)
-            u[n1 * R2 + k2] = (n1 * k2 == 0) ? w[k2] : mulcs(w[k2], W.c[(n1 * k2) % R], (T)DIR * W.s[(n1 * k2) % R]);
+            u[n1 * R2 + k2] = (4 * n1 * k2) % R == 0
+                                  ? turn<DIR>(w[k2], 4 * n1 * k2 / R)
+                                  : mulcs(w[k2], W.c[(n1 * k2) % R], (T)DIR * W.s[(n1 * k2) % R]);
     }
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) {
@@ -155,18 +165,49 @@ __device__ __forceinline__ void bfly_split(C* v) {
     }
 }
 
+// R = R1 * R2 with coprime factors: the index maps n = R2 a + R1 b and k = k1 (mod R1), k2 (mod R2) leave no
+// twiddles between the two steps (Good, 1958; Thomas, 1963).
+__host__ __device__ constexpr int crt(int k1, int R1, int k2, int R2) {
+    for (int k = 0; k < R1 * R2; ++k)
+        if (k % R1 == k1 && k % R2 == k2) return k;
+    return 0;
+}
+template <int R1, int R2, int DIR, typename C>
+__device__ __forceinline__ void bfly_coprime(C* v) {
+    constexpr int R = R1 * R2;
+    C u[R];
+#pragma unroll
+    for (int b = 0; b < R2; ++b) {
+        C w[R1];
+#pragma unroll
+        for (int a = 0; a < R1; ++a) w[a] = v[(R2 * a + R1 * b) % R];
+        bfly_prime<R1, DIR>(w);
+#pragma unroll
+        for (int a = 0; a < R1; ++a) u[a * R2 + b] = w[a];
+    }
+#pragma unroll
+    for (int a = 0; a < R1; ++a) {
+        C w[R2];
+#pragma unroll
+        for (int b = 0; b < R2; ++b) w[b] = u[a * R2 + b];
+        bfly_prime<R2, DIR>(w);
+#pragma unroll
+        for (int b = 0; b < R2; ++b) v[crt(a, R1, b, R2)] = w[b];
+    }
+}
+
 template <int R, int DIR, typename C>
 __device__ __forceinline__ void bfly(C* v) {
     if constexpr (R == 2 || R == 3 || R == 4 || R == 5 || R == 7) bfly_prime<R, DIR>(v);
-    else if constexpr (R == 6) bfly_split<2, 3, DIR>(v);
+    else if constexpr (R == 6) bfly_coprime<2, 3, DIR>(v);
     else if constexpr (R == 8) bfly_split<2, 4, DIR>(v);
     else if constexpr (R == 9) bfly_split<3, 3, DIR>(v);
-    else if constexpr (R == 10) bfly_split<2, 5, DIR>(v);
-    else if constexpr (R == 12) bfly_split<4, 3, DIR>(v);
-    else if constexpr (R == 14) bfly_split<2, 7, DIR>(v);
-    else if constexpr (R == 15) bfly_split<3, 5, DIR>(v);
+    else if constexpr (R == 10) bfly_coprime<2, 5, DIR>(v);
+    else if constexpr (R == 12) bfly_coprime<4, 3, DIR>(v);
+    else if constexpr (R == 14) bfly_coprime<2, 7, DIR>(v);
+    else if constexpr (R == 15) bfly_coprime<3, 5, DIR>(v);
     else if constexpr (R == 16) bfly_split<4, 4, DIR>(v);
-    else if constexpr (R == 20) bfly_split<4, 5, DIR>(v);
+    else if constexpr (R == 20) bfly_coprime<4, 5, DIR>(v);
     else static_assert(R == 2, "unsupported radix");
 }
 

@@ -111,7 +111,8 @@ struct BatchWork {
     void* metric = nullptr;     // transform table of the drift (metric.cu), every chain
     std::vector<char> hmetric;  // its host copy
     bool metric_ok = false;     // every chain's lattice has the real transforms
-    int maxL = 0, maxNt = 0;
+    int maxL = 0, maxNt = 0, tau_tiles = 0;
+    size_t tau_smem = 0;
     std::vector<BChainDev> hch; // host copy of the chain table of the current trajectory
 };
 
