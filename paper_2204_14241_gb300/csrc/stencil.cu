@@ -468,13 +468,19 @@ static ATile make_atile(const Lat& lat, int TX, int TY, int C) {
     return t;
 }
 
-// One launch of the fused A with the direction update on tile tl.
+// One launch of the fused A on tile tl, with the direction update (pnew) or, small complex64 fields, without.
 template <typename R>
 static void go_apply_A(hmc_ctx* ctx, const Lat& lat, const ATile& tl, int nrhs, const R* phi, const Site<R>* x,
                        Site<R>* y, double* part, const CgScalars* cgs, const Site<R>* pold, Site<R>* pnew) {
     const dim3 grid(tl.ntx * tl.nty, tl.nchunk, nrhs);
-    k_apply_A<R, true><<<grid, kAThreads, a_smem_bytes<R>(tl), ctx->stream>>>(lat, make_coef<R>(ctx->p), tl, phi, x, y,
-                                                                              part, cgs, pold, pnew);
+    auto go = [&](auto kernel) {
+        kernel<<<grid, kAThreads, a_smem_bytes<R>(tl), ctx->stream>>>(lat, make_coef<R>(ctx->p), tl, phi, x, y, part, cgs,
+                                                                      pold, pnew);
+    };
+    if constexpr (sizeof(R) == 4) {
+        if (!pnew) return go(k_apply_A<R, false>);
+    }
+    go(k_apply_A<R, true>);
 }
 
 // Times every valid (TX, TY, C) on the call's own buffers (the launch is idempotent: y, pnew
@@ -541,12 +547,16 @@ int launch_apply_A(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x,
             if (strip_supported(lat) && aligned32(y))
                 return launch_apply_A_strip(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
         }
-        return launch_A_two_pass<R>(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
+        // (a second launch costs the host 2 us, what the passes save only past some 8000 sites in complex64)
+        if (sizeof(R) == 8 || nrhs * lat.V > 8192)
+            return launch_A_two_pass<R>(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
     }
     static PerDevice attr;
     uint64_t bit;
     if (attr.pending(&bit)) {
         HMC_CUDA(ctx, cudaFuncSetAttribute(k_apply_A<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        if (sizeof(R) == 4)
+            HMC_CUDA(ctx, cudaFuncSetAttribute(k_apply_A<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
         attr.mark(bit);
     }
     const int prec = sizeof(R) == 8 ? HMC_FP64 : HMC_FP32;
