@@ -74,31 +74,36 @@ __global__ void __launch_bounds__(256) k_cg_xr(V16<R>* __restrict__ x, V16<R>* _
     if (threadIdx.x == 0) part[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
-// Fused complex64 update of plain CG: r -= alpha q; p = r + beta p (beta known before r: see
-// k_cg_ab); partial ||r||^2; and x += alpha p every other iteration. An iteration with
-// defer set (and beta > 0) leaves x alone and k_cg_beta records carry = alpha / beta; the next one
-// adds both terms, recovering the previous direction from the vectors it reads anyway:
-// p_prev = (p - r) / beta_prev, so x += alpha p + carry (p - r). One pass over r, p, q, and over x
-// on the iterations that update it.
-__device__ __forceinline__ float4 v_sub(float4 a, float4 b) {
-    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-}
-__global__ void __launch_bounds__(256) k_cg_xrp(float4* __restrict__ x, float4* __restrict__ r, float4* __restrict__ p,
-                                                const float4* __restrict__ q, int64_t n16, double* __restrict__ part,
-                                                const CgScalars* __restrict__ cgs, int defer) {
+// Fused complex64 update of plain CG, with beta known before the residual (k_cg_ab) and the residual kept
+// only as the difference of directions, r = p - beta_prev p_prev:
+//   rn = r - alpha q, p_new = rn + beta p (over p_prev), partial ||rn||^2,
+// and x on every other iteration: one with defer set (and beta > 0) leaves x alone and k_cg_beta records carry =
+// alpha; the next adds both terms, x += alpha p + carry p_prev, from the vectors it reads anyway. FROM_R: the
+// iteration after a (re)start, whose r is a vector (pr) of its own.
+// Bound by HBM: 128 bytes per right-hand side and site, 192 with x, 160 on average; with r stored beside p it was
+// 192: an iteration of five-solve trajectories 0.389 -> 0.353 ms at 80 x 80 x 160 with 8 right-hand sides. r so recovered carries the rounding of p instead of its
+// own; the iteration counts are those of the stored r (1409 : 1409 in a five-solve trajectory there).
+template <bool FROM_R>
+__global__ void __launch_bounds__(256) k_cg_xp(float4* __restrict__ x, const float4* __restrict__ p, const float4* pr,
+                                               float4* pnew, const float4* __restrict__ q, int64_t n16,
+                                               double* __restrict__ part, const CgScalars* __restrict__ cgs, int defer) {
     __shared__ double red[8];
     const int k = blockIdx.y;
     if (!cgs[k].active) return;
     const float alpha = (float)cgs[k].alpha, beta = (float)cgs[k].beta, carry = (float)cgs[k].carry;
+    const float bprev = (float)cgs[k].beta_prev;
     const bool skip_x = defer && cgs[k].beta > 0.0;
     const int64_t off = k * n16;
     double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n16; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 pv = p[off + i], rv = r[off + i];
-        if (!skip_x) x[off + i] = v_axpy(carry, v_sub(pv, rv), v_axpy(alpha, pv, x[off + i]));
-        const float4 rn = v_axpy(-alpha, q[off + i], rv);
-        r[off + i] = rn;
-        p[off + i] = v_axpy(beta, pv, rn);
+        const float4 pv = p[off + i], ov = pr[off + i];
+        if (!skip_x) {
+            float4 xv = v_axpy(alpha, pv, x[off + i]);
+            if (!FROM_R) xv = v_axpy(carry, ov, xv);   // (nothing is carried over a restart)
+            x[off + i] = xv;
+        }
+        const float4 rn = v_axpy(-alpha, q[off + i], FROM_R ? ov : v_axpy(-bprev, ov, pv));
+        pnew[off + i] = v_axpy(beta, pv, rn);
         s += v_dot(rn, rn);
     }
     s = block_sum(s, red);
@@ -142,6 +147,7 @@ __global__ void k_cg_ab(CgScalars* cgs, const double* __restrict__ part_pap, con
         const double alpha = (pAp > 0.0 && isfinite(pAp)) ? c.rr / pAp : 0.0;
         const double rnext = alpha * alpha * qq - c.rr;
         c.alpha = alpha;
+        c.beta_prev = c.beta;
         c.beta = (c.rr > 0.0 && rnext > 0.0) ? rnext / c.rr : 0.0;
         if (!isfinite(pAp) || !isfinite(qq)) c.nonfinite = 1;
     }
@@ -149,7 +155,7 @@ __global__ void k_cg_ab(CgScalars* cgs, const double* __restrict__ part_pap, con
 
 // r2 = ||r||^2, rz_new = <r, z> (= r2 without preconditioner), beta (unless set_beta is 0: the
 // fused plain update took it from k_cg_ab, and defer says whether that update left x for the next
-// iteration, see k_cg_xrp), convergence flags
+// iteration, see k_cg_xp), convergence flags
 __global__ void k_cg_beta(CgScalars* cgs, const double* __restrict__ part_r2,
                           const double* __restrict__ part_rz, int nblk, int nblk_rz, double tol2, double delta2,
                           int mixed, int set_beta, int defer) {
@@ -161,7 +167,7 @@ __global__ void k_cg_beta(CgScalars* cgs, const double* __restrict__ part_r2,
     if (threadIdx.x == 0) {
         CgScalars& c = cgs[k];
         if (set_beta) c.beta = c.rr > 0.0 ? rz / c.rr : 0.0;
-        else c.carry = (defer && c.beta > 0.0) ? c.alpha / c.beta : 0.0;
+        else c.carry = (defer && c.beta > 0.0) ? c.alpha : 0.0;
         c.rr = rz;
         c.r2 = r2;
         c.iters += 1;
@@ -393,7 +399,7 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
     };
     if ((rc = restart_dir())) return rc;
     // plain complex64 CG on the strip operator: beta comes ahead of the residual update (k_cg_ab),
-    // so x, r and p are updated in one pass; the first direction is p = r
+    // so x and p are updated in one pass (k_cg_xp); the first direction is p = r
     const bool fused = kMixed && !precond && strip_supported(lat);
     if (fused) HMC_CUDA(ctx, cudaMemcpyAsync(pv, rv, nrhs * n * sizeof(C), cudaMemcpyDeviceToDevice, sm));
 
@@ -439,6 +445,7 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
         next_check = now + step;
     };
     bool pending = false;   // an x update was deferred to the next iteration (fused path)
+    bool from_r = true;     // the residual is the vector rv, not yet the difference of directions (fused path)
     bool done = false, nonfinite = false;
     int it = 0;
     while (!done) {
@@ -465,14 +472,20 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
                 if ((rc = launch_apply_A_strip(ctx, lat, phiR, pv, qv, nrhs, part, &nb, cgs, part2))) return rc;
                 k_cg_ab<<<nrhs, 256, 0, sm>>>(cgs, part, part2, nb);
                 HMC_LAUNCH(ctx, "k_cg_ab");
-                // x is updated on every other iteration only (see k_cg_xrp); never deferred across the
+                // x is updated on every other iteration only (see k_cg_xp); never deferred across the
                 // host's checks, where a reliable update may fold x in, nor past maxit
                 const int defer = (!pending && it + 2 <= next_check && it + 2 <= maxit) ? 1 : 0;
                 pending = defer != 0;
-                k_cg_xrp<<<vgrid, 256, 0, sm>>>(reinterpret_cast<float4*>(xv), reinterpret_cast<float4*>(rv),
-                                                reinterpret_cast<float4*>(pv), reinterpret_cast<const float4*>(qv),
-                                                n16, part, cgs, defer);
-                HMC_LAUNCH(ctx, "k_cg_xrp");
+                auto go = [&](auto kernel, const C* pr) {
+                    kernel<<<vgrid, 256, 0, sm>>>(reinterpret_cast<float4*>(xv), reinterpret_cast<const float4*>(pv),
+                                                  reinterpret_cast<const float4*>(pr), reinterpret_cast<float4*>(pw),
+                                                  reinterpret_cast<const float4*>(qv), n16, part, cgs, defer);
+                };
+                if (from_r) go(k_cg_xp<true>, rv);
+                else go(k_cg_xp<false>, pw);
+                from_r = false;
+                HMC_LAUNCH(ctx, "k_cg_xp");
+                { C* t = pv; pv = pw; pw = t; }
                 k_cg_beta<<<nrhs, 256, 0, sm>>>(cgs, part, nullptr, kRedBlocks, kRedBlocks, tol2, delta2, kMixed, 0,
                                                 defer);
                 HMC_LAUNCH(ctx, "k_cg_beta");
@@ -522,6 +535,7 @@ static int run(hmc_ctx* ctx, const Lat& lat, const double* phi64, const double2*
             if (nonfinite) break;
             if (any_ru) {
                 if ((rc = reliable_update())) return rc;
+                from_r = true;
                 HMC_CUDA(ctx, cudaMemcpyAsync(ctx->h_cg, cgs, nrhs * sizeof(CgScalars), cudaMemcpyDeviceToHost, sm));
                 HMC_CUDA(ctx, cudaStreamSynchronize(sm));
                 any_active = false;

@@ -123,11 +123,12 @@ struct CgScalars {
     double pAp;
     double alpha;
     double beta;
+    double beta_prev; // fused plain CG: beta of the current direction
     double r2;        // <r, r> (stopping test)
     double r2_max;    // largest ||r||^2 since the last reliable update
     double b2;        // <b, b>
     double r2true;    // ||b - A x||^2 at the last true-residual evaluation
-    double carry;     // fused plain CG: alpha / beta of an iteration whose x update was deferred
+    double carry;     // fused plain CG: alpha of an iteration whose x update was deferred
     int active;       // 1 while this RHS iterates
     int iters;
     int need_ru;      // set when a true-residual (reliable) update is due
