@@ -374,7 +374,7 @@ template <> struct TauSplit<80> { static constexpr int N1 = 10, N2 = 8; };
 template <> struct TauSplit<160> { static constexpr int N1 = 16, N2 = 10; };
 #define HMC_TAU2_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32) X(40) X(48) X(64) X(80) X(160)
 
-constexpr int kTauLines = 16, kTauThreads = 256;
+constexpr int kTauLines = 16, kTauThreads = 160;
 
 // The tau pass in three steps over a shared tile [N][16] of one right-hand side's 16
 // consecutive inner indices (4 sites x 4 components), N = N1 * N2, loaded whole first:
@@ -432,9 +432,11 @@ __device__ __forceinline__ void tau_outer(float2* __restrict__ sm, float2* __res
 // digit-permuted order of the split; A.cosk the cos k table in the order of the x and y
 // positions. A.part (optional): per block sum P-hat |y-hat|^2 / N (= <y_in, P y_in> when y_in is
 // the unitary (x, y) transform of a vector).
-// Resident blocks per SM: six (40 registers) for the short lengths; five (48 registers) from N = 80
-// on, where the 16-point DFTs of the middle step would spill at 40.
-constexpr int tau_min_blocks(int N) { return N >= 80 ? 5 : 6; }
+// 160 threads: the middle step of N = 160 and the outer ones of N = 80 have 160 tasks, and more, smaller blocks
+// overlap their loads, steps and stores better (129 us against 138 with five blocks of 256 at 80 x 80 x 160
+// with 8 right-hand sides). Eight blocks an SM (48 registers) from N = 80 on, where the 16-point DFTs of the middle
+// step would spill at 40; nine below.
+constexpr int tau_min_blocks(int N) { return N >= 80 ? 8 : 9; }
 template <int N>
 __global__ void __launch_bounds__(kTauThreads, tau_min_blocks(N)) k_tau(FftcArgs A) {
     constexpr int N1 = TauSplit<N>::N1, N2 = TauSplit<N>::N2;
