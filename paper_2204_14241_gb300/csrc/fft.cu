@@ -531,23 +531,28 @@ template <typename R>
 int launch_precond(hmc_ctx* ctx, const Lat& lat, const cplx<R>* x, cplx<R>* y, int nrhs, cplx<R>* scratch) {
     const int L = lat.L, Nt = lat.Nt;
     int rc;
-    if constexpr (sizeof(R) == 4) {
-        // the (x, y) passes and tau pass that PCG runs, with the (band-major) spectrum in scratch:
-        // those passes do not run in place
-        const PcTables* pt = get_pc(ctx, L, Nt);
-        const int64_t n = (int64_t)nrhs * Nt * L * L * 4;
-        auto apart = [n](const void* a, const void* b) {
-            const cplx<R>* u = static_cast<const cplx<R>*>(a);
-            const cplx<R>* v = static_cast<const cplx<R>*>(b);
-            return u + n <= v || v + n <= u;
-        };
-        if (pt && pt->cosk32_xy && fftc_can(Nt, 4 * (int64_t)L * L) && scratch && apart(scratch, x) &&
-            apart(scratch, y)) {
-            cplx<R>* mid = scratch;
-            if ((rc = fftc_xy_apply(ctx, lat, x, mid, nrhs, -1, nullptr))) return rc;
-            if ((rc = fftc_precond_tau(ctx, lat, mid, nrhs, nullptr, pt, pt->cosk32_xy, nullptr, nullptr, true)))
-                return rc;
-            return fftc_xy_apply(ctx, lat, mid, y, nrhs, +1, nullptr);
+    // the routes with the spectrum in scratch do not run in place
+    const int64_t n = (int64_t)nrhs * Nt * L * L * 4;
+    auto apart = [n](const cplx<R>* u, const cplx<R>* v) { return u + n <= v || v + n <= u; };
+    if (scratch && apart(scratch, x) && apart(scratch, y)) {
+        if constexpr (sizeof(R) == 4) {
+            // the (x, y) passes and tau pass that PCG runs, with the (band-major) spectrum in scratch
+            const PcTables* pt = get_pc(ctx, L, Nt);
+            if (pt && pt->cosk32_xy && fftc_can(Nt, 4 * (int64_t)L * L)) {
+                if ((rc = fftc_xy_apply(ctx, lat, x, scratch, nrhs, -1, nullptr))) return rc;
+                if ((rc = fftc_precond_tau(ctx, lat, scratch, nrhs, nullptr, pt, pt->cosk32_xy, nullptr, nullptr, true)))
+                    return rc;
+                return fftc_xy_apply(ctx, lat, scratch, y, nrhs, +1, nullptr);
+            }
+        }
+        // by planes against axis by axis, complex128: 9.15 against 13.92 ms at 80 x 80 x 160 with 8 right-hand sides, 45
+        // against 111 us at 16 x 16 x 32 with 2. complex64: 87 against 320 us at 36 x 36 x 70 with 8, 14 against 62
+        // at 10 x 10 x 20; where both axis lengths are compiled 14 against 21 at 4 x 4 x 8, 28.7 against 30.7 at
+        // 32 x 32 x 64 with 2, but 219 against 153 at 64 x 64 x 128 with 4
+        if (!(sizeof(R) == 4 && n > 4 * 131072 && fftc_can(L, 4) && fftc_can(Nt, 4 * (int64_t)L * L))) {
+            bool done;
+            rc = precond_planes<R>(ctx, lat, x, y, nrhs, scratch, &done);
+            if (rc || done) return rc;
         }
     }
     if ((rc = fft_axis<R>(ctx, y, (int64_t)nrhs * Nt * L, L, 4, -1, x))) return rc;

@@ -1,0 +1,33 @@
+"""The preconditioner by planes (complex128; complex64 lattices without compiled passes) against the oracle: extents
+of one and two transform factors, odd numbers of slices, tau tiles with a ragged end, blocks of several planes with
+a short last one, and the fallbacks (x == y is the same route; 125 slices have no split and take the axis kernels).
+Bounds: test_gpu_parity's operator bounds, 1e-12 (FP64) and 1e-5 (FP32)."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import solver
+from oracle.model import Params
+from paper_2204_14241_gb300 import inputs as I, presets
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("L,Nt,k", [(2, 2, 1), (2, 3, 3), (4, 6, 1), (6, 5, 2), (10, 9, 1), (14, 7, 3), (18, 15, 2),
+                                    (20, 40, 1), (6, 125, 1), (30, 12, 1), (36, 21, 1)])
+def test_planes(L, Nt, k, dtype):
+    from paper_2204_14241_gb300.hmc import Context
+    tol = 1e-5 if dtype == torch.complex64 else 1e-12
+    ctx = Context(L, Nt, nrhs_max=k, **presets.baseline())
+    P = Params(L=L, Nt=Nt, **presets.baseline())
+    x = torch.from_numpy(I.fermion_noise(7, k, L, Nt)).cuda().to(dtype)
+    y = torch.full_like(x, float("nan"))
+    ctx.apply_precond(x, out=y)
+    paper = lambda a: [I.to_paper_fermion(v) for v in a.cpu().numpy().astype(np.complex128)]
+    for a, b in zip(paper(y), paper(x)):
+        r = solver.apply_precond(P, b)
+        assert np.linalg.norm(a - r) < tol * np.linalg.norm(r)
+    ctx.apply_precond(x, out=x)
+    assert torch.equal(x, y)
