@@ -1011,10 +1011,17 @@ static int make_plan(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond, TeamPr
             const int tasks = 2 * lat.Nt, avail = cap / nrhs;
             if (avail < 1) return HMC_OK;
             const int rounds = (tasks + avail - 1) / avail;
-            // one block an SM and a last round that leaves SMs idle: 1162 us an iteration at 60 x 60 x 120 in FP64,
-            // 1103 by the separate kernels
-            if (most == kTeamSmem && 5 * (int64_t)tasks < 4 * (int64_t)rounds * avail) return HMC_OK;
             plan->T = (tasks + rounds - 1) / rounds;
+            // More blocks than planes share the other phases: an SM each where the planes leave SMs idle, all that fit
+            // where planes double up on some SMs (8 of 152 at 40 x 40 x 80, for which every phase waited), as long
+            // as a block's threads (FP64: two warps) have an item each. Microseconds an iteration, a block per plane :
+            // now: complex64 34.0 : 30.7 at 40 x 40 x 40, 40.1 : 37.9 at 40 x 40 x 80, 31.0 : 26.8 at 20 x 20 x 40 with
+            // 4 right-hand sides, FP64 76.8 : 67.7 at 24 x 24 x 48, 1052 (separate kernels) : 725 at 60 x 60 x 120; with
+            // less than an item a thread 20.3 : 21.1 at 20 x 20 x 40 with 2.
+            const int64_t most_T = n / (sizeof(R) == 8 ? 64 : 256);
+            const int alone = ctx->num_sms / nrhs;
+            if (tasks <= alone) plan->T = std::max<int>(tasks, (int)std::min<int64_t>(alone, most_T));
+            else if (avail <= most_T) plan->T = avail;
             plan->smem = pre_tiles<R>(pre, lat, plan->T, most);
             return HMC_OK;
         }
@@ -1120,14 +1127,14 @@ static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2*
 //                  152 : 137 with 2 at 80 x 80 x 160: past about a million sites the strip operator's traffic
 //                  counts; other lattices 394 : 412 at 70 x 70 x 140 with 8
 //  CG, complex128  2991 : 4300 at 80 x 80 x 160 with 8
-//  PCG, complex64  lattices with compiled FFT passes 82 : 93 at 40 x 40 x 80 with 3, but 229 : 182 with 8; others
-//                  (no compiled length) 1316 : 2805 at 70 x 70 x 140 with 8
-//  PCG, complex128 3441 : 4328 at 64 x 64 x 128 with 4
+//  PCG, complex64  lattices with compiled FFT passes 81 : 119 at 64 x 64 x 128, 136 : 168 at 48 x 48 x 96 with 4, but
+//                  167 : 157 at 40 x 40 x 80 with 8; others (no compiled length) 115 : 448 at 36 x 36 x 70 with 8
+//  PCG, complex128 2148 : 2461 at 80 x 80 x 160
 static bool worth_it(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond) {
     const int64_t sites = (int64_t)nrhs * lat.V;
     if (sites > (int64_t)1 << 23) return false;   // the largest measured
     if (ctx->p.solver_mode != HMC_SOLVER_MIXED) return true;
-    if (precond) return sites <= 400000 || !(fftc_supported(lat.L) && fftc_can(lat.Nt, 4 * (int64_t)lat.L * lat.L));
+    if (precond) return sites <= 900000 || !(fftc_supported(lat.L) && fftc_can(lat.Nt, 4 * (int64_t)lat.L * lat.L));
     return sites <= 1250000 || !strip_supported(lat);
 }
 
