@@ -681,7 +681,9 @@ static int twisted_fourier(hmc_ctx* ctx, const Lat& lat, const double2* src, dou
     const int64_t n = 4 * lat.V * (int64_t)nrhs, slice = 4 * (int64_t)L * L;
     const unsigned nb = (unsigned)((n + 255) / 256);
     const int dir = inverse ? +1 : -1;
-    int rc;
+    bool done;
+    int rc = twisted_planes(ctx, lat, src, dst, nrhs, inverse, ctx->d_q64, &done);
+    if (rc || done) return rc;
     if (!inverse) {
         if (src != dst) HMC_CUDA(ctx, cudaMemcpyAsync(dst, src, n * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream));
         k_twist<<<nb, 256, 0, ctx->stream>>>(dst, pt->twist, Nt, slice, n, -1);

@@ -309,6 +309,9 @@ int launch_precond(hmc_ctx* ctx, const Lat& lat, const cplx<R>* x, cplx<R>* y, i
 // lattice rules that out
 template <typename R>
 int precond_planes(hmc_ctx* ctx, const Lat& lat, const cplx<R>* x, cplx<R>* y, int nrhs, cplx<R>* scratch, bool* done);
+// dst = F~ src (inverse) or F~^* src by planes, through scratch (apart from both; dst may be src)
+int twisted_planes(hmc_ctx* ctx, const Lat& lat, const double2* src, double2* dst, int nrhs, int inverse, double2* scratch,
+                   bool* done);
 // x += alpha p, r -= alpha q, z = P r for every active RHS with partial sums of ||r||^2 and
 // <r, z> (rows of *nblk_out entries per RHS in part_r2, of *nblk_rz_out in part_rz).
 template <typename R>

@@ -12,6 +12,7 @@
 // against 0.320 at 36 x 36 x 70 with 8 in complex64. Re K-hat keeps the order of operations of the axis kernels:
 // as e^{i w} - (1 + ...) its cancellation at the smallest modes made errors up to three times as large.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "dft_smem.cuh"
@@ -33,6 +34,7 @@ template <typename R> struct PreArgs {
     int L, Nt, LL;
     int x1, x2, t1, t2;
     int np, planes;            // planes of a block, planes in all (right-hand sides x slices x groups)
+    int swap;                  // forward passes of complex128: re and im exchanged on the way in
     int W;                     // entries of a group's plane in a tau tile
     FastDiv dL, dLL, dCL, dW, dCW;   // by L, L^2, components x L, W, components x W
 };
@@ -64,7 +66,7 @@ __global__ void __launch_bounds__(256, 2) k_pre_xy(const __grid_constant__ PreAr
             tile[at] = FWD ? mk<C>(u.x, u.y) : mk<C>(u.y, u.x);
             tile[at + 1] = FWD ? mk<C>(u.z, u.w) : mk<C>(u.w, u.z);
         } else {
-            tile[at] = FWD ? *v : swapc(*v);
+            tile[at] = FWD && !a.swap ? *v : swapc(*v);
         }
     });
     __syncthreads();
@@ -176,44 +178,103 @@ __global__ void __launch_bounds__(256, 2) k_pre_tau(const __grid_constant__ PreA
     }
 }
 
+// The tau transform of the twisted Fourier transforms of complex128 vectors (few and small beside the solve between
+// them: launches and passes count), from the spectrum of W sites of all four components to the site layout in the order of frequencies. inverse: times the twist behind the transform, whose
+// input k_pre_xy has exchanged, else its conjugate before.
+__global__ void __launch_bounds__(256, 2) k_twisted_tau(const __grid_constant__ PreArgs<double> a, int tiles, int inverse) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int L = a.L, Nt = a.Nt, LL = a.LL, W = a.W;
+    const int k = blockIdx.x / tiles, j0 = (blockIdx.x - k * tiles) * W, live = min(W, LL - j0);
+    double2 *tile = reinterpret_cast<double2*>(smem), *tw = tile + Nt * 4 * W, *twist = tw + Nt;
+    for (int i = threadIdx.x; i < Nt; i += blockDim.x) {
+        tw[i] = __ldg(a.twt + i);
+        twist[i] = __ldg(a.twist + i);
+    }
+    __syncthreads();
+    const double2* z = a.src + (int64_t)k * Nt * 4 * LL + j0;
+    for (int e = threadIdx.x; e < Nt * 4 * W; e += blockDim.x) {
+        const int row = fdiv(e, a.dW), l = e - row * W;   // row = 4 t + component
+        const double2 v = l < live ? z[(int64_t)row * LL + l] : make_double2(0.0, 0.0);
+        tile[e] = inverse ? v : cmulconj(twist[row >> 2], v);
+    }
+    __syncthreads();
+    dft_forward(tile, Lines{1, 0, 4 * W, a.dCW, 1, 2}, a.t1, a.t2, 4 * W, tw);
+    double2* out = a.dst + (int64_t)k * Nt * 4 * LL;
+    for (int e = threadIdx.x; e < Nt * 4 * W; e += blockDim.x) {
+        const int q = e >> 2, c = e & 3, p = fdiv(q, a.dW), l = q - p * W;
+        if (l >= live) continue;
+        const int j = j0 + l, y = fdiv(j, a.dL), x = j - y * L, n = dft_freq(p, a.t1, a.t2);
+        const double2 v = tile[(4 * p + c) * W + l], u = cscale(inverse ? cmul(swapc(v), twist[n]) : v, a.scale);
+        out[((int64_t)n * LL + dft_freq(y, a.x1, a.x2) * L + dft_freq(x, a.x1, a.x2)) * 4 + c] = u;
+    }
+}
+
 // ---- host --------------------------------------------------------------------------------------------
+struct XyLaunch {
+    unsigned blocks;
+    int threads;
+    size_t smem;
+};
+// Geometry, tables and the (x, y) passes' launch; false where the extents have no split or a plane does not fit.
+template <typename R> static bool plane_args(hmc_ctx* ctx, const Lat& lat, int nrhs, PreArgs<R>* a, XyLaunch* xy) {
+    constexpr int NC = kComp<R>, G = 4 / NC;
+    const FftPlan *px = get_plan(ctx, lat.L), *pt = get_plan(ctx, lat.Nt);
+    const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
+    if (!px || !pt || !pc || !dft_split(lat.L, &a->x1, &a->x2) || !dft_split(lat.Nt, &a->t1, &a->t2)) return false;
+    const int L = lat.L, Nt = lat.Nt, LL = L * L;
+    const int64_t planes = (int64_t)nrhs * Nt * G;
+    const size_t psize = (size_t)L * (L | 1) * NC * sizeof(cplx<R>), ptab = L * sizeof(cplx<R>);
+    if (psize + ptab > kPSmem || planes > (1 << 30)) return false;
+    // enough planes for a block's threads to have a site each, but not fewer blocks than two an SM
+    a->np = (int)std::max<int64_t>(1, std::min<int64_t>({(256 + LL - 1) / LL, planes / (2 * ctx->num_sms), (int64_t)((kPSmem / 2 - ptab) / psize)}));
+    a->planes = (int)planes;
+    a->L = L;
+    a->Nt = Nt;
+    a->LL = LL;
+    a->dL = fast_div(L);
+    a->dLL = fast_div(LL);
+    a->dCL = fast_div(NC * L);
+    if constexpr (sizeof(R) == 4) {
+        a->twx = px->tw32; a->twt = pt->tw32; a->twist = pc->twist32;
+    } else {
+        a->twx = px->tw64; a->twt = pt->tw64; a->twist = pc->twist;
+    }
+    a->cosk = pc->cosk;
+    a->eitw = pc->eitw;
+    xy->blocks = (unsigned)((planes + a->np - 1) / a->np);
+    xy->threads = a->np * LL >= 256 ? 256 : 128;
+    xy->smem = a->np * psize + ptab;
+    return true;
+}
+template <typename R> static int plane_attr(hmc_ctx* ctx) {
+    static PerDevice attr;
+    uint64_t bit;
+    if (!attr.pending(&bit)) return HMC_OK;
+    for (const void* f : {(const void*)k_pre_xy<R, true>, (const void*)k_pre_xy<R, false>, (const void*)k_pre_tau<R>})
+        HMC_CUDA(ctx, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmem));
+    if (sizeof(R) == 8)
+        HMC_CUDA(ctx, cudaFuncSetAttribute(k_twisted_tau, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmem));
+    attr.mark(bit);
+    return HMC_OK;
+}
+
 template <typename R>
 int precond_planes(hmc_ctx* ctx, const Lat& lat, const cplx<R>* x, cplx<R>* y, int nrhs, cplx<R>* scratch, bool* done) {
     *done = false;
     constexpr int NC = kComp<R>, G = 4 / NC;
-    const FftPlan *px = get_plan(ctx, lat.L), *pt = get_plan(ctx, lat.Nt);
-    const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
     PreArgs<R> a{};
-    if (!scratch || !px || !pt || !pc || !dft_split(lat.L, &a.x1, &a.x2) || !dft_split(lat.Nt, &a.t1, &a.t2)) return HMC_OK;
-    const int L = lat.L, Nt = lat.Nt, LL = L * L;
-    const int64_t planes = (int64_t)nrhs * Nt * G;
-    const size_t psize = (size_t)L * (L | 1) * NC * sizeof(cplx<R>), ptab = L * sizeof(cplx<R>);
+    XyLaunch xy;
+    if (!scratch || !plane_args<R>(ctx, lat, nrhs, &a, &xy)) return HMC_OK;
+    const int Nt = lat.Nt, LL = a.LL;
     const size_t col = (size_t)(Nt * NC) * sizeof(cplx<R>) + sizeof(double), ttab = (size_t)Nt * (2 * sizeof(cplx<R>) + sizeof(double) + sizeof(R));
-    if (psize + ptab > kPSmem || 2 * col + ttab > kPSmem / 2 || planes > (1 << 30)) return HMC_OK;
-    // enough planes for a block's threads to have a site each, but not fewer blocks than two an SM
-    const int64_t slots = 2 * ctx->num_sms;
-    a.np = (int)std::max<int64_t>(1, std::min<int64_t>({(256 + LL - 1) / LL, planes / slots, (int64_t)((kPSmem / 2 - ptab) / psize)}));
-    a.planes = (int)planes;
+    if (2 * col + ttab > kPSmem / 2) return HMC_OK;
     // tau tiles of 256-byte rows, narrower where they would leave SMs idle
     a.W = std::min<int>(16, (int)((kPSmem / 2 - ttab) / col));
-    while (a.W > 4 && (int64_t)nrhs * G * ((LL + a.W - 1) / a.W) < slots) a.W /= 2;
+    while (a.W > 4 && (int64_t)nrhs * G * ((LL + a.W - 1) / a.W) < 2 * ctx->num_sms) a.W /= 2;
     a.W = std::max(2, std::min(a.W, LL));
     const int tiles = (LL + a.W - 1) / a.W;
-    a.L = L;
-    a.Nt = Nt;
-    a.LL = LL;
-    a.dL = fast_div(L);
-    a.dLL = fast_div(LL);
-    a.dCL = fast_div(NC * L);
     a.dW = fast_div(a.W);
     a.dCW = fast_div(NC * a.W);
-    if constexpr (sizeof(R) == 4) {
-        a.twx = px->tw32; a.twt = pt->tw32; a.twist = pc->twist32;
-    } else {
-        a.twx = px->tw64; a.twt = pt->tw64; a.twist = pc->twist;
-    }
-    a.cosk = pc->cosk;
-    a.eitw = pc->eitw;
     a.dtau = ctx->p.dtau;
     for (int s = 0; s < 2; ++s) {
         a.mu[s] = ctx->p.mu[s];
@@ -221,30 +282,53 @@ int precond_planes(hmc_ctx* ctx, const Lat& lat, const cplx<R>* x, cplx<R>* y, i
         a.ty[s] = 2.0 * ctx->p.t_v[s];
     }
     a.scale = (R)(1.0 / ((double)LL * Nt));   // the unnormalised transforms both ways
-    static PerDevice attr;
-    uint64_t bit;
-    if (attr.pending(&bit)) {
-        for (const void* f : {(const void*)k_pre_xy<R, true>, (const void*)k_pre_xy<R, false>, (const void*)k_pre_tau<R>})
-            HMC_CUDA(ctx, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmem));
-        attr.mark(bit);
-    }
+    int rc;
+    if ((rc = plane_attr<R>(ctx))) return rc;
     *done = true;
-    const unsigned blocks = (unsigned)((planes + a.np - 1) / a.np);
-    const size_t psm = a.np * psize + ptab;
-    const int thr = a.np * LL >= 256 ? 256 : 128;
     a.src = x;
     a.dst = scratch;
-    k_pre_xy<R, true><<<blocks, thr, psm, ctx->stream>>>(a);
+    k_pre_xy<R, true><<<xy.blocks, xy.threads, xy.smem, ctx->stream>>>(a);
     HMC_LAUNCH(ctx, "k_pre_xy");
     k_pre_tau<R><<<(unsigned)(nrhs * G * tiles), 256, a.W * col + ttab, ctx->stream>>>(a, tiles);
     HMC_LAUNCH(ctx, "k_pre_tau");
     a.src = scratch;
     a.dst = y;
-    k_pre_xy<R, false><<<blocks, thr, psm, ctx->stream>>>(a);
+    k_pre_xy<R, false><<<xy.blocks, xy.threads, xy.smem, ctx->stream>>>(a);
     HMC_LAUNCH(ctx, "k_pre_xy");
     return HMC_OK;
 }
 template int precond_planes<float>(hmc_ctx*, const Lat&, const float2*, float2*, int, float2*, bool*);
 template int precond_planes<double>(hmc_ctx*, const Lat&, const double2*, double2*, int, double2*, bool*);
+
+// dst = F~ src (inverse, its order as printed: T times the inverse unitary DFT) or F~^* src, through scratch. Two
+// launches for four or five of fft.cu's axis kernels: green_estimate with 8 probes 2.04 -> 2.01 ms at 16 x 16 x 32, with
+// one 0.362 -> 0.343 at 4 x 4 x 8.
+int twisted_planes(hmc_ctx* ctx, const Lat& lat, const double2* src, double2* dst, int nrhs, int inverse, double2* scratch,
+                   bool* done) {
+    *done = false;
+    PreArgs<double> a{};
+    XyLaunch xy;
+    if (!plane_args<double>(ctx, lat, nrhs, &a, &xy)) return HMC_OK;
+    a.W = std::min(4, a.LL);
+    const int tiles = (a.LL + a.W - 1) / a.W;
+    const size_t smem = (size_t)lat.Nt * (4 * a.W + 2) * sizeof(double2);
+    if (smem > kPSmem) return HMC_OK;
+    int rc;
+    if ((rc = plane_attr<double>(ctx))) return rc;
+    *done = true;
+    a.dW = fast_div(a.W);
+    a.dCW = fast_div(4 * a.W);
+    a.swap = inverse;
+    a.scale = 1.0 / std::sqrt((double)a.LL * lat.Nt);
+    a.src = src;
+    a.dst = scratch;
+    k_pre_xy<double, true><<<xy.blocks, xy.threads, xy.smem, ctx->stream>>>(a);
+    HMC_LAUNCH(ctx, "k_pre_xy");
+    a.src = scratch;
+    a.dst = dst;
+    k_twisted_tau<<<(unsigned)(nrhs * tiles), 256, smem, ctx->stream>>>(a, tiles, inverse);
+    HMC_LAUNCH(ctx, "k_twisted_tau");
+    return HMC_OK;
+}
 
 }  // namespace hmc

@@ -1,4 +1,4 @@
-"""The preconditioner by planes (complex128; complex64 lattices without compiled passes) against the oracle: extents
+"""The preconditioner and the twisted Fourier transforms by planes (complex128; complex64 lattices without compiled passes) against the oracle: extents
 of one and two transform factors, odd numbers of slices, tau tiles with a ragged end, blocks of several planes with
 a short last one, and the fallbacks (x == y is the same route; 125 slices have no split and take the axis kernels).
 Bounds: test_gpu_parity's operator bounds, 1e-12 (FP64) and 1e-5 (FP32)."""
@@ -31,3 +31,26 @@ def test_planes(L, Nt, k, dtype):
         assert np.linalg.norm(a - r) < tol * np.linalg.norm(r)
     ctx.apply_precond(x, out=x)
     assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("L,Nt,k", [(2, 3, 1), (4, 6, 3), (6, 5, 2), (14, 15, 1), (10, 49, 1), (18, 8, 2)])
+def test_twisted_transforms(L, Nt, k):
+    """green_estimate at g = 0, r-independent: D is diagonal under F~, so the estimate with Rademacher probes is exactly
+    1 / K-hat per Fourier mode up to the solver's tolerance (1e-12 here; the smallest |K-hat|^2 in play is above 1e-3)."""
+    from paper_2204_14241_gb300.hmc import Context
+    kw = dict(presets.baseline())
+    kw["g"] = 0.0
+    ctx = Context(L, Nt, nrhs_max=k, cg_tol=1e-12, **kw)
+    g = torch.Generator().manual_seed(5)
+    v = (torch.randint(0, 2, (k, Nt, L, L, 2, 2), generator=g) * 2 - 1).to(torch.complex128).cuda()
+    phi = torch.zeros((3, Nt, L, L), dtype=torch.float64, device="cuda")
+    out = ctx.green_estimate(phi, v, precond=True)[0].cpu().numpy().reshape(Nt, L, L, 2, 2)
+    w = (2 * np.arange(Nt) + 1) * np.pi / Nt
+    c = np.cos(2 * np.pi * np.arange(L) / L)
+    dt, mu, th, tv = (kw[n] for n in ("dtau", "mu", "t_h", "t_v"))
+    for a in range(2):
+        eps = mu[a] + 2 * th[a] * c[None, None, :] + 2 * tv[a] * c[None, :, None]
+        K = np.exp(1j * w)[:, None, None] - 1 - dt * eps
+        assert np.abs(K).min() > 0.03
+        for s in range(2):
+            assert np.abs(out[..., a, s] - 1 / K).max() < 1e-8 * np.abs(1 / K).max()
