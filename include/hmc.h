@@ -80,7 +80,8 @@ typedef struct {
                            + 4 X_{n-2} - X_{n-3}; ...; lower degree while fewer solutions exist),
                            m FP64 vectors of workspace. The same stopping test applies in every
                            case. */
-    int autotune;       /* 0: tile shapes of the fused A kernel from a fixed rule (default; the
+    int autotune;       /* 0: tile shapes of the fused A kernel (complex64 up to 8192 sites in all, and
+                           solves that fold the direction into it) from a fixed rule (default; the
                            reduction order, hence every bit of the results, is reproducible);
                            1: on first use per (L, Nt, nrhs, precision) time the valid tile and
                            time-chunk shapes on the call's own buffers and keep the fastest */
@@ -91,8 +92,9 @@ typedef struct {
                               barrier that nothing completes, so it always gives up */
     int batch_chains;   /* nonzero: trajectory() advances all chains together and every force
                            evaluation solves all (chain, RHS) pairs in one persistent cooperative
-                           launch (mixed solver mode only; CG without the preconditioner; grid
-                           barriers bounded by wait_spin_limit microseconds, default 2 s) */
+                           launch, a team of blocks per pair (mixed solver mode only; CG without the
+                           preconditioner; the teams' barriers, as those of single-chain solves in
+                           one launch, bounded by wait_spin_limit microseconds, default 2 s) */
     int batch_graph;    /* with batch_chains: the leapfrog part of a trajectory (every force
                            evaluation, kick and drift of all chains) runs as one CUDA graph,
                            captured on first use and replayed while n_leap, eps, the chains'
@@ -135,7 +137,8 @@ const char* hmc_last_error(const hmc_ctx* ctx);   /* ctx may be NULL (global las
 int apply_M(hmc_ctx* ctx, int chain, int prec, const void* phi, const void* x, void* y,
             int dagger, int nrhs);
 
-/* y = A x = D (D^dagger x) (Eq. linsys), fused in one pass. If norm2 is not NULL it
+/* y = A x = D (D^dagger x) (Eq. linsys): one fused launch for complex64 on lattices with a strip
+ * kernel or of up to 8192 sites, two passes through workspace otherwise. If norm2 is not NULL it
  * receives (host, nrhs doubles) ||D^dagger x_k||^2 = x_k^dagger A x_k. */
 int apply_MdagM(hmc_ctx* ctx, int chain, int prec, const void* phi, const void* x, void* y,
                 int nrhs, double* norm2);
@@ -153,9 +156,8 @@ int apply_MdagM(hmc_ctx* ctx, int chain, int prec, const void* phi, const void* 
  *   HMC_FP64 or HMC_FP32 (as for apply_MdagM); phi, x, y: device, layouts as for apply_MdagM,
  *   16-byte aligned, the byte range of y disjoint from those of x and phi; 1 <= nrhs <= 65535
  *   (<= 64 when norm2 is requested); cuda_stream: cudaStream_t or NULL for the default stream.
- * It always runs the generic fused kernel (the one apply_MdagM uses for FP64 and for L not a
- * multiple of 16), never the complex64 strip kernel, so for complex64 with L a multiple of 16
- * it is slower than apply_MdagM; the results agree to rounding.
+ * It always runs the generic fused kernel, which forms D^dagger x again around every tile and needs
+ * no workspace, so on larger lattices it is slower than apply_MdagM; the results agree to rounding.
  * Set-up: the first call on each device (with that device current) looks up the device
  * address of the scratch array (cudaGetSymbolAddress); make that first call before any
  * stream capture. Every call on a device shares the one array and overwrites it, and each

@@ -81,8 +81,9 @@ __global__ void __launch_bounds__(256) k_cg_xr(V16<R>* __restrict__ x, V16<R>* _
 // alpha; the next adds both terms, x += alpha p + carry p_prev, from the vectors it reads anyway. FROM_R: the
 // iteration after a (re)start, whose r is a vector (pr) of its own.
 // Bound by HBM: 128 bytes per right-hand side and site, 192 with x, 160 on average; with r stored beside p it was
-// 192: an iteration of five-solve trajectories 0.389 -> 0.353 ms at 80 x 80 x 160 with 8 right-hand sides. r so recovered carries the rounding of p instead of its
-// own; the iteration counts are those of the stored r (1409 : 1409 in a five-solve trajectory there).
+// 192: an iteration of five-solve trajectories 0.389 -> 0.353 ms at 80 x 80 x 160 with 8 right-hand sides. r so
+// recovered carries the rounding of p instead of its own; the iteration counts are those of the stored r (1409 : 1409
+// in a five-solve trajectory there).
 template <bool FROM_R>
 __global__ void __launch_bounds__(256) k_cg_xp(float4* __restrict__ x, const float4* __restrict__ p, const float4* pr,
                                                float4* pnew, const float4* __restrict__ q, int64_t n16,

@@ -748,7 +748,7 @@ extern "C" int hmc_trajectory_stats(const hmc_ctx* ctx, int chain, hmc_traj_stat
 
 // One HMC update of every chain together (hmc_params.batch_chains): the same steps as run_chain,
 // with the per-chain work issued back to back without host synchronisation and every force solve
-// of all chains in one persistent launch (batched_cg). Concatenated layouts: fermion vectors
+// of all chains in one persistent launch (batch.cu). Concatenated layouts: fermion vectors
 // [chain][k][V_c][4] at item offset K off_c, boson fields [chain][3][V_c] at 3 off_c. The host
 // synchronises once, for the energies and the Metropolis decisions.
 static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {

@@ -751,7 +751,7 @@ __device__ __forceinline__ void boson_site(const Lat& lat, const BosonCoef& bc,
 // With ACT, partials: [0, nblk) = sum_k 2 Re<pf, X> - |Y|^2, [nblk, 2 nblk) = S_B density; pf is read for
 // them only. The FP64 pipe bounds it: 24 operations per site and right-hand side for the force and 16 for
 // the action, every product in a fused multiply-add (about 60 as sums of complex products). 80 x 80 x 160 with
-// 8 right-hand sides and Y given: 1.14 ms before, 0.42 without and 0.62 with the action.
+// 8 right-hand sides and Y given: 1.14 ms before, 0.42 without and 0.70 with the action.
 template <bool ACT>
 __global__ void __launch_bounds__(256) k_force(Lat lat, Coef<double> cf, BosonCoef bc,
                                                const double* __restrict__ phi,

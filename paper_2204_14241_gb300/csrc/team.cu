@@ -9,7 +9,7 @@
 //
 // Small lattices are bound by latency, a launch or a barrier after every few microseconds of work: with a
 // launch per step and the host reading flags an iteration took 27 to 60 us (CG, PCG) whatever the size, here
-// 4 to 8 and 13 to 30 up to some 30000 sites. From about 10^5 sites memory bounds complex64 and the FP64 pipe
+// 4 to 8 and 13 to 27 up to some 30000 sites. From about 10^5 sites memory bounds complex64 and the FP64 pipe
 // complex128.
 //
 // Work is dealt in items, one band's two spin components of one site (16 bytes in complex64): a block
