@@ -832,7 +832,9 @@ template <> const double2* plan_tw<double>(const FftPlan* p) { return p->tw64; }
 template <typename R> static bool pre_setup(hmc_ctx* ctx, const Lat& lat, TeamPre<R>* q) {
     const FftPlan *px = get_plan(ctx, lat.L), *ptau = get_plan(ctx, lat.Nt);
     const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
-    if (!px || !ptau || !pc || !dft_split(lat.L, &q->x1, &q->x2) || !dft_split(lat.Nt, &q->t1, &q->t2)) return false;
+    if (!px || !ptau || !pc || !dft_split(lat.L, &q->x1, &q->x2, sizeof(R) == 8) ||
+        !dft_split(lat.Nt, &q->t1, &q->t2, sizeof(R) == 8))
+        return false;
     q->twx = plan_tw<R>(px);
     q->twt = plan_tw<R>(ptau);
     if constexpr (sizeof(R) == 4) {

@@ -1,6 +1,7 @@
-"""Preconditioned one-launch solves with more blocks than (slice, band) planes: blocks without a plane, planes that
-outnumber the blocks by a few, a plane per block. The solver stops at a true relative residual of 1e-10, computed in
-complex128; the residual formed here with the FP64 normal operator differs from it by rounding, under 1e-12."""
+"""Preconditioned one-launch solves with two-step transforms of 6 to 10 points in FP64, and with more blocks than
+(slice, band) planes: blocks without a plane, planes that outnumber the blocks by a few, a plane per block. The solver
+stops at a true relative residual of 1e-10, computed in complex128; the residual formed here with the FP64 normal
+operator differs from it by rounding, under 1e-12."""
 
 import pytest
 import torch
@@ -11,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("solver", ["mixed", "fp64"])
-@pytest.mark.parametrize("L,Nt,k", [(20, 5, 1), (20, 24, 1), (20, 40, 1), (20, 40, 4), (40, 80, 1), (24, 48, 2)])
-def test_more_blocks_than_planes(L, Nt, k, solver):
+@pytest.mark.parametrize("L,Nt,k", [(6, 9, 2), (8, 8, 1), (10, 6, 3), (20, 5, 1), (20, 24, 1), (20, 40, 1), (20, 40, 4), (40, 80, 1), (24, 48, 2)])
+def test_preconditioned_teams(L, Nt, k, solver):
     from paper_2204_14241_gb300.hmc import Context
     ctx = Context(L, Nt, nrhs_max=k, solver=solver, **presets.baseline())
     g = torch.Generator(device="cuda")
