@@ -127,6 +127,45 @@ __device__ __forceinline__ It<R> d_item(const BChainDev& g, const Coef<R>& cf, c
     return o;
 }
 
+// Spin q of the item alone, complex128: the same operations in the same order, for blocks of up to 64 items. Their two
+// warps leave half of the SM's FP64 pipe idle, a warp's operation holding its quarter for 64 clocks; an item by two
+// lanes takes 19 of them instead of 35. From 96 items on all quarters are busy either way and the shared factors
+// would be formed twice. Microseconds an iteration, an item a lane : a spin a lane: CG 11.6 : 10.2 at 8 x 8 x 16, 12.1 : 10.7
+// at 16 x 16 x 16; PCG 21.9 : 20.7 at 4 x 4 x 8.
+template <bool DAG, bool BM>
+__device__ __forceinline__ double2 d_spin(const BChainDev& g, const Coef<double>& cf, const double* __restrict__ phi, int i,
+                                          int q, const double2* v) {
+    const int L = g.L, LL = g.LL, hop = 2 * ((int)g.V - LL), u = BM ? 1 : 2;
+    int band, s, t, rem;
+    if (BM) {
+        const int k = fdiv(i, g.dLL);
+        band = k & 1;
+        t = k >> 1;
+        rem = i - k * LL;
+        s = t * LL + rem;
+    } else {
+        band = i & 1;
+        s = i >> 1;
+        t = fdiv(s, g.dLL);
+        rem = s - t * LL;
+    }
+    const int y = fdiv(rem, g.dL), x = rem - y * L, other = BM ? (band ? i - LL : i + LL) : i ^ 1;
+    auto ld = [&](int j) { return v[2 * j + q]; };
+    const double2 c = ld(i), ws = ld(other), wo = v[2 * other + 1 - q];
+    const double2 xm = ld(x ? i - u : i + u * (L - 1)), xp = ld(x + 1 < L ? i + u : i - u * (L - 1));
+    const double2 ym = ld(y ? i - u * L : i + u * (LL - L)), yp = ld(y + 1 < L ? i + u * L : i - u * (LL - L));
+    const int edge = DAG ? (t == 0) : (t + 1 == g.Nt);
+    const double2 tn = ld(DAG ? (edge ? i + hop : i - 2 * LL) : (edge ? i - hop : i + 2 * LL));
+    const double f = flip(cf.cpl, (x + y) & 1);
+    const double q1 = f * __ldg(phi + s), q2 = flip(f * __ldg(phi + g.V + s), q), q3 = flip(f * __ldg(phi + 2 * g.V + s), q);
+    const double d = band ? cf.diag[1] : cf.diag[0], hx = band ? cf.hx[1] : cf.hx[0], hy = band ? cf.hy[1] : cf.hy[0];
+    const double hr = fma(hx, xm.x + xp.x, fma(hy, ym.x + yp.x, flip(tn.x, edge)));
+    const double hi = fma(hx, xm.y + xp.y, fma(hy, ym.y + yp.y, flip(tn.y, edge)));
+    return make_double2(fma(d, c.x, fma(q3, ws.x, fma(q1, wo.x, fma(q2, wo.y, hr)))),
+                        fma(d, c.y, fma(q3, ws.y, fma(q1, wo.y, fma(-q2, wo.x, hi)))));
+}
+constexpr int kSpinItems = 64;   // most items of a block for d_spin
+
 // Per-thread sum of squares: FP64, or an FP32 pair with exact products and compensated additions (48
 // bits). Converting every component of an FP32 vector for an FP64 sum takes more of the FP64 pipe's
 // time (two lanes a clock per SM) than the rest of a phase takes.
@@ -621,6 +660,15 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 st_it<R>(t, i, o);
                 sq_it(acc, o);
             }
+        } else if (!kMixed && per <= kSpinItems) {
+            if constexpr (!kMixed) {
+                for (int e = 2 * i0 + threadIdx.x; e < 2 * i1; e += blockDim.x) {
+                    const double2 o = d_spin<true, PRE>(g, a.cf, phi, e >> 1, e & 1, pold);
+                    t[e] = o;
+                    acc.sq(o.x);
+                    acc.sq(o.y);
+                }
+            }
         } else {
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 const It<R> o = d_item<R, true, PRE>(g, a.cf, phi, i, ldr(pold));
@@ -646,15 +694,40 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             sq_it(acc, rn);
             return rn;
         };
+        auto update_spin = [&](int i, int q) {
+            if constexpr (!kMixed) {
+                const double2 v = d_spin<false, PRE>(g, a.cf, phi, i, q, t);
+                const int e = 2 * i + q, o = PRE ? 2 * from_bm(g, i) + q : e;
+                const double2 pv = pnew[e], xv = x[o], rv = r[e];
+                x[o] = make_double2(fma(al, pv.x, xv.x), fma(al, pv.y, xv.y));
+                const double2 rn = make_double2(fma(-al, v.x, rv.x), fma(-al, v.y, rv.y));
+                r[e] = rn;
+                acc.sq(rn.x);
+                acc.sq(rn.y);
+                return rn;
+            } else {
+                return mk<C>(0.f, 0.f);
+            }
+        };
         if constexpr (PRE) {
             each_round([&](int t0, int np) {
-                each_site(t0, np, [&](int i, int at) {
-                    const It<R> v = update(i);
-                    pt.tile[at] = v.s[0];
-                    pt.tile[at + 1] = v.s[1];
-                });
+                if (!kMixed && np * g.LL <= kSpinItems) {
+                    const int RS = row_stride(g.L);
+                    for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
+                        const int pl = fdiv(e >> 1, g.dLL), j = (e >> 1) - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * g.L;
+                        pt.tile[pl * a.pre.plane + (y * RS + xx) * 2 + (e & 1)] = update_spin((t0 + pl * tm.T) * g.LL + j, e & 1);
+                    }
+                } else {
+                    each_site(t0, np, [&](int i, int at) {
+                        const It<R> v = update(i);
+                        pt.tile[at] = v.s[0];
+                        pt.tile[at + 1] = v.s[1];
+                    });
+                }
                 plane_forward<R>(a.pre, pt, g, t0, tm.T, np, z);
             });
+        } else if (!kMixed && per <= kSpinItems) {
+            for (int e = 2 * i0 + threadIdx.x; e < 2 * i1; e += blockDim.x) update_spin(e >> 1, e & 1);
         } else {
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) update(i);
         }
@@ -747,8 +820,15 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             if (!inverse()) return false;
         } else if constexpr (!kMixed) {
             const R be = c.beta;
-            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
-                st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), ld_it<R>(r, i)));
+            if (per <= kSpinItems) {
+                for (int e = 2 * i0 + threadIdx.x; e < 2 * i1; e += blockDim.x) {
+                    const C pv = pold[e], rv = r[e];
+                    pold[e] = mk<C>(fma(be, pv.x, rv.x), fma(be, pv.y, rv.y));
+                }
+            } else {
+                for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
+                    st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), ld_it<R>(r, i)));
+            }
             if (!sync()) return false;
         }
     }
