@@ -288,6 +288,7 @@ struct Team {
     unsigned long long* part;   // [2][gridDim.x] partial sums, by the barrier's parity
     unsigned long long* cpart;  // [2][16], shared memory: the same for a cluster
     unsigned epoch;
+    int warps;                  // warps of a block with values in a sum (FP64), the rest hold zeros
     bool never;                 // the next barrier waits for more arrivals than there are blocks (timeout test)
     bool shared_sm;             // other blocks may be at work on this SM
     int* flags;
@@ -346,8 +347,8 @@ __device__ __forceinline__ bool sync_sum(Team& tm, C& ctl, unsigned long long* r
     if (w == 0) {
         if constexpr (k64) {
             // one warp adds the block's values: in the shuffle tree of every warp each addition would take
-            // the SM's FP64 pipe 16 clocks a warp
-            for (int j = 1; j < nw; ++j) {
+            // the SM's FP64 pipe 16 clocks a warp; 64 clocks a warp of values here, so small systems skip the empty ones
+            for (int j = 1; j < tm.warps; ++j) {
                 S o;
                 o.from(red[lane + 32 * j]);
                 acc.plus(o);
@@ -482,6 +483,12 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     const R* phi;
     if constexpr (kMixed) phi = g.phi32;
     else phi = g.phi64;
+    if constexpr (!kMixed) {   // the largest phase's lanes
+        int lanes = 2 * min(per, kSpinItems);
+        lanes = max(lanes, per);
+        if constexpr (PRE) lanes = max(lanes, max(max(2 * min(a.pre.np * g.LL, kSpinItems), a.pre.np * g.LL), g.Nt * a.pre.W));
+        tm.warps = min((int)blockDim.x >> 5, (lanes + 31) >> 5);
+    }
     auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](const NoSum&) {}); };
     auto in = [&](int i) { return PRE ? to_bm(g, i) : i; };   // from the public layout to the solver's
     auto ld64 = [](const double2* v) { return [v](int j) { return ld_it<double>(v, j); }; };
@@ -857,6 +864,7 @@ k_team(const __grid_constant__ TeamArgs<R> a) {
     Team tm;
     tm.part = a.part;
     tm.cpart = cpart;
+    tm.warps = blockDim.x >> 5;
     tm.never = a.test_timeout != 0;
     tm.shared_sm = a.pairs != nullptr;
     tm.flags = a.flags;
