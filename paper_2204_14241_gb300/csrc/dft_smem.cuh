@@ -80,10 +80,11 @@ __device__ __forceinline__ int dft_pos(int k, int n1, int n2) { return n1 * (k %
 // ---- host --------------------------------------------------------------------------------------------
 // N = n1 n2 with both factors among dft_step's radices, their sum (the work per point) least; up to 10
 // points in one step: a step costs its latency, not its work, at the sizes that take few points. spread: two steps
-// from 6 points on, for FP64 transforms of few lines (a warp's operation takes its quarter of the SM's FP64 pipe 64
-// clocks however few lanes are at work, 56 of them for 8 points by a thread, 24 in two steps by four and two: FP64
-// PCG in one launch 28.9 -> 23.9 us an iteration at 8 x 8 x 8, 38.6 -> 30.6 at 10 x 10 x 10, 23.6 -> 22.0 at
-// 4 x 4 x 8).
+// from 6 points on, for FP64 (a warp's operation takes its quarter of the SM's FP64 pipe 64 clocks however few lanes
+// are at work, 56 of them for 8 points by a thread, 24 in two steps by four and two): PCG in one launch 28.9 -> 23.9 us
+// an iteration at 8 x 8 x 8, 38.6 -> 30.6 at 10 x 10 x 10; the drift 30.2 -> 24.6 at 8 x 8 x 8, 36.9 -> 28.7 at
+// 10 x 10 x 10; the complex128 preconditioner 34.8 -> 28.4 there. Many lines lose nothing: 133 -> 122 at 10 x 10 x 96
+// with 8 right-hand sides.
 // False when there is none.
 inline bool dft_split(int n, int* n1, int* n2, bool spread = false) {
     static const int radix[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};

@@ -305,7 +305,7 @@ static int tile_width(const hmc_ctx* ctx, int total, int n1, int n2, size_t line
 
 static bool make_desc(hmc_ctx* ctx, const Lat& lat, MetricDesc* d) {
     const FftPlan *px = get_plan(ctx, lat.L), *pt = get_plan(ctx, lat.Nt);
-    if (lat.L < 4 || !px || !pt || !dft_split(lat.L, &d->x1, &d->x2) || !dft_split(lat.Nt, &d->t1, &d->t2)) return false;
+    if (lat.L < 4 || !px || !pt || !dft_split(lat.L, &d->x1, &d->x2, true) || !dft_split(lat.Nt, &d->t1, &d->t2, true)) return false;
     if (plane_smem(lat.L) > kMSmem) return false;
     d->L = lat.L;
     d->Nt = lat.Nt;

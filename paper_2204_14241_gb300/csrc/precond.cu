@@ -220,7 +220,9 @@ template <typename R> static bool plane_args(hmc_ctx* ctx, const Lat& lat, int n
     constexpr int NC = kComp<R>, G = 4 / NC;
     const FftPlan *px = get_plan(ctx, lat.L), *pt = get_plan(ctx, lat.Nt);
     const PcTables* pc = get_pc(ctx, lat.L, lat.Nt);
-    if (!px || !pt || !pc || !dft_split(lat.L, &a->x1, &a->x2) || !dft_split(lat.Nt, &a->t1, &a->t2)) return false;
+    if (!px || !pt || !pc || !dft_split(lat.L, &a->x1, &a->x2, sizeof(R) == 8) ||
+        !dft_split(lat.Nt, &a->t1, &a->t2, sizeof(R) == 8))
+        return false;
     const int L = lat.L, Nt = lat.Nt, LL = L * L;
     const int64_t planes = (int64_t)nrhs * Nt * G;
     const size_t psize = (size_t)L * (L | 1) * NC * sizeof(cplx<R>), ptab = L * sizeof(cplx<R>);
