@@ -80,7 +80,7 @@ typedef struct {
                            + 4 X_{n-2} - X_{n-3}; ...; lower degree while fewer solutions exist),
                            m FP64 vectors of workspace. The same stopping test applies in every
                            case. */
-    int autotune;       /* 0: tile shapes of the fused A kernel (complex64 up to 8192 sites in all, and
+    int autotune;       /* 0: tile shapes of the fused A kernel (complex64 up to 2^18 sites in all, and
                            solves that fold the direction into it) from a fixed rule (default; the
                            reduction order, hence every bit of the results, is reproducible);
                            1: on first use per (L, Nt, nrhs, precision) time the valid tile and
@@ -138,7 +138,7 @@ int apply_M(hmc_ctx* ctx, int chain, int prec, const void* phi, const void* x, v
             int dagger, int nrhs);
 
 /* y = A x = D (D^dagger x) (Eq. linsys): one fused launch for complex64 on lattices with a strip
- * kernel or of up to 8192 sites, two passes through workspace otherwise. If norm2 is not NULL it
+ * kernel or of up to 2^18 sites, two passes through workspace otherwise. If norm2 is not NULL it
  * receives (host, nrhs doubles) ||D^dagger x_k||^2 = x_k^dagger A x_k. */
 int apply_MdagM(hmc_ctx* ctx, int chain, int prec, const void* phi, const void* x, void* y,
                 int nrhs, double* norm2);

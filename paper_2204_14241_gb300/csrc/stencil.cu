@@ -547,8 +547,9 @@ int launch_apply_A(hmc_ctx* ctx, const Lat& lat, const R* phi, const cplx<R>* x,
             if (strip_supported(lat) && aligned32(y))
                 return launch_apply_A_strip(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
         }
-        // (a second launch costs the host 2 us, what the passes save only past some 8000 sites in complex64)
-        if (sizeof(R) == 8 || nrhs * lat.V > 8192)
+        // A second launch costs a caller 3 us, more than the passes save up to 2^18 sites in complex64: 12.3 us fused
+        // against 14.5 a call at 24 x 24 x 48 with 8 right-hand sides, 20.5 against 15.5 at 36 x 36 x 70 with 4.
+        if (sizeof(R) == 8 || nrhs * lat.V > 262144)
             return launch_A_two_pass<R>(ctx, lat, phi, x, y, nrhs, part, nblk_out, cgs);
     }
     static PerDevice attr;

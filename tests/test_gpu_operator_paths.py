@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("shift", [0, 2])   # complex64 entries: 16 bytes
 @pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128])
-@pytest.mark.parametrize("L,Nt,k", [(2, 3, 1), (6, 5, 2), (16, 5, 2), (18, 15, 1)])
+@pytest.mark.parametrize("L,Nt,k", [(2, 3, 1), (6, 5, 2), (16, 5, 2), (18, 15, 1), (36, 70, 3)])
 def test_alignment_and_routes(L, Nt, k, dtype, shift):
     from paper_2204_14241_gb300.hmc import Context
     tol, rdt = (1e-5, torch.float32) if dtype == torch.complex64 else (1e-12, torch.float64)
