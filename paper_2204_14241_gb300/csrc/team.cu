@@ -323,6 +323,11 @@ __device__ __forceinline__ bool wait_arrivals(const Team& tm, unsigned want) {
     return true;
 }
 
+// Hardware barrier of a cluster's blocks: shared memory written before it, own or remote, is seen after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Barrier of the team's blocks with the sum of `acc` over all their threads; writes before it are seen by
 // plain loads after it. All blocks add in the same order; lane 0 then runs fin(sum) for everybody. False
 // (with the error word set) when the wait gives up.
@@ -366,11 +371,12 @@ __device__ __forceinline__ bool sync_sum(Team& tm, C& ctl, unsigned long long* r
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(lane));
                 asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(theirs), "l"(acc.bits()) : "memory");
             }
+            __syncwarp();   // the barrier's .aligned form wants the whole warp
         }
     }
     bool ok = true;
     if constexpr (CLU) {
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_sync();
         if (w == 0) {
             acc = S();
             if (lane < tm.T) acc.from(tm.cpart[16 * par + lane]);
@@ -861,6 +867,8 @@ k_team(const __grid_constant__ TeamArgs<R> a) {
     __shared__ unsigned long long cpart[2 * 16];
     __shared__ BChainDev g;
     __shared__ Ctl<R> ctl;
+    // A block of a cluster writes to the others' cpart, which is theirs only once they have started.
+    if constexpr (CLU) cluster_sync();
     Team tm;
     tm.part = a.part;
     tm.cpart = cpart;
