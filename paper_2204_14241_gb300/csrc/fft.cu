@@ -751,10 +751,10 @@ __global__ void __launch_bounds__(256) k_spectral(double2* __restrict__ v, const
     }
 }
 
-// out = Re(v) (eps == 0) or out += eps Re(v)
-__global__ void k_unpack_real(const double2* __restrict__ v, double* __restrict__ out, int64_t n, double eps) {
+// out = Re(v) or (add) out += eps Re(v)
+__global__ void k_unpack_real(const double2* __restrict__ v, double* __restrict__ out, int64_t n, double eps, bool add) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = eps == 0.0 ? v[i].x : out[i] + eps * v[i].x;
+    if (i < n) out[i] = add ? out[i] + eps * v[i].x : v[i].x;
 }
 
 static int fft3_real_field(hmc_ctx* ctx, const Lat& lat, double2* v, int dir) {
@@ -767,9 +767,9 @@ static int fft3_real_field(hmc_ctx* ctx, const Lat& lat, double2* v, int dir) {
 }
 
 int metric_op(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in,
-              double* out, double eps, double* scalar_dev) {
+              double* out, double eps, bool add, double* scalar_dev) {
     bool done = false;
-    int rc = metric_real(ctx, lat, op, sig, in, out, eps, scalar_dev, &done);
+    int rc = metric_real(ctx, lat, op, sig, in, out, eps, add, scalar_dev, &done);
     if (rc || done) return rc;
     // extents without a two-factor split, or planes past an SM's shared memory: complex transforms axis by axis
     const int64_t n = 3 * lat.V;
@@ -792,7 +792,7 @@ int metric_op(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const dou
     k_spectral<<<nb, 256, 0, ctx->stream>>>(v, sig, n, op == HMC_METRIC_MOMENTUM ? 1 : 0, nullptr, nullptr);
     HMC_LAUNCH(ctx, "k_spectral");
     if ((rc = fft3_real_field(ctx, lat, v, +1))) return rc;
-    k_unpack_real<<<nb, 256, 0, ctx->stream>>>(v, out, n, eps);
+    k_unpack_real<<<nb, 256, 0, ctx->stream>>>(v, out, n, eps, add);
     HMC_LAUNCH(ctx, "k_unpack_real");
     return HMC_OK;
 }

@@ -515,7 +515,7 @@ extern "C" int metric_apply(hmc_ctx* ctx, int chain, int op, const void* sig, co
     }
     DevGuard g(ctx);
     const Lat& lat = ctx->chains[chain].lat;
-    if ((rc = metric_op(ctx, lat, op, (const double*)sig, (const double*)in, (double*)out, 0.0, ctx->d_red))) return rc;
+    if ((rc = metric_op(ctx, lat, op, (const double*)sig, (const double*)in, (double*)out, 0.0, false, ctx->d_red))) return rc;
     if (op == HMC_METRIC_KINETIC || op == HMC_METRIC_MNORM) return fetch_red(ctx, 1, scalar);
     return HMC_OK;
 }
@@ -605,8 +605,8 @@ static int run_chain(hmc_ctx* ctx, int c, const hmc_traj_in* in, double out_e[6]
     // heatbath varphi = D chi, momentum, initial energies
     if ((rc = launch_apply_D<double>(ctx, lat, phi, chi, ctx->d_pf, 0, K))) return rc;
     if ((rc = tm.mark(kPhaseMetric))) return rc;
-    if ((rc = metric_op(ctx, lat, HMC_METRIC_MOMENTUM, sig, z, ctx->d_pi, 0.0, nullptr))) return rc;
-    if ((rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, ctx->d_pi, nullptr, 0.0, E))) return rc;
+    if ((rc = metric_op(ctx, lat, HMC_METRIC_MOMENTUM, sig, z, ctx->d_pi, 0.0, false, nullptr))) return rc;
+    if ((rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, ctx->d_pi, nullptr, 0.0, false, E))) return rc;
     if ((rc = tm.mark(kPhaseOther))) return rc;
     int nbb = 0;
     if ((rc = launch_boson(ctx, lat, ch.r, phi, nullptr, ctx->d_part, &nbb))) return rc;
@@ -681,7 +681,7 @@ static int run_chain(hmc_ctx* ctx, int c, const hmc_traj_in* in, double out_e[6]
         HMC_LAUNCH(ctx, "k_axpy");
         for (int i = 1; i <= in->n_leap && !rc; ++i) {
             if ((rc = tm.mark(kPhaseMetric))) break;
-            if ((rc = metric_op(ctx, lat, HMC_METRIC_VELOCITY, sig, ctx->d_pi, phi, eps, nullptr))) break;
+            if ((rc = metric_op(ctx, lat, HMC_METRIC_VELOCITY, sig, ctx->d_pi, phi, eps, true, nullptr))) break;
             if ((rc = do_force(i == in->n_leap))) break;
             k_axpy<<<gb, 256, 0, sm>>>(i < in->n_leap ? eps : 0.5 * eps, ctx->d_F, ctx->d_pi, nb);
             HMC_LAUNCH(ctx, "k_axpy");
@@ -689,13 +689,13 @@ static int run_chain(hmc_ctx* ctx, int c, const hmc_traj_in* in, double out_e[6]
         if (in->n_leap == 0 && !rc) rc = do_force(true);
     }
     if (!rc) rc = tm.mark(kPhaseMetric);
-    if (!rc) rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, ctx->d_pi, nullptr, 0.0, E + 3);
+    if (!rc) rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, ctx->d_pi, nullptr, 0.0, false, E + 3);
     if (!rc) rc = tm.mark(kPhaseOther);
     if (!rc && jump2) {
         // squared M-norm of the proposed jump (Eq. ESJD), accepted or not
         k_sub<<<gb, 256, 0, sm>>>(phi, ctx->d_phi_save, ctx->d_vel, nb);
         HMC_LAUNCH(ctx, "k_sub");
-        rc = metric_op(ctx, lat, HMC_METRIC_MNORM, sig, ctx->d_vel, nullptr, 0.0, ctx->d_red + 60);
+        rc = metric_op(ctx, lat, HMC_METRIC_MNORM, sig, ctx->d_vel, nullptr, 0.0, false, ctx->d_red + 60);
     }
     *iters = tot_it;
     *worst = wr;
@@ -795,8 +795,8 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
         HMC_LAUNCH(ctx, "k_norm2");
         if ((rc = reduce_rows(ctx, ctx->d_part, 1, 1024, E + 6 * c + 2))) return rc;
         const double* sig = (const double*)in->sigma_hat[c];
-        if ((rc = metric_op(ctx, lat, HMC_METRIC_MOMENTUM, sig, z, bvec(ctx->d_pi, c), 0.0, nullptr))) return rc;
-        if ((rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, bvec(ctx->d_pi, c), nullptr, 0.0, E + 6 * c))) return rc;
+        if ((rc = metric_op(ctx, lat, HMC_METRIC_MOMENTUM, sig, z, bvec(ctx->d_pi, c), 0.0, false, nullptr))) return rc;
+        if ((rc = metric_op(ctx, lat, HMC_METRIC_KINETIC, sig, bvec(ctx->d_pi, c), nullptr, 0.0, false, E + 6 * c))) return rc;
         int nbb = 0;
         if ((rc = launch_boson(ctx, lat, ctx->chains[c].r, phi, nullptr, ctx->d_part, &nbb))) return rc;
         if ((rc = reduce_rows(ctx, ctx->d_part, 1, nbb, E + 6 * c + 1))) return rc;
@@ -874,7 +874,7 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
             if (ctx->batch.metric_ok && (r2 = metric_batch_drift(ctx, eps))) return r2;
             for (int c = 0; c < nc && !ctx->batch.metric_ok; ++c)
                 if ((r2 = metric_op(ctx, ctx->chains[c].lat, HMC_METRIC_VELOCITY, (const double*)in->sigma_hat[c],
-                                    bvec(ctx->d_pi, c), (double*)in->phi[c], eps, nullptr)))
+                                    bvec(ctx->d_pi, c), (double*)in->phi[c], eps, true, nullptr)))
                     return r2;
             if ((r2 = mark(kPhaseOther))) return r2;
             if ((r2 = do_force(i == in->n_leap))) return r2;
@@ -969,13 +969,13 @@ static int run_batched(hmc_ctx* ctx, const hmc_traj_in* in, hmc_traj_out* out) {
     if (!rc) rc = tm.mark(kPhaseMetric);
     for (int c = 0; c < nc && !rc; ++c) {
         rc = metric_op(ctx, ctx->chains[c].lat, HMC_METRIC_KINETIC, (const double*)in->sigma_hat[c], bvec(ctx->d_pi, c),
-                       nullptr, 0.0, E + 6 * c + 3);
+                       nullptr, 0.0, false, E + 6 * c + 3);
         if (!rc && out && out->jump2) {
             const Lat& lat = ctx->chains[c].lat;
             const int64_t nb = 3 * lat.V;
             k_sub<<<(unsigned)((nb + 255) / 256), 256, 0, sm>>>(phis[c], bvec(ctx->d_phi_save, c), ctx->d_vel, nb);
             HMC_LAUNCH(ctx, "k_sub");
-            rc = metric_op(ctx, lat, HMC_METRIC_MNORM, (const double*)in->sigma_hat[c], ctx->d_vel, nullptr, 0.0,
+            rc = metric_op(ctx, lat, HMC_METRIC_MNORM, (const double*)in->sigma_hat[c], ctx->d_vel, nullptr, 0.0, false,
                            ctx->d_red + c % 64);
             if (!rc) HMC_CUDA(ctx, cudaMemcpyAsync(out->jump2 + c, ctx->d_red + c % 64, sizeof(double),
                                                    cudaMemcpyDeviceToHost, sm));

@@ -330,14 +330,15 @@ int launch_pcg_xy_inverse(hmc_ctx* ctx, const Lat& lat, const float2* zhat, cons
                           int nrhs, const CgScalars* cgs);
 // metric.cu: the same on real transforms; *done = false where the lattice rules them out
 int metric_real(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in, double* out, double eps,
-                double* scalar_dev, bool* done);
+                bool add, double* scalar_dev, bool* done);
 // the drift phi += eps F^-1(sigma F pi) of every chain of a batch (pi in ctx->d_pi), three launches:
 // metric_batch_begin uploads a trajectory's table (and sets batch.metric_ok), metric_batch_drift enqueues one
 int metric_batch_alloc(hmc_ctx* ctx);
 int metric_batch_begin(hmc_ctx* ctx, const double* const* sig, double* const* phi);
 int metric_batch_drift(hmc_ctx* ctx, double eps);
+// one metric operation (fft.cu): the field operations set out, or (add) out += eps times their result, whatever eps is
 int metric_op(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in,
-              double* out, double eps, double* scalar_dev);
+              double* out, double eps, bool add, double* scalar_dev);
 
 // randomized diagonal estimator of F~^* D^{-1} F~ over nrhs probes (fft.cu)
 int green_run(hmc_ctx* ctx, int chain, const double* phi, const double2* v, int nrhs, double2* out, int precond,

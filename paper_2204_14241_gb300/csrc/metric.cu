@@ -224,24 +224,25 @@ __device__ __forceinline__ void pack_pair(double2* row, const int* pos, int L, i
         row[pos[L - k]] = make_double2(v.x - u.y, u.x + v.y);
     }
 }
-__device__ __forceinline__ void put_rows(const MetricDesc& d, const double2* rows, int pairs, int64_t first, double eps) {
+__device__ __forceinline__ void put_rows(const MetricDesc& d, const double2* rows, int pairs, int64_t first, double eps, bool add) {
     const int L = d.L, RA = L | 1;
     double* out = d.out + first * 2 * L;
-    const double s = eps == 0.0 ? d.scale : eps * d.scale;
+    const double s = add ? eps * d.scale : d.scale;
     for (int e = threadIdx.x; e < pairs * L; e += blockDim.x) {
         const int j = fdiv(e, d.dL), x = e - j * L;
         const double2 z = rows[j * RA + x];
         double *o0 = out + 2 * j * L + x, *o1 = o0 + L;
-        if (eps == 0.0) {
-            *o0 = s * z.y;
-            *o1 = s * z.x;
-        } else {
+        if (add) {
             *o0 = fma(s, z.y, *o0);
             *o1 = fma(s, z.x, *o1);
+        } else {
+            *o0 = s * z.y;
+            *o1 = s * z.x;
         }
     }
 }
-__global__ void __launch_bounds__(256, 2) k_metric_x_inv(const __grid_constant__ MetricDesc d, int W, FastDiv dW, double eps) {
+__global__ void __launch_bounds__(256, 2) k_metric_x_inv(const __grid_constant__ MetricDesc d, int W, FastDiv dW, double eps,
+                                                          bool add) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int L = d.L, Hx = d.Hx, RA = L | 1, total = 3 * d.Nt * (L / 2), c0 = blockIdx.x * W, live = min(W, total - c0);
     double2 *rows = reinterpret_cast<double2*>(smem), *tw = rows + W * RA;
@@ -256,12 +257,12 @@ __global__ void __launch_bounds__(256, 2) k_metric_x_inv(const __grid_constant__
     }
     __syncthreads();
     dft_inverse(rows, Lines{1, 0, W, dW, RA, 2 * RA}, d.x1, d.x2, 1, tw);
-    put_rows(d, rows, live, c0, eps);
+    put_rows(d, rows, live, c0, eps, add);
 }
 
-// The planes back: out = scale * (real field), or out += eps * that.
+// The planes back: out = scale * (real field), or (add) out += eps * that.
 __global__ void __launch_bounds__(256, 2) k_metric_inv(const MetricDesc* __restrict__ tab,
-                                                       const __grid_constant__ MetricDesc one, double eps) {
+                                                       const __grid_constant__ MetricDesc one, double eps, bool add) {
     extern __shared__ __align__(16) unsigned char smem[];
     const MetricDesc& d = tab ? tab[blockIdx.y] : one;
     const int L = d.L, Hx = d.Hx, RA = L | 1, RB = Hx | 1;
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(256, 2) k_metric_inv(const MetricDesc* __restr
     }
     __syncthreads();
     dft_inverse(p.rows, Lines{1, 0, L / 2, d.dHalf, RA, 2 * RA}, d.x1, d.x2, 1, p.tw);
-    put_rows(d, p.rows, L / 2, (int64_t)blockIdx.x * (L / 2), eps);
+    put_rows(d, p.rows, L / 2, (int64_t)blockIdx.x * (L / 2), eps, add);
 }
 
 // ---- host --------------------------------------------------------------------------------------------
@@ -351,7 +352,7 @@ static int plane_threads(int L) { return L >= 32 ? 256 : L >= 16 ? 128 : 64; }
 static double op_scale(int op, double V) { return (op == HMC_METRIC_KINETIC ? 0.5 : 1.0) / (4.0 * V); }
 
 int metric_real(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const double* in, double* out, double eps,
-                double* scalar_dev, bool* done) {
+                bool add, double* scalar_dev, bool* done) {
     MetricDesc d{};
     *done = make_desc(ctx, lat, &d);
     if (!*done) return HMC_OK;
@@ -388,9 +389,9 @@ int metric_real(hmc_ctx* ctx, const Lat& lat, int op, const double* sig, const d
     if (lines) {
         k_metric_y<true><<<gy, 256, Wy * yline + xtab, ctx->stream>>>(d, Wy, fast_div(Wy));
         HMC_LAUNCH(ctx, "k_metric_y");
-        k_metric_x_inv<<<gx, 256, Wx * xline + xtab, ctx->stream>>>(d, Wx, fast_div(Wx), eps);
+        k_metric_x_inv<<<gx, 256, Wx * xline + xtab, ctx->stream>>>(d, Wx, fast_div(Wx), eps, add);
     } else {
-        k_metric_inv<<<(unsigned)planes, plane_threads(lat.L), plane_smem(lat.L), ctx->stream>>>(nullptr, d, eps);
+        k_metric_inv<<<(unsigned)planes, plane_threads(lat.L), plane_smem(lat.L), ctx->stream>>>(nullptr, d, eps, add);
     }
     HMC_LAUNCH(ctx, "k_metric_inv");
     return HMC_OK;
@@ -444,7 +445,7 @@ int metric_batch_drift(hmc_ctx* ctx, double eps) {
     k_metric_fwd<<<planes, thr, plane_smem(w.maxL), ctx->stream>>>(tab, MetricDesc{});
     HMC_LAUNCH(ctx, "k_metric_fwd");
     if ((rc = launch_tau(ctx, tab, MetricDesc{}, nc, w.tau_tiles, w.maxNt, w.tau_smem, HMC_METRIC_VELOCITY))) return rc;
-    k_metric_inv<<<planes, thr, plane_smem(w.maxL), ctx->stream>>>(tab, MetricDesc{}, eps);
+    k_metric_inv<<<planes, thr, plane_smem(w.maxL), ctx->stream>>>(tab, MetricDesc{}, eps, true);
     HMC_LAUNCH(ctx, "k_metric_inv");
     return HMC_OK;
 }
