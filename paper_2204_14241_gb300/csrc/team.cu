@@ -167,8 +167,9 @@ __device__ __forceinline__ double2 d_spin(const BChainDev& g, const Coef<double>
 constexpr int kSpinItems = 64;   // most items of a block for d_spin
 
 // Per-thread sum of squares: FP64, or an FP32 pair with exact products and compensated additions (48
-// bits). Converting every component of an FP32 vector for an FP64 sum takes more of the FP64 pipe's
-// time (two lanes a clock per SM) than the rest of a phase takes.
+// bits, as long as the squares stay well inside FP32's range: Scale). Converting every component of an FP32
+// vector for an FP64 sum takes more of the FP64 pipe's time (two lanes a clock per SM) than the rest of a phase
+// takes.
 template <typename R> struct Sum2;
 template <> struct Sum2<double> {
     using T = double;
@@ -270,11 +271,39 @@ struct NoSum {   // a barrier without a sum
     __device__ __forceinline__ double get() const { return 0.0; }
 };
 
+// Complex64 systems are iterated in units of 2^-e, a power of two that keeps the sums of squares, FP32 pairs with
+// FP32's range, away from its ends: squares that lose their low bits below 2^-102, sums that overflow. e follows the
+// true residual at the start and at each reliable update, and changes only when a component's mean square has left
+// 2^-60 .. 2^30: 2^-20 each for the fall until the next update and for ||D^dagger p||^2 against ||p||^2, 2^97 for
+// the number of terms, transforms without their scale and P-hat. A power of two changes no mantissa, so the
+// iterates are those of an unlimited range, bit for bit.
+struct Scale {
+    int e;             // the iterated vectors are 2^e times the system's
+    float s, change;   // 2^e; factor from the units of the vectors in memory, 1 unless e has just changed
+    double s2, inv;    // 2^(2 e), 2^-e
+    __device__ __forceinline__ static double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+    __device__ __forceinline__ void set(int k) {
+        change = (float)pow2(k - e);
+        e = k;
+        s = (float)pow2(k);
+        s2 = pow2(2 * k);
+        inv = pow2(-k);
+    }
+    // for the norm r2, finite and in the system's units, of n items (4 components each)
+    __device__ __forceinline__ void follow(double r2, int n) {
+        change = 1.f;
+        if (!(r2 > 0.0)) return;
+        const int at = ((__double2hiint(r2) >> 20) - 1023) - (33 - __clz(n));   // exponent of the mean square
+        if (at + 2 * e < -60 || at + 2 * e > 30) set(max(max(-100, e - 100), min(min(100, e + 100), -at / 2)));
+    }
+};
+
 // ---- team ------------------------------------------------------------------------------------------
 // A solve's state, in shared memory, written by one thread.
 template <typename R> struct Ctl {
     double b2, r2true;         // ||b||^2, the last true ||r||^2
-    double stop, ru_below;     // tol^2 ||b||^2; ||r||^2 at which a reliable update is due
+    double stop, ru_below;     // tol^2 ||b||^2 and the ||r||^2 at which a reliable update is due, times scale.s2
+    Scale scale;
     Num<R> rr;
     R alpha, beta;
     int it, n_ru, hold, wait;
@@ -530,17 +559,42 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         if (!sync_sum<CLU>(tm, c, red, sb, [&](const Sum2<double>& v) { c.b2 = v.v; })) return false;
         if (!sync_sum<CLU>(tm, c, red, sr, [&](const Sum2<double>& v) {
                 c.r2true = v.v;
-                c.rr = Num<R>(v.v);
                 c.alpha = c.beta = (R)0;
                 c.it = c.n_ru = c.hold = 0;
                 c.wait = 4;
                 c.stop = a.tol2 * c.b2;
-                c.ru_below = kMixed ? fmax(c.stop, a.delta2 * v.v) : c.stop;
                 c.nonfinite = !(isfinite(c.b2) && isfinite(v.v));
                 c.active = !c.nonfinite && c.b2 > 0.0 && v.v > c.stop;
+                double u = v.v;
+                if constexpr (kMixed) {
+                    c.scale.e = 0;
+                    c.scale.set(0);
+                    if (c.active) c.scale.follow(v.v, n);
+                    c.stop *= c.scale.s2;
+                    u *= c.scale.s2;
+                }
+                c.rr = Num<R>(u);
+                c.ru_below = kMixed ? fmax(c.stop, a.delta2 * u) : c.stop;
             }))
             return false;
     }
+    // r and the old direction to the units of a scale that has just changed
+    auto rescale = [&]() {
+        if constexpr (kMixed) {
+            const float f = c.scale.change;
+            if (f != 1.f) {
+                for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+                    const int o = in(i);
+                    const It<R> zero{};
+                    st_it<R>(r, o, axpy_it<R>(f, ld_it<R>(r, o), zero));
+                    st_it<R>(pold, o, axpy_it<R>(f, ld_it<R>(pold, o), zero));
+                }
+                return sync();
+            }
+        }
+        return true;
+    };
+    if (c.active && !rescale()) return false;
 
     // this block's (slice, band) planes, tasks rank, rank + T, ..., as many at a time as the tile holds
     auto each_round = [&](const auto& f) {
@@ -770,10 +824,11 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                     const It<R> lo = ld_it<R>(x, in(i));
                     It<double> hi = ld_it<double>(x64, i);
+                    const double inv = c.scale.inv;
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
-                        hi.s[s].x += (double)lo.s[s].x;
-                        hi.s[s].y += (double)lo.s[s].y;
+                        hi.s[s].x = fma(inv, (double)lo.s[s].x, hi.s[s].x);
+                        hi.s[s].y = fma(inv, (double)lo.s[s].y, hi.s[s].y);
                     }
                     st_it<double>(x64, i, hi);
                     st_it<R>(x, in(i), It<R>{});
@@ -783,12 +838,17 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
             if (!sync()) return false;
             Sum2<double> acc64;
+            R unit = 1;
+            if constexpr (kMixed) unit = c.scale.s;
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 const It<double> rd =
                     axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i));
                 It<R> rl;
 #pragma unroll
-                for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rd.s[s].x, (R)rd.s[s].y);
+                for (int s = 0; s < 2; ++s) {
+                    rl.s[s] = mk<C>((R)rd.s[s].x, (R)rd.s[s].y);
+                    if (kMixed) rl.s[s] = mk<C>(unit * rl.s[s].x, unit * rl.s[s].y);
+                }
                 st_it<R>(r, in(i), rl);
                 sq_it(acc64, rd);
             }
@@ -796,11 +856,21 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                     const double v = sum.v;
                     c.r2true = v;
                     ++c.n_ru;
+                    double u = v;
+                    if (kMixed) u *= c.scale.s2;
                     if (!isfinite(v)) c.nonfinite = 1;
-                    else if (v <= c.stop) c.active = 0;
+                    else if (u <= c.stop) c.active = 0;
                     else {
-                        if (kMixed) c.ru_below = fmax(c.stop, a.delta2 * v);
-                        if constexpr (!PRE) c.rr = Num<R>(v);
+                        if constexpr (kMixed) {
+                            const double before = c.scale.s2;
+                            c.scale.follow(v, n);
+                            if (c.scale.change != 1.f) {
+                                u = v * c.scale.s2;
+                                c.stop = c.stop / before * c.scale.s2;
+                            }
+                            c.ru_below = fmax(c.stop, a.delta2 * u);
+                        }
+                        if constexpr (!PRE) c.rr = Num<R>(u);
                         if (c.met) {
                             c.hold = c.it + c.wait;
                             c.wait = 8;
@@ -809,6 +879,8 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 }))
                 return false;
             if (c.nonfinite || !c.active || c.last) break;
+            // (PCG: z and c.rr keep the old units for the beta of the tau pass, a ratio)
+            if (!rescale()) return false;
         }
         if constexpr (PRE) {
             if (!sync_sum<CLU>(tm, c, red, tau(), [&](const Sum2<R>& v) {
