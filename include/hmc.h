@@ -293,11 +293,12 @@ int hmc_fma_peak(int prec, double* flop_per_s);
  * work, usable without a GPU. Errors: HMC_ERR_ARG. */
 int hmc_strip_plan(int L, int Nt, int nrhs, int slots, int* nch, int* order, int* nblk);
 
-/* Index checks of a library built with -DHMC_BOUNDS: the operator, force and strip kernels check
- * their global and shared-memory indices, record a failed check in a device error word and skip
- * the access (no trap). *word receives the OR of the codes recorded since the last call (1: D
- * operator, 2: force, 4: strip kernel global access, 8: strip kernel shared access) and clears
- * them; *enabled (may be NULL) is 1 in the bounds build. In the normal build *word is 0 and the
+/* Index checks of a library built with -DHMC_BOUNDS: the operator, force and strip kernels, the
+ * one-launch solver, the metric and the preconditioner check their global and shared-memory indices,
+ * record a failed check in a device error word and skip the access or make it at the first entry (no
+ * trap). *word receives the OR of the codes recorded since the last call (1: D operator, 2: force, 4:
+ * strip kernel global access, 8: strip kernel shared access, 16: one-launch solver, 32: metric, 64:
+ * preconditioner, 128: an FFT tile in shared memory) and clears them; *enabled (may be NULL) is 1 in the bounds build. In the normal build *word is 0 and the
  * checks compile to nothing. Synchronises the device. */
 int hmc_bounds_status(unsigned int* word, int* enabled);
 

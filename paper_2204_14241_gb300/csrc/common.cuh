@@ -194,7 +194,23 @@ static inline unsigned int bounds_take_tu() {
 #define HMC_IN(cond, code) true
 static inline unsigned int bounds_take_tu() { return 0; }
 #endif
-enum { kBndApplyD = 1, kBndForce = 2, kBndStripGlobal = 4, kBndStripShared = 8 };
+enum { kBndApplyD = 1, kBndForce = 2, kBndStripGlobal = 4, kBndStripShared = 8, kBndTeam = 16, kBndMetric = 32,
+       kBndPrecond = 64, kBndTile = 128 };
+// p, an entry of the n at base; bounds build: the first of them in place of one outside
+template <typename T> __device__ __forceinline__ T* in_range(T* p, T* base, int64_t n, int code) {
+    return HMC_IN(p >= base && p < base + n, code) ? p : base;
+}
+// Entry i of a tile in the block's dynamic shared memory; bounds build: the first one in place of one outside of it
+template <typename C> __device__ __forceinline__ C& tile_at(C* tile, int i) {
+#ifdef HMC_BOUNDS
+    extern __shared__ __align__(16) unsigned char hmc_dynamic_smem[];
+    unsigned bytes;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+    const unsigned char* at = reinterpret_cast<const unsigned char*>(tile + i);
+    if (!HMC_IN(at >= hmc_dynamic_smem && at + sizeof(C) <= hmc_dynamic_smem + bytes, kBndTile)) return tile[0];
+#endif
+    return tile[i];
+}
 
 // ---- asynchronous global -> shared copies (cp.async) ------------------------------------------
 // 16-byte copies bypass L1 (.cg); both addresses 16-byte aligned. 4-byte copies go through L1.

@@ -30,14 +30,14 @@ __device__ __noinline__ void dft_pass(C* sm, const Lines ln, int nf, int fs, int
         C* base = sm + p * ln.plane + (l & 1) * ln.l1 + (l >> 1) * ln.ls + f * fs;
         C v[R];
 #pragma unroll
-        for (int m = 0; m < R; ++m) v[m] = base[m * ps];
+        for (int m = 0; m < R; ++m) v[m] = tile_at(base, m * ps);
         bfly<R, -1>(v);
         if (tw) {
 #pragma unroll
             for (int m = 1; m < R; ++m) v[m] = cmul(v[m], tw[f * m]);
         }
 #pragma unroll
-        for (int m = 0; m < R; ++m) base[m * ps] = v[m];
+        for (int m = 0; m < R; ++m) tile_at(base, m * ps) = v[m];
     }
 }
 template <typename C>

@@ -733,7 +733,7 @@ extern "C" int hmc_bounds_status(unsigned int* word, int* enabled) {
 #else
     if (enabled) *enabled = 0;
 #endif
-    *word = bounds_take_stencil() | bounds_take_strip();
+    *word = bounds_take_stencil() | bounds_take_strip() | bounds_take_team() | bounds_take_metric() | bounds_take_precond();
     return HMC_OK;
 }
 

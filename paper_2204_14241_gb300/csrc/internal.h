@@ -347,6 +347,9 @@ int green_run(hmc_ctx* ctx, int chain, const double* phi, const double2* v, int 
 // bounds build: per-translation-unit device error words (0 in the normal build)
 unsigned int bounds_take_stencil();
 unsigned int bounds_take_strip();
+unsigned int bounds_take_team();
+unsigned int bounds_take_metric();
+unsigned int bounds_take_precond();
 
 // batch.cu: all (chain, RHS) pairs of the context solve A X = b in one persistent launch (mixed
 // precision, no preconditioner). b, x: concatenated [chain][k][V][4] complex128.

@@ -38,6 +38,17 @@ struct MetricDesc {
     double scale;
 };
 
+// entries of the fields and of the spectrum by address, for the index checks of the bounds build
+__device__ __forceinline__ double ld_field(const MetricDesc& d, const double* base, const double* p) {
+    return __ldg(in_range(p, base, (int64_t)3 * d.Nt * d.L * d.L, kBndMetric));
+}
+__device__ __forceinline__ double& out_at(const MetricDesc& d, double* p) {
+    return *in_range(p, d.out, (int64_t)3 * d.Nt * d.L * d.L, kBndMetric);
+}
+__device__ __forceinline__ double2& spec_at(const MetricDesc& d, double2* p) {
+    return *in_range(p, d.spec, (int64_t)3 * d.Nt * d.L * d.Hx, kBndMetric);
+}
+
 struct PlaneTiles {
     double2 *rows, *half, *tw;   // [L / 2][L | 1], [L][Hx | 1], [L]
     int* pos;                    // position of a frequency along x
@@ -70,23 +81,23 @@ __global__ void __launch_bounds__(256, 2) k_metric_fwd(const MetricDesc* __restr
     // rows 2j and 2j + 1 as the real and imaginary part of one line
     for (int e = threadIdx.x; e < (L / 2) * L; e += blockDim.x) {
         const int j = fdiv(e, d.dL), x = e - j * L;
-        p.rows[j * RA + x] = make_double2(__ldg(in + 2 * j * L + x), __ldg(in + (2 * j + 1) * L + x));
+        tile_at(p.rows, j * RA + x) = make_double2(ld_field(d, d.in, in + 2 * j * L + x), ld_field(d, d.in, in + (2 * j + 1) * L + x));
     }
     __syncthreads();
     dft_forward(p.rows, Lines{1, 0, L / 2, d.dHalf, RA, 2 * RA}, d.x1, d.x2, 1, p.tw);
     // twice each row's half spectrum: Z(k) + conj Z(-k) and (Z(k) - conj Z(-k)) / i
     for (int e = threadIdx.x; e < (L / 2) * Hx; e += blockDim.x) {
         const int j = fdiv(e, d.dHx), k = e - j * Hx;
-        const double2 z = p.rows[j * RA + p.pos[k]], w = p.rows[j * RA + p.pos[k ? L - k : 0]];
-        p.half[2 * j * RB + k] = make_double2(z.x + w.x, z.y - w.y);
-        p.half[(2 * j + 1) * RB + k] = make_double2(z.y + w.y, w.x - z.x);
+        const double2 z = tile_at(p.rows, j * RA + p.pos[k]), w = tile_at(p.rows, j * RA + p.pos[k ? L - k : 0]);
+        tile_at(p.half, 2 * j * RB + k) = make_double2(z.x + w.x, z.y - w.y);
+        tile_at(p.half, (2 * j + 1) * RB + k) = make_double2(z.y + w.y, w.x - z.x);
     }
     __syncthreads();
     dft_forward(p.half, Lines{1, 0, Hx, d.dHx, 1, 2}, d.x1, d.x2, RB, p.tw);
     double2* out = d.spec + (int64_t)blockIdx.x * L * Hx;
     for (int e = threadIdx.x; e < L * Hx; e += blockDim.x) {
         const int y = fdiv(e, d.dHx), k = e - y * Hx;
-        out[e] = p.half[y * RB + k];
+        spec_at(d, out + e) = tile_at(p.half, y * RB + k);
     }
 }
 
@@ -107,7 +118,7 @@ __global__ void __launch_bounds__(256, 2) k_metric_tau(const MetricDesc* __restr
     for (int i = threadIdx.x; i < Nt; i += blockDim.x) tw[i] = __ldg(d.twt + i);
     for (int e = threadIdx.x; e < Nt * W; e += blockDim.x) {
         const int t = fdiv(e, d.dW), l = e - t * W;
-        tile[e] = l < live ? spec[(int64_t)t * cols + l] : make_double2(0.0, 0.0);
+        tile_at(tile, e) = l < live ? spec_at(d, spec + (int64_t)t * cols + l) : make_double2(0.0, 0.0);
     }
     __syncthreads();
     const Lines ln{1, 0, W, d.dW, 1, 2};
@@ -122,14 +133,14 @@ __global__ void __launch_bounds__(256, 2) k_metric_tau(const MetricDesc* __restr
         const int my = dft_freq(py, d.x1, d.x2), mym = my ? L - my : 0, kxm = kx ? L - kx : 0;
         const bool mirrored = kx != 0 && kx != L / 2;   // -k lies outside the half spectrum
         const int64_t at = base + n * LL + my * L + kx, atm = base + nm * LL + mym * L + kxm;
-        const double2 v = tile[e];
+        const double2 v = tile_at(tile, e);
         if (op == HMC_METRIC_ACCUM) {
             const double q = (v.x * v.x + v.y * v.y) * d.scale;
-            d.out[at] += q;
-            if (mirrored) d.out[atm] += q;
+            out_at(d, d.out + at) += q;
+            if (mirrored) out_at(d, d.out + atm) += q;
             continue;
         }
-        const double s0 = __ldg(d.sig + at), s1 = __ldg(d.sig + atm);
+        const double s0 = ld_field(d, d.sig, d.sig + at), s1 = ld_field(d, d.sig, d.sig + atm);
         double w;
         if (op == HMC_METRIC_VELOCITY || op == HMC_METRIC_KINETIC) w = s0 + s1;
         else if (op == HMC_METRIC_MOMENTUM) {
@@ -143,7 +154,7 @@ __global__ void __launch_bounds__(256, 2) k_metric_tau(const MetricDesc* __restr
             const double q = w * (v.x * v.x + v.y * v.y);
             acc += mirrored ? q : 0.5 * q;
         } else {
-            tile[e] = make_double2(w * v.y, w * v.x);   // re and im exchanged: inverse steps follow
+            tile_at(tile, e) = make_double2(w * v.y, w * v.x);   // re and im exchanged: inverse steps follow
         }
     }
     if (op == HMC_METRIC_ACCUM) return;
@@ -156,7 +167,7 @@ __global__ void __launch_bounds__(256, 2) k_metric_tau(const MetricDesc* __restr
     dft_inverse(tile, ln, d.t1, d.t2, W, tw);
     for (int e = threadIdx.x; e < Nt * W; e += blockDim.x) {
         const int t = fdiv(e, d.dW), l = e - t * W;
-        if (l < live) spec[(int64_t)t * cols + l] = swapc(tile[e]);
+        if (l < live) spec_at(d, spec + (int64_t)t * cols + l) = swapc(tile_at(tile, e));
     }
 }
 
@@ -178,17 +189,18 @@ __global__ void __launch_bounds__(256, 2) k_metric_x_fwd(const __grid_constant__
     const double* in = d.in + (int64_t)c0 * 2 * L;
     for (int e = threadIdx.x; e < W * L; e += blockDim.x) {
         const int j = fdiv(e, d.dL), x = e - j * L;
-        rows[j * RA + x] = j < live ? make_double2(__ldg(in + 2 * j * L + x), __ldg(in + (2 * j + 1) * L + x))
-                                    : make_double2(0.0, 0.0);
+        tile_at(rows, j * RA + x) =
+            j < live ? make_double2(ld_field(d, d.in, in + 2 * j * L + x), ld_field(d, d.in, in + (2 * j + 1) * L + x))
+                     : make_double2(0.0, 0.0);
     }
     __syncthreads();
     dft_forward(rows, Lines{1, 0, W, dW, RA, 2 * RA}, d.x1, d.x2, 1, tw);
     double2* out = d.spec + (int64_t)c0 * 2 * Hx;
     for (int e = threadIdx.x; e < live * Hx; e += blockDim.x) {
         const int j = fdiv(e, d.dHx), k = e - j * Hx;
-        const double2 z = rows[j * RA + pos[k]], w = rows[j * RA + pos[k ? L - k : 0]];
-        out[2 * j * Hx + k] = make_double2(z.x + w.x, z.y - w.y);
-        out[(2 * j + 1) * Hx + k] = make_double2(z.y + w.y, w.x - z.x);
+        const double2 z = tile_at(rows, j * RA + pos[k]), w = tile_at(rows, j * RA + pos[k ? L - k : 0]);
+        spec_at(d, out + 2 * j * Hx + k) = make_double2(z.x + w.x, z.y - w.y);
+        spec_at(d, out + (2 * j + 1) * Hx + k) = make_double2(z.y + w.y, w.x - z.x);
     }
 }
 template <bool INV>
@@ -200,28 +212,28 @@ __global__ void __launch_bounds__(256, 2) k_metric_y(const __grid_constant__ Met
     auto at = [&](int e, int* y) -> double2* {   // spectrum entry of tile entry e, null past the last column
         *y = fdiv(e, dW);
         const int c = c0 + e - *y * W, plane = fdiv(c, d.dHx);
-        return c < total ? d.spec + ((int64_t)plane * L + *y) * Hx + (c - plane * Hx) : nullptr;
+        return c < total ? &spec_at(d, d.spec + ((int64_t)plane * L + *y) * Hx + (c - plane * Hx)) : nullptr;
     };
     int y;
     for (int e = threadIdx.x; e < L * W; e += blockDim.x) {
         const double2* q = at(e, &y);
         const double2 v = q ? *q : make_double2(0.0, 0.0);
-        tile[e] = INV ? swapc(v) : v;
+        tile_at(tile, e) = INV ? swapc(v) : v;
     }
     __syncthreads();
     const Lines ln{1, 0, W, dW, 1, 2};
     if (INV) dft_inverse(tile, ln, d.x1, d.x2, W, tw);
     else dft_forward(tile, ln, d.x1, d.x2, W, tw);
     for (int e = threadIdx.x; e < L * W; e += blockDim.x)
-        if (double2* q = at(e, &y)) *q = INV ? swapc(tile[e]) : tile[e];
+        if (double2* q = at(e, &y)) *q = INV ? swapc(tile_at(tile, e)) : tile_at(tile, e);
 }
 // rows u and v as the line u + i v from their half spectra (and the conjugates at -k), re and im exchanged
 __device__ __forceinline__ void pack_pair(double2* row, const int* pos, int L, int k, double2 u, double2 v) {
     if (k == 0 || k == L / 2) {
-        row[pos[k]] = make_double2(v.x, u.x);   // real columns
+        tile_at(row, pos[k]) = make_double2(v.x, u.x);   // real columns
     } else {
-        row[pos[k]] = make_double2(u.y + v.x, u.x - v.y);
-        row[pos[L - k]] = make_double2(v.x - u.y, u.x + v.y);
+        tile_at(row, pos[k]) = make_double2(u.y + v.x, u.x - v.y);
+        tile_at(row, pos[L - k]) = make_double2(v.x - u.y, u.x + v.y);
     }
 }
 __device__ __forceinline__ void put_rows(const MetricDesc& d, const double2* rows, int pairs, int64_t first, double eps, bool add) {
@@ -230,8 +242,8 @@ __device__ __forceinline__ void put_rows(const MetricDesc& d, const double2* row
     const double s = add ? eps * d.scale : d.scale;
     for (int e = threadIdx.x; e < pairs * L; e += blockDim.x) {
         const int j = fdiv(e, d.dL), x = e - j * L;
-        const double2 z = rows[j * RA + x];
-        double *o0 = out + 2 * j * L + x, *o1 = o0 + L;
+        const double2 z = tile_at(rows, j * RA + x);
+        double *o0 = &out_at(d, out + 2 * j * L + x), *o1 = &out_at(d, out + (2 * j + 1) * L + x);
         if (add) {
             *o0 = fma(s, z.y, *o0);
             *o1 = fma(s, z.x, *o1);
@@ -248,12 +260,12 @@ __global__ void __launch_bounds__(256, 2) k_metric_x_inv(const __grid_constant__
     double2 *rows = reinterpret_cast<double2*>(smem), *tw = rows + W * RA;
     int* pos = reinterpret_cast<int*>(tw + L);
     x_tables(d, tw, pos);
-    for (int e = live * RA + threadIdx.x; e < W * RA; e += blockDim.x) rows[e] = make_double2(0.0, 0.0);
+    for (int e = live * RA + threadIdx.x; e < W * RA; e += blockDim.x) tile_at(rows, e) = make_double2(0.0, 0.0);
     __syncthreads();
-    const double2* in = d.spec + (int64_t)c0 * 2 * Hx;
+    double2* in = d.spec + (int64_t)c0 * 2 * Hx;
     for (int e = threadIdx.x; e < live * Hx; e += blockDim.x) {
         const int j = fdiv(e, d.dHx), k = e - j * Hx;
-        pack_pair(rows + j * RA, pos, L, k, in[2 * j * Hx + k], in[(2 * j + 1) * Hx + k]);
+        pack_pair(rows + j * RA, pos, L, k, spec_at(d, in + 2 * j * Hx + k), spec_at(d, in + (2 * j + 1) * Hx + k));
     }
     __syncthreads();
     dft_inverse(rows, Lines{1, 0, W, dW, RA, 2 * RA}, d.x1, d.x2, 1, tw);
@@ -268,21 +280,23 @@ __global__ void __launch_bounds__(256, 2) k_metric_inv(const MetricDesc* __restr
     const int L = d.L, Hx = d.Hx, RA = L | 1, RB = Hx | 1;
     if ((int)blockIdx.x >= 3 * d.Nt) return;
     const PlaneTiles p = plane_tiles(d, smem);
-    const double2* in = d.spec + (int64_t)blockIdx.x * L * Hx;
+    double2* in = d.spec + (int64_t)blockIdx.x * L * Hx;
     for (int e = threadIdx.x; e < L * Hx; e += blockDim.x) {
         const int y = fdiv(e, d.dHx), k = e - y * Hx;
-        p.half[y * RB + k] = swapc(in[e]);
+        tile_at(p.half, y * RB + k) = swapc(spec_at(d, in + e));
     }
     __syncthreads();
     dft_inverse(p.half, Lines{1, 0, Hx, d.dHx, 1, 2}, d.x1, d.x2, RB, p.tw);
     for (int e = threadIdx.x; e < (L / 2) * Hx; e += blockDim.x) {
         const int j = fdiv(e, d.dHx), k = e - j * Hx;
-        pack_pair(p.rows + j * RA, p.pos, L, k, swapc(p.half[2 * j * RB + k]), swapc(p.half[(2 * j + 1) * RB + k]));
+        pack_pair(p.rows + j * RA, p.pos, L, k, swapc(tile_at(p.half, 2 * j * RB + k)), swapc(tile_at(p.half, (2 * j + 1) * RB + k)));
     }
     __syncthreads();
     dft_inverse(p.rows, Lines{1, 0, L / 2, d.dHalf, RA, 2 * RA}, d.x1, d.x2, 1, p.tw);
     put_rows(d, p.rows, L / 2, (int64_t)blockIdx.x * (L / 2), eps, add);
 }
+
+unsigned int bounds_take_metric() { return bounds_take_tu(); }
 
 // ---- host --------------------------------------------------------------------------------------------
 // Lines of a tile, of `total` lines of n1 n2 points: the width whose waves of two blocks an SM cost the FP64 pipe

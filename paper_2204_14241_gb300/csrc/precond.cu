@@ -39,6 +39,12 @@ template <typename R> struct PreArgs {
     FastDiv dL, dLL, dCL, dW, dCW;   // by L, L^2, components x L, W, components x W
 };
 
+// entries of the source and the destination by address (nrhs right-hand sides of 4 V entries), for the index checks of
+// the bounds build
+template <typename T, typename R> __device__ __forceinline__ T* entry(T* p, T* base, const PreArgs<R>& a) {
+    return in_range(p, base, (int64_t)a.planes * a.LL * (sizeof(R) == 4 ? 2 : 1), kBndPrecond);
+}
+
 template <typename R> constexpr int kComp = sizeof(R) == 4 ? 2 : 1;   // components of a group
 
 // FWD: planes of the site layout to the spectrum, else back, times scale. Plane q = (k Nt + t) groups + group.
@@ -60,13 +66,13 @@ __global__ void __launch_bounds__(256, 2) k_pre_xy(const __grid_constant__ PreAr
         }
     };
     each([&](int64_t site, int64_t spec, int at) {
-        const C* v = a.src + (FWD ? site : spec);
+        const C* v = entry(a.src + (FWD ? site : spec), a.src, a);
         if constexpr (NC == 2) {
             const float4 u = *reinterpret_cast<const float4*>(v);
-            tile[at] = FWD ? mk<C>(u.x, u.y) : mk<C>(u.y, u.x);
-            tile[at + 1] = FWD ? mk<C>(u.z, u.w) : mk<C>(u.w, u.z);
+            tile_at(tile, at) = FWD ? mk<C>(u.x, u.y) : mk<C>(u.y, u.x);
+            tile_at(tile, at + 1) = FWD ? mk<C>(u.z, u.w) : mk<C>(u.w, u.z);
         } else {
-            tile[at] = FWD && !a.swap ? *v : swapc(*v);
+            tile_at(tile, at) = FWD && !a.swap ? *v : swapc(*v);
         }
     });
     __syncthreads();
@@ -80,13 +86,13 @@ __global__ void __launch_bounds__(256, 2) k_pre_xy(const __grid_constant__ PreAr
         dft_inverse(tile, rows, a.x1, a.x2, NC, tw);
     }
     each([&](int64_t site, int64_t spec, int at) {
-        C* v = a.dst + (FWD ? spec : site);
+        C* v = entry(a.dst + (FWD ? spec : site), a.dst, a);
         const R s = a.scale;
         if constexpr (NC == 2) {
-            const C u = tile[at], w = tile[at + 1];
+            const C u = tile_at(tile, at), w = tile_at(tile, at + 1);
             *reinterpret_cast<float4*>(v) = FWD ? make_float4(u.x, u.y, w.x, w.y) : make_float4(s * u.y, s * u.x, s * w.y, s * w.x);
         } else {
-            *v = FWD ? tile[at] : mk<C>(s * tile[at].y, s * tile[at].x);
+            *v = FWD ? tile_at(tile, at) : mk<C>(s * tile_at(tile, at).y, s * tile_at(tile, at).x);
         }
     });
 }
@@ -134,11 +140,11 @@ __global__ void __launch_bounds__(256, 2) k_pre_tau(const __grid_constant__ PreA
         const C f = twist[t];
         if constexpr (NC == 2) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (l < live) v = *reinterpret_cast<const float4*>(z + t * step + 2 * l);
-            tile[2 * e] = cmulconj(f, mk<C>(v.x, v.y));
-            tile[2 * e + 1] = cmulconj(f, mk<C>(v.z, v.w));
+            if (l < live) v = *reinterpret_cast<const float4*>(entry(z + t * step + 2 * l, a.dst, a));
+            tile_at(tile, 2 * e) = cmulconj(f, mk<C>(v.x, v.y));
+            tile_at(tile, 2 * e + 1) = cmulconj(f, mk<C>(v.z, v.w));
         } else {
-            tile[e] = l < live ? cmulconj(f, z[t * step + l]) : mk<C>(0, 0);
+            tile_at(tile, e) = l < live ? cmulconj(f, *entry(z + t * step + l, a.dst, a)) : mk<C>(0, 0);
         }
     }
     __syncthreads();
@@ -159,8 +165,8 @@ __global__ void __launch_bounds__(256, 2) k_pre_tau(const __grid_constant__ PreA
         const R ph = (R)1 / (re * re + im * im);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            const C v = tile[NC * e + c];
-            tile[NC * e + c] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
+            const C v = tile_at(tile, NC * e + c);
+            tile_at(tile, NC * e + c) = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
         }
     }
     __syncthreads();
@@ -170,10 +176,10 @@ __global__ void __launch_bounds__(256, 2) k_pre_tau(const __grid_constant__ PreA
         if (l >= live) continue;
         const C f = twist[t];
         if constexpr (NC == 2) {
-            const C u = cmul(swapc(tile[2 * e]), f), v = cmul(swapc(tile[2 * e + 1]), f);
-            *reinterpret_cast<float4*>(z + t * step + 2 * l) = make_float4(u.x, u.y, v.x, v.y);
+            const C u = cmul(swapc(tile_at(tile, 2 * e)), f), v = cmul(swapc(tile_at(tile, 2 * e + 1)), f);
+            *reinterpret_cast<float4*>(entry(z + t * step + 2 * l, a.dst, a)) = make_float4(u.x, u.y, v.x, v.y);
         } else {
-            z[t * step + l] = cmul(swapc(tile[e]), f);
+            *entry(z + t * step + l, a.dst, a) = cmul(swapc(tile_at(tile, e)), f);
         }
     }
 }
@@ -194,8 +200,8 @@ __global__ void __launch_bounds__(256, 2) k_twisted_tau(const __grid_constant__ 
     const double2* z = a.src + (int64_t)k * Nt * 4 * LL + j0;
     for (int e = threadIdx.x; e < Nt * 4 * W; e += blockDim.x) {
         const int row = fdiv(e, a.dW), l = e - row * W;   // row = 4 t + component
-        const double2 v = l < live ? z[(int64_t)row * LL + l] : make_double2(0.0, 0.0);
-        tile[e] = inverse ? v : cmulconj(twist[row >> 2], v);
+        const double2 v = l < live ? *entry(z + (int64_t)row * LL + l, a.src, a) : make_double2(0.0, 0.0);
+        tile_at(tile, e) = inverse ? v : cmulconj(twist[row >> 2], v);
     }
     __syncthreads();
     dft_forward(tile, Lines{1, 0, 4 * W, a.dCW, 1, 2}, a.t1, a.t2, 4 * W, tw);
@@ -204,10 +210,12 @@ __global__ void __launch_bounds__(256, 2) k_twisted_tau(const __grid_constant__ 
         const int q = e >> 2, c = e & 3, p = fdiv(q, a.dW), l = q - p * W;
         if (l >= live) continue;
         const int j = j0 + l, y = fdiv(j, a.dL), x = j - y * L, n = dft_freq(p, a.t1, a.t2);
-        const double2 v = tile[(4 * p + c) * W + l], u = cscale(inverse ? cmul(swapc(v), twist[n]) : v, a.scale);
-        out[((int64_t)n * LL + dft_freq(y, a.x1, a.x2) * L + dft_freq(x, a.x1, a.x2)) * 4 + c] = u;
+        const double2 v = tile_at(tile, (4 * p + c) * W + l), u = cscale(inverse ? cmul(swapc(v), twist[n]) : v, a.scale);
+        *entry(out + ((int64_t)n * LL + dft_freq(y, a.x1, a.x2) * L + dft_freq(x, a.x1, a.x2)) * 4 + c, a.dst, a) = u;
     }
 }
+
+unsigned int bounds_take_precond() { return bounds_take_tu(); }
 
 // ---- host --------------------------------------------------------------------------------------------
 struct XyLaunch {

@@ -41,9 +41,11 @@
 namespace hmc {
 
 template <typename R> struct It { cplx<R> s[2]; };   // one band of one site: its two spin components
+// (n: items of the vector, for the index checks of the bounds build)
 
-template <typename R> __device__ __forceinline__ It<R> ld_it(const cplx<R>* v, int64_t i) {
-    It<R> o;
+template <typename R> __device__ __forceinline__ It<R> ld_it(const cplx<R>* v, int64_t i, int64_t n) {
+    It<R> o{};
+    if (!HMC_IN(i >= 0 && i < n, kBndTeam)) return o;
     if constexpr (sizeof(R) == 4) {
         const float4 a = *reinterpret_cast<const float4*>(v + 2 * i);
         o.s[0] = make_float2(a.x, a.y);
@@ -54,7 +56,8 @@ template <typename R> __device__ __forceinline__ It<R> ld_it(const cplx<R>* v, i
     }
     return o;
 }
-template <typename R> __device__ __forceinline__ void st_it(cplx<R>* v, int64_t i, const It<R>& o) {
+template <typename R> __device__ __forceinline__ void st_it(cplx<R>* v, int64_t i, int64_t n, const It<R>& o) {
+    if (!HMC_IN(i >= 0 && i < n, kBndTeam)) return;
     if constexpr (sizeof(R) == 4) {
         *reinterpret_cast<float4*>(v + 2 * i) = make_float4(o.s[0].x, o.s[0].y, o.s[1].x, o.s[1].y);
     } else {
@@ -150,8 +153,11 @@ __device__ __forceinline__ double2 d_spin(const BChainDev& g, const Coef<double>
         rem = s - t * LL;
     }
     const int y = fdiv(rem, g.dL), x = rem - y * L, other = BM ? (band ? i - LL : i + LL) : i ^ 1;
-    auto ld = [&](int j) { return v[2 * j + q]; };
-    const double2 c = ld(i), ws = ld(other), wo = v[2 * other + 1 - q];
+    auto at = [&](int j, int spin) {
+        return HMC_IN(j >= 0 && j < 2 * (int)g.V, kBndTeam) ? v[2 * j + spin] : make_double2(0.0, 0.0);
+    };
+    auto ld = [&](int j) { return at(j, q); };
+    const double2 c = ld(i), ws = ld(other), wo = at(other, 1 - q);
     const double2 xm = ld(x ? i - u : i + u * (L - 1)), xp = ld(x + 1 < L ? i + u : i - u * (L - 1));
     const double2 ym = ld(y ? i - u * L : i + u * (LL - L)), yp = ld(y + 1 < L ? i + u * L : i - u * (LL - L));
     const int edge = DAG ? (t == 0) : (t + 1 == g.Nt);
@@ -491,9 +497,9 @@ __device__ __forceinline__ void plane_forward(const TeamPre<R>& q, const PreTab<
     for (int e = threadIdx.x; e < np * g.LL; e += blockDim.x) {
         const int pl = fdiv(e, g.dLL), j = e - pl * g.LL, y = fdiv(j, g.dL), at = pl * q.plane + (y * RS + j - y * L) * 2;
         It<R> v;
-        v.s[0] = p.tile[at];
-        v.s[1] = p.tile[at + 1];
-        st_it<R>(z, (t0 + pl * T) * g.LL + j, v);
+        v.s[0] = tile_at(p.tile, at);
+        v.s[1] = tile_at(p.tile, at + 1);
+        st_it<R>(z, (t0 + pl * T) * g.LL + j, 2 * g.V, v);
     }
     __syncthreads();
 }
@@ -526,33 +532,33 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     }
     auto sync = [&]() { return sync_sum<CLU>(tm, c, red, NoSum(), [](const NoSum&) {}); };
     auto in = [&](int i) { return PRE ? to_bm(g, i) : i; };   // from the public layout to the solver's
-    auto ld64 = [](const double2* v) { return [v](int j) { return ld_it<double>(v, j); }; };
-    auto ldr = [](const C* v) { return [v](int j) { return ld_it<R>(v, j); }; };
+    auto ld64 = [n](const double2* v) { return [v, n](int j) { return ld_it<double>(v, j, n); }; };
+    auto ldr = [n](const C* v) { return [v, n](int j) { return ld_it<R>(v, j, n); }; };
 
     // ---- start: r = b - A x (or b), zero directions, norms ----------------------------------------
     if (a.use_x0) {
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, n, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
         if (!sync()) return false;
     }
     {
         Sum2<double> sb, sr;
         for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            const It<double> bb = ld_it<double>(b, i);
+            const It<double> bb = ld_it<double>(b, i, n);
             It<double> rr = bb;
             if (a.use_x0) {
                 rr = axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), bb);
             } else {
-                st_it<double>(x64, i, It<double>{});
-                st_it<double>(t64, i, It<double>{});   // D^dagger x of the zero start
+                st_it<double>(x64, i, n, It<double>{});
+                st_it<double>(t64, i, n, It<double>{});   // D^dagger x of the zero start
             }
             It<R> rl;
 #pragma unroll
             for (int s = 0; s < 2; ++s) rl.s[s] = mk<C>((R)rr.s[s].x, (R)rr.s[s].y);
             const int o = in(i);
-            st_it<R>(r, o, rl);
-            if constexpr (kMixed) st_it<R>(x, o, It<R>{});
+            st_it<R>(r, o, n, rl);
+            if constexpr (kMixed) st_it<R>(x, o, n, It<R>{});
             // the first direction is r (or z): the on-the-fly and the inverse-FFT forms add 0 * p
-            st_it<R>(pold, o, !kMixed && !PRE ? rl : It<R>{});
+            st_it<R>(pold, o, n, !kMixed && !PRE ? rl : It<R>{});
             sq_it(sb, bb);
             sq_it(sr, rr);
         }
@@ -586,8 +592,8 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                     const int o = in(i);
                     const It<R> zero{};
-                    st_it<R>(r, o, axpy_it<R>(f, ld_it<R>(r, o), zero));
-                    st_it<R>(pold, o, axpy_it<R>(f, ld_it<R>(pold, o), zero));
+                    st_it<R>(r, o, n, axpy_it<R>(f, ld_it<R>(r, o, n), zero));
+                    st_it<R>(pold, o, n, axpy_it<R>(f, ld_it<R>(pold, o, n), zero));
                 }
                 return sync();
             }
@@ -613,9 +619,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
     auto forward = [&]() {
         each_round([&](int t0, int np) {
             each_site(t0, np, [&](int i, int at) {
-                const It<R> v = ld_it<R>(r, i);
-                pt.tile[at] = v.s[0];
-                pt.tile[at + 1] = v.s[1];
+                const It<R> v = ld_it<R>(r, i, n);
+                tile_at(pt.tile, at) = v.s[0];
+                tile_at(pt.tile, at + 1) = v.s[1];
             });
             plane_forward<R>(a.pre, pt, g, t0, tm.T, np, z);
         });
@@ -634,14 +640,15 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 base_s[p] = q.c0[band] + q.chx[band] * pt.cosk[xx] + q.chy[band] * pt.cosk[y];
             }
             C* zp = z + ((int64_t)band * g.LL + j0) * 2;
+            const int left = n - (band * g.LL + j0);   // items from zp on
             const int step = 2 * g.LL, live = min(q.W, g.LL - j0), ne = g.Nt * q.W;   // items
             for (int e = threadIdx.x; e < ne; e += blockDim.x) {
                 const int ts = fdiv(e, q.dW), l = e - ts * q.W;
                 const C w = pt.twist[ts];
                 It<R> v{};
-                if (l < live) v = ld_it<R>(zp, (int64_t)ts * step + l);
-                pt.tile[2 * e] = cmulconj(w, v.s[0]);
-                pt.tile[2 * e + 1] = cmulconj(w, v.s[1]);
+                if (l < live) v = ld_it<R>(zp, (int64_t)ts * step + l, left);
+                tile_at(pt.tile, 2 * e) = cmulconj(w, v.s[0]);
+                tile_at(pt.tile, 2 * e + 1) = cmulconj(w, v.s[1]);
             }
             __syncthreads();
             dft_forward(pt.tile, ln, q.t1, q.t2, w2, pt.twt);
@@ -652,10 +659,10 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 const R ph = (R)1 / (re * re + w.y * w.y);
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
-                    const C v = pt.tile[2 * e + s];
+                    const C v = tile_at(pt.tile, 2 * e + s);
                     acc.add(ph, v.x);
                     acc.add(ph, v.y);
-                    pt.tile[2 * e + s] = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
+                    tile_at(pt.tile, 2 * e + s) = mk<C>(ph * v.y, ph * v.x);   // re and im exchanged: inverse steps follow
                 }
             }
             __syncthreads();
@@ -664,9 +671,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 const int ts = fdiv(e, q.dW), l = e - ts * q.W;
                 const C w = pt.twist[ts];
                 It<R> v;
-                v.s[0] = cmul(swapc(pt.tile[2 * e]), w);
-                v.s[1] = cmul(swapc(pt.tile[2 * e + 1]), w);
-                if (l < live) st_it<R>(zp, (int64_t)ts * step + l, v);
+                v.s[0] = cmul(swapc(tile_at(pt.tile, 2 * e)), w);
+                v.s[1] = cmul(swapc(tile_at(pt.tile, 2 * e + 1)), w);
+                if (l < live) st_it<R>(zp, (int64_t)ts * step + l, left, v);
             }
             __syncthreads();
         }
@@ -680,9 +687,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         each_round([&](int t0, int np) {
             const Lines rows{np, q.plane, 2 * L, q.d2L, 1, 2 * RS}, cols{np, q.plane, 2 * L, q.d2L, 1, 2};
             each_site(t0, np, [&](int i, int at) {
-                const It<R> v = ld_it<R>(z, i);
-                pt.tile[at] = swapc(v.s[0]);
-                pt.tile[at + 1] = swapc(v.s[1]);
+                const It<R> v = ld_it<R>(z, i, n);
+                tile_at(pt.tile, at) = swapc(v.s[0]);
+                tile_at(pt.tile, at + 1) = swapc(v.s[1]);
             });
             __syncthreads();
             dft_inverse(pt.tile, cols, q.x1, q.x2, 2 * RS, pt.twx);
@@ -691,10 +698,10 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 It<R> v;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
-                    const C d = pt.tile[at + s];
+                    const C d = tile_at(pt.tile, at + s);
                     v.s[s] = mk<C>(sc * d.y, sc * d.x);
                 }
-                st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), v));
+                st_it<R>(pold, i, n, axpy_it<R>(be, ld_it<R>(pold, i, n), v));
             });
             __syncthreads();
         });
@@ -722,9 +729,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 It<R> pc;
                 const It<R> o = d_item<R, true, PRE>(
-                    g, a.cf, phi, i, [&](int j) { return axpy_it<R>(be, ld_it<R>(pold, j), ld_it<R>(r, j)); }, &pc);
-                st_it<R>(pnew, i, pc);
-                st_it<R>(t, i, o);
+                    g, a.cf, phi, i, [&](int j) { return axpy_it<R>(be, ld_it<R>(pold, j, n), ld_it<R>(r, j, n)); }, &pc);
+                st_it<R>(pnew, i, n, pc);
+                st_it<R>(t, i, n, o);
                 sq_it(acc, o);
             }
         } else if (!kMixed && per <= kSpinItems) {
@@ -739,7 +746,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         } else {
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 const It<R> o = d_item<R, true, PRE>(g, a.cf, phi, i, ldr(pold));
-                st_it<R>(t, i, o);
+                st_it<R>(t, i, n, o);
                 sq_it(acc, o);
             }
         }
@@ -755,9 +762,9 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
         auto update = [&](int i) {
             const It<R> q = d_item<R, false, PRE>(g, a.cf, phi, i, ldr(t));
             const int o = PRE && !kMixed ? from_bm(g, i) : i;   // FP64 iterates in the caller's x
-            st_it<R>(x, o, axpy_it<R>(al, ld_it<R>(pnew, i), ld_it<R>(x, o)));
-            const It<R> rn = axpy_it<R>(-al, q, ld_it<R>(r, i));
-            st_it<R>(r, i, rn);
+            st_it<R>(x, o, n, axpy_it<R>(al, ld_it<R>(pnew, i, n), ld_it<R>(x, o, n)));
+            const It<R> rn = axpy_it<R>(-al, q, ld_it<R>(r, i, n));
+            st_it<R>(r, i, n, rn);
             sq_it(acc, rn);
             return rn;
         };
@@ -782,13 +789,13 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                     const int RS = row_stride(g.L);
                     for (int e = threadIdx.x; e < 2 * np * g.LL; e += blockDim.x) {
                         const int pl = fdiv(e >> 1, g.dLL), j = (e >> 1) - pl * g.LL, y = fdiv(j, g.dL), xx = j - y * g.L;
-                        pt.tile[pl * a.pre.plane + (y * RS + xx) * 2 + (e & 1)] = update_spin((t0 + pl * tm.T) * g.LL + j, e & 1);
+                        tile_at(pt.tile, pl * a.pre.plane + (y * RS + xx) * 2 + (e & 1)) = update_spin((t0 + pl * tm.T) * g.LL + j, e & 1);
                     }
                 } else {
                     each_site(t0, np, [&](int i, int at) {
                         const It<R> v = update(i);
-                        pt.tile[at] = v.s[0];
-                        pt.tile[at + 1] = v.s[1];
+                        tile_at(pt.tile, at) = v.s[0];
+                        tile_at(pt.tile, at + 1) = v.s[1];
                     });
                 }
                 plane_forward<R>(a.pre, pt, g, t0, tm.T, np, z);
@@ -822,34 +829,34 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
             // ---- reliable update: x64 += x, r = b - A x64 in FP64 ----
             if constexpr (kMixed) {
                 for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-                    const It<R> lo = ld_it<R>(x, in(i));
-                    It<double> hi = ld_it<double>(x64, i);
+                    const It<R> lo = ld_it<R>(x, in(i), n);
+                    It<double> hi = ld_it<double>(x64, i, n);
                     const double inv = c.scale.inv;
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
                         hi.s[s].x = fma(inv, (double)lo.s[s].x, hi.s[s].x);
                         hi.s[s].y = fma(inv, (double)lo.s[s].y, hi.s[s].y);
                     }
-                    st_it<double>(x64, i, hi);
-                    st_it<R>(x, in(i), It<R>{});
+                    st_it<double>(x64, i, n, hi);
+                    st_it<R>(x, in(i), n, It<R>{});
                 }
                 if (!sync()) return false;
             }
-            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
+            for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) st_it<double>(t64, i, n, d_item<double, true, false>(g, a.cf64, g.phi64, i, ld64(x64)));
             if (!sync()) return false;
             Sum2<double> acc64;
             R unit = 1;
             if constexpr (kMixed) unit = c.scale.s;
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 const It<double> rd =
-                    axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i));
+                    axpy_it<double>(-1.0, d_item<double, false, false>(g, a.cf64, g.phi64, i, ld64(t64)), ld_it<double>(b, i, n));
                 It<R> rl;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
                     rl.s[s] = mk<C>((R)rd.s[s].x, (R)rd.s[s].y);
                     if (kMixed) rl.s[s] = mk<C>(unit * rl.s[s].x, unit * rl.s[s].y);
                 }
-                st_it<R>(r, in(i), rl);
+                st_it<R>(r, in(i), n, rl);
                 sq_it(acc64, rd);
             }
             if (!sync_sum<CLU>(tm, c, red, acc64, [&](const Sum2<double>& sum) {
@@ -912,7 +919,7 @@ __device__ __forceinline__ bool team_run(const TeamArgs<R>& a, Team& tm, Ctl<R>&
                 }
             } else {
                 for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
-                    st_it<R>(pold, i, axpy_it<R>(be, ld_it<R>(pold, i), ld_it<R>(r, i)));
+                    st_it<R>(pold, i, n, axpy_it<R>(be, ld_it<R>(pold, i, n), ld_it<R>(r, i, n)));
             }
             if (!sync()) return false;
         }
@@ -981,6 +988,8 @@ k_team(const __grid_constant__ TeamArgs<R> a) {
         } while (a.queue);
     }
 }
+
+unsigned int bounds_take_team() { return bounds_take_tu(); }
 
 // ---- host --------------------------------------------------------------------------------------------
 void team_geometry(BChainDev* d, const Lat& lat) {
