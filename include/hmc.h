@@ -85,16 +85,24 @@ typedef struct {
                            reduction order, hence every bit of the results, is reproducible);
                            1: on first use per (L, Nt, nrhs, precision) time the valid tile and
                            time-chunk shapes on the call's own buffers and keep the fastest */
-    int wait_spin_limit;   /* polls of a device-side wait before it gives up (0: 1 << 20); a wait
-                              that gives up makes the call return HMC_ERR_TIMEOUT */
+    int wait_spin_limit;   /* limit of device-side waits: polls of the strip operator's (0: 1 << 20),
+                              microseconds of a team's barrier in a batched solve (0: 2 s). A
+                              single-chain solve in one launch gives its barriers 2 s whatever this
+                              says; a small one runs as a thread-block cluster, whose hardware barrier
+                              knows no limit. A wait that gives up makes the call return
+                              HMC_ERR_TIMEOUT */
     int test_wait_timeout; /* nonzero (tests only): the first device-side wait of every fused-A
-                              launch (and the first grid barrier of a batched solve) targets a
-                              barrier that nothing completes, so it always gives up */
+                              launch and the first team barrier of every solve in one launch (which
+                              is then no cluster and waits wait_spin_limit microseconds, single-chain
+                              solves too) targets a barrier that nothing completes, so it always
+                              gives up */
     int batch_chains;   /* nonzero: trajectory() advances all chains together and every force
                            evaluation solves all (chain, RHS) pairs in one persistent cooperative
                            launch, a team of blocks per pair (mixed solver mode only; CG without the
-                           preconditioner; the teams' barriers, as those of single-chain solves in
-                           one launch, bounded by wait_spin_limit microseconds, default 2 s) */
+                           preconditioner; the teams' barriers bounded by wait_spin_limit
+                           microseconds, default 2 s). A pair's blocks, and with them the order of
+                           its sums, follow from the volumes of all chains: the same batch gives the
+                           same bits, a chain in another batch the same to the solver's tolerance */
     int batch_graph;    /* with batch_chains: the leapfrog part of a trajectory (every force
                            evaluation, kick and drift of all chains) runs as one CUDA graph,
                            captured on first use and replayed while n_leap, eps, the chains'
@@ -182,6 +190,9 @@ int apply_precond(hmc_ctx* ctx, int chain, int prec, const void* x, void* y, int
  * zero initial guess, for nrhs right-hand sides at once. phi: [3][V] double; b, x:
  * complex128. Stops when the FP64 true residual of every RHS is <= tol ||b||.
  * tol <= 0 or maxit <= 0 select the context defaults. st may be NULL.
+ * Most solves of up to about a million sites in all (FP64: 2^23) are one launch that may occupy every SM
+ * until it ends; kernels of other streams wait for it. Mixed mode wants the components of b within
+ * FP32's range.
  * Returns HMC_ERR_NOCONV if maxit was reached (x then holds the last iterate). */
 int cg_solve(hmc_ctx* ctx, int chain, const void* phi, const void* b, void* x, int nrhs,
              double tol, int maxit, int precond, hmc_cg_stats* st);

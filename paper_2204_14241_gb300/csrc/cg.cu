@@ -306,7 +306,7 @@ int launch_phi_to32(hmc_ctx* ctx, const double* a, float* b, int64_t n) {
 // passes through ctx->d_z64: t_ = D^dagger x, then r = b - D t_ with the complex64 copy and the
 // partial norms fused into the second pass (launch_residual_D). GB300's FP64 pipe bounds both
 // passes; a fused D D^dagger kernel would recompute t_ on a one-site ring around each tile (about
-// 2.4 site operations per output site against 2.0 here) and measured slower (3.33 ms against 2.55
+// 2.4 site operations per output site against 2.0 here) and measured slower (3.32 ms against 1.98
 // ms for A at 80x80x160 with 8 RHS). d_z64 is dead whenever this runs: the next direction restart
 // recomputes z. Right-hand sides already converged (cgs) are skipped.
 static int residual64(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2* x, const double2* b,

@@ -229,7 +229,9 @@ template <typename R> __device__ __forceinline__ void sq_it(Sum2<R>& a, const It
 }
 
 // Scalars of the recurrence: FP64, or an FP32 pair (48 bits) in complex64, where they end in an FP32 alpha or
-// beta: one thread works on them while the rest wait, and an FP64 operation takes 65 clocks, a division 570.
+// beta: one thread works on them while the rest wait, and an FP64 operation takes 65 clocks, a division 570. Of
+// 3200 quotients of random sums of 512 to 442368 squares, pairs and FP64 gave the same FP32 number in all (the sums'
+// own errors: 1e-14 and 3e-16 at most).
 template <typename R> struct Num;
 template <> struct Num<double> {
     double v;
@@ -1308,7 +1310,11 @@ static int solve(hmc_ctx* ctx, const Lat& lat, const double* phi, const double2*
 //  CG, complex128  2991 : 4300 at 80 x 80 x 160 with 8
 //  PCG, complex64  lattices with compiled FFT passes 81 : 119 at 64 x 64 x 128, 136 : 168 at 48 x 48 x 96 with 4, but
 //                  167 : 157 at 40 x 40 x 80 with 8; others (no compiled length) 115 : 448 at 36 x 36 x 70 with 8
-//  PCG, complex128 2148 : 2461 at 80 x 80 x 160
+//  PCG, complex128 2141 : 2445 at 80 x 80 x 160, 3636 : 4757, 6598 : 9227 and 12458 : 18307 there with 2, 4 and 8,
+//                  1016 : 1194 at 40 x 40 x 80 with 4, 1600 : 2122 at 20 x 20 x 40 with 64
+// On both sides of the complex64 limits: CG 68 : 77 at 48 x 48 x 96 with 5, 73 : 151 at 16 x 16 x 160 with 30, past it
+// 80 : 88 at 48 x 48 x 96 with 6; PCG 139 : 136 at 40 x 40 x 80 with 7, 125 : 165 at 20 x 20 x 40 with 50, past it
+// 188 : 177 at 64 x 64 x 128 with 2, 249 : 163 at 80 x 80 x 160.
 static bool worth_it(hmc_ctx* ctx, const Lat& lat, int nrhs, int precond) {
     const int64_t sites = (int64_t)nrhs * lat.V;
     if (sites > (int64_t)1 << 23) return false;   // the largest measured
